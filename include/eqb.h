@@ -204,7 +204,7 @@ eqb_status eqb_margin_hist_lei(const eqb_bf16 *z, const float *tau, int64_t T,
                                void *stream);
 
 /* Bytes of device workspace eqb_layer_step needs for E experts (the two
- * [E,256] histograms, two block counters, u, rho, q_hat and a 65,536-float
+ * [E,256] histograms, block counters, u, rho, q_hat and a 65,536-float
  * LEI coefficient table, each 256-byte aligned; 788,480 bytes for
  * E = 256). */
 size_t eqb_layer_workspace_bytes(int32_t E);

@@ -54,6 +54,9 @@ struct RouteArgs {
 // (per-expert state of the per-microbatch kernels lives in shared memory).
 constexpr int kMaxE = 1024;
 
+// Most expert tiles a histogram pass is cut into.
+constexpr int kMaxHistTiles = 31;
+
 struct HistArgs {
   const uint16_t* z;
   const float* tau;
@@ -67,15 +70,15 @@ struct HistArgs {
   // hist + p*E*256, and pass 2 takes shard p's selected bins from u + p*E.
   const int64_t* shard_off = nullptr;
   int P = 0;
-  // Algorithm 1's selection run by the pass's last block to finish counting
-  // (the one-call step; no shards): *done counts the blocks that finished
-  // (zero before the pass).  Pass 1 selects u, rho at rank r; pass 2 selects
-  // q_hat from u, rho and forms b_next (Eq. 2).  Selection flags go to
-  // sel_err.
+  // Algorithm 1's selections inside pass 2 (the one-call step; no shards):
+  // with `coarse` (pass 1's [E,256] counts) every block selects u, rho of its
+  // experts at rank r itself.  With `done` (zero before the pass), done[i]
+  // counts the blocks of expert tile i that finished, the tile's last one
+  // selects its q_hat, done[kMaxHistTiles] counts the tiles selected, and the
+  // last one forms b_next (Eq. 2).  Selection flags go to sel_err.
+  const int32_t* coarse = nullptr;
   int32_t* done = nullptr;
-  int64_t r = 0;
-  uint8_t* sel_u = nullptr;
-  int32_t* rho = nullptr;
+  int32_t r = 0;
   uint16_t* q_hat = nullptr;
   float* b_next = nullptr;
   int32_t* sel_err = nullptr;
@@ -108,23 +111,24 @@ struct GshardArgs {
 constexpr int64_t kLeiCoefCap = 65536;
 
 // The step's scratch, carved from one caller-provided buffer (256-byte
-// aligned pieces): the two [E,256] histograms and the passes' two block
-// counters (adjacent, cleared together before every step), u, rho, q_hat and
-// the [M,E] LEI coefficient table.
+// aligned pieces): the two [E,256] histograms and the fine pass's block
+// counters (adjacent, cleared together before every step), u and rho of the
+// separate selections, q_hat and the [M,E] LEI coefficient table.
 struct StepWorkspace {
   int32_t* H;
   int32_t* L;
-  int32_t* done;  // [2]: blocks of pass 1 and of pass 2 done counting
+  int32_t* done;  // kMaxHistTiles + 1 counters
   uint8_t* u;
   int32_t* rho;
   uint16_t* q;
   float* coef;
 };
+constexpr size_t kDoneBytes = (kMaxHistTiles + 1) * 4;
 constexpr size_t carve_round(size_t n) { return (n + 255) / 256 * 256; }
 constexpr size_t step_workspace_bytes(int E) {
-  return 2 * carve_round(static_cast<size_t>(E) * 1024) + carve_round(8) + carve_round(static_cast<size_t>(E)) +
-         carve_round(4 * static_cast<size_t>(E)) + carve_round(2 * static_cast<size_t>(E)) +
-         carve_round(4 * static_cast<size_t>(kLeiCoefCap));
+  return 2 * carve_round(static_cast<size_t>(E) * 1024) + carve_round(kDoneBytes) +
+         carve_round(static_cast<size_t>(E)) + carve_round(4 * static_cast<size_t>(E)) +
+         carve_round(2 * static_cast<size_t>(E)) + carve_round(4 * static_cast<size_t>(kLeiCoefCap));
 }
 // Carves `base` (or, with base == nullptr, only measures); returns the bytes
 // used, step_workspace_bytes(E) by construction.

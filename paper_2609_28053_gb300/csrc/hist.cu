@@ -15,15 +15,18 @@
 // PRMT (sign replicate) plus one LOP3 give both internal keys (kappa ^ 0x8000, so the stored high byte is the
 // true one ^ 0x80 and is translated back at the flush).
 //
-// Bins: a CTA owns ET experts (all E when E <= 256 is a power of two) and
-// keeps their 256 bins as 16-bit counters, two experts per 32-bit word: the
-// experts of one z word share a word, the even one in the low half, so the
-// increment is a constant.  ET * 512 bytes: 128 KiB for E = 256.  The ET/8
-// lanes covering one token each own 8 experts; lane c's rows start c words
-// past a 1 KiB boundary so equal bins of the 32 lanes fall in 32 banks.  A
-// counter gains at most one per token, so the CTA flushes (adds its non-zero
-// counters into the global int32 [E,256] histogram) at least every 65,535
-// tokens; the flush is also how token partitions are summed in device memory.
+// Bins: a CTA owns a tile of up to 128 experts (cut_hist) and keeps their
+// 256 bins as 16-bit counters, two experts per 32-bit word: the experts of
+// one z word share a word, the even one in the low half, so the increment is
+// a constant.  512 bytes per expert: 64 KiB for 128 experts.  Thread i owns
+// chunk i mod nct (8 experts) of token slot i / nct, so a warp reads
+// contiguous pieces of rows whatever the expert count; chunk c's rows start
+// c words past a 1 KiB boundary so equal bins of different chunks fall in
+// different banks.  Where a warp holds several tokens of a tile, the tile can
+// have as many copies of its bins (added at the flush).  A counter gains at
+// most one per token, so the CTA flushes (adds its non-zero counters into
+// the global int32 [E,256] histogram) at least every 65,535 tokens; the
+// flush is also how token partitions are summed in device memory.
 // Each lane keeps eight 16-byte loads in flight (eight tokens per round),
 // which covers the DRAM latency without L2 prefetches.
 //
@@ -58,102 +61,113 @@ __device__ __forceinline__ void stream_lei(const LeiStream& ls, int E, int* next
   }
 }
 
-// Algorithm 1's selection in the pass's last block to finish counting (see
-// HistArgs::done), by its nw counting warps (warp wid, lane) with barrier
-// sync(): pass 1 selects u, rho for every expert at rank a.r; pass 2 selects
-// q_hat from u, rho into global memory and a shared copy qs, then forms
-// b_next (Eq. 2).  Each warp loads the counts of three experts at a time
-// (four spill registers of the counting loop); the counts were added by
-// every block's atomics and are read from L2.
-template <int PASS, class Sync>
-__device__ void last_block_select(const HistArgs& a, int nw, int wid, int lane, uint16_t* qs, Sync sync) {
-  constexpr int B = 3;
-  const int E = a.E;
-  for (int e0 = wid; e0 < E; e0 += nw * B) {
+// Algorithm 1's selection for the experts [ea, eb) of a tile by nw warps
+// (warp wid, lane), one warp per expert, the counts of two experts in flight:
+// pick(e, i, bin, rest) receives, in every lane, expert e's first bin whose
+// prefix count reaches target(i), i = e - ea, and the rank left in it (bin
+// -1: unreachable).  The counts were added by other blocks' atomics and are
+// read from L2.  FIRST: counts in the bins of non-finite margins are flagged.
+template <bool FIRST, class Target, class Pick>
+__device__ __forceinline__ void select_tile(const int32_t* hist, int ea, int eb, int nw, int wid, int lane,
+                                            int32_t* err, Target target, Pick pick) {
+  constexpr int B = 2;
+#pragma unroll 1
+  for (int e0 = ea + wid; e0 < eb; e0 += nw * B) {
     int4 ca[B], cb[B];
-    int32_t rk[B];
-    uint32_t uk[B];
 #pragma unroll
     for (int k = 0; k < B; ++k) {
-      const int e = min(e0 + k * nw, E - 1);
-      const int4* h = reinterpret_cast<const int4*>(a.hist + (int64_t)e * 256 + lane * 8);
+      const int e = min(e0 + k * nw, eb - 1);
+      const int4* h = reinterpret_cast<const int4*>(hist + (int64_t)e * 256 + lane * 8);
       ca[k] = __ldcg(h);
       cb[k] = __ldcg(h + 1);
-      rk[k] = PASS == 2 ? __ldcg(a.rho + e) : 0;
-      uk[k] = PASS == 2 ? __ldcg(a.sel_u + e) : 0u;
     }
 #pragma unroll
     for (int k = 0; k < B; ++k) {
       const int e = e0 + k * nw;
-      if (e >= E) break;
-      const int64_t cnt[8] = {ca[k].x, ca[k].y, ca[k].z, ca[k].w, cb[k].x, cb[k].y, cb[k].z, cb[k].w};
-      if (PASS == 1)
-        warp_select(cnt, e, 1, a.r, 0u, a.sel_u, a.rho, nullptr, a.sel_err, lane);
-      else
-        warp_select(cnt, e, 2, (int64_t)rk[k], uk[k], a.sel_u, a.rho, a.q_hat, a.sel_err, lane, qs + e);
+      if (e >= eb) break;
+      const int32_t cnt[8] = {ca[k].x, ca[k].y, ca[k].z, ca[k].w, cb[k].x, cb[k].y, cb[k].z, cb[k].w};
+      if (FIRST && ((lane == 0 && cnt[0] != 0) || (lane == 31 && cnt[7] != 0))) raise_flag(err, kErrNonfinite);
+      int32_t rest = 0;
+      const int bin = warp_pick<int32_t>(cnt, target(e - ea), lane, rest);
+      if (bin < 0 && lane == 0) raise_flag(err, kErrRank);
+      pick(e, e - ea, bin, rest);
     }
-  }
-  if (PASS == 2) {
-    sync();  // every q_hat is in qs
-    block_bias_update<true>(qs, E, a.b_next, nw * 32, sync);
   }
 }
 
-template <int LPT>
-struct HistLayout {
-  static constexpr int ET = LPT * 8;            // experts per CTA
-  static constexpr int TPS = 32 / LPT;          // tokens per warp step
-  static constexpr int kRows = ET / 2;          // one row per expert pair
-  static constexpr int kWords = kRows * 256 + LPT;
-  __host__ __device__ static int row_word(int row) { return row * 256 + (row >> 2); }
-};
+// First word of pair row `row` of a block's bins (see above).
+__device__ __forceinline__ int row_word(int row) { return row * 256 + (row >> 2); }
+// Words of the bins of nct chunks, a multiple of four.
+__host__ __device__ constexpr int bin_words(int nct) { return (nct * 1024 + nct + 3) & ~3; }
+// Widest tile of a block, in 8-expert chunks.
+constexpr int kMaxTileChunks = 16;
+static_assert(kMaxE / 64 <= kMaxHistTiles, "tiles of 8 chunks or more");
 
-template <int PASS, int LPT, bool LEI>
-__global__ void __launch_bounds__(1024) hist_kernel(HistArgs a, int64_t tokens_per_cta, LeiStream ls) {
-  using Lay = HistLayout<LPT>;
+template <int PASS, bool LEI>
+__global__ void __launch_bounds__(1024) hist_kernel(HistArgs a, int tile_chunks, int copies,
+                                                    int64_t tokens_per_cta, LeiStream ls) {
   extern __shared__ __align__(16) uint32_t bins[];
   __shared__ int lei_next;  // next injection chunk of this block (fused only)
+  __shared__ uint8_t su[PASS == 2 ? kMaxTileChunks * 8 : 1];    // the tile's u and rho (the one-call step)
+  __shared__ int32_t srho[PASS == 2 ? kMaxTileChunks * 8 : 1];
   const int E = a.E;
-  const int e0 = blockIdx.x * Lay::ET;
+  const int e0 = blockIdx.x * tile_chunks * 8;
+  const int nct = min(tile_chunks, (E - e0) >> 3);  // chunks of this tile (the last may be narrower)
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int nw = LEI ? (blockDim.x >> 5) - (blockDim.x >> 7) : (blockDim.x >> 5);  // counting warps
   const int nt = nw * 32;
-  const int c = lane % LPT;     // 8-expert chunk of the tile owned by this lane
-  const int tok = lane / LPT;   // token slot inside the warp step
+  const int slots = nt / nct;                        // tokens per round of the block
+  const int tok = static_cast<int>(threadIdx.x) / nct;  // token slot (>= slots: no counting)
+  const int c = static_cast<int>(threadIdx.x) - tok * nct;  // 8-expert chunk of the tile owned by this thread
   // Barrier of the counting warps (all warps unless fused).
   auto sync_counting = [&]() {
     if (LEI) asm volatile("bar.sync 1, %0;" ::"r"(nt) : "memory");
     else __syncthreads();
   };
 
-  for (int i = threadIdx.x; i < Lay::kWords; i += blockDim.x) bins[i] = 0u;
+  const int ncp = PASS == 2 ? 1 : copies;
+  for (int i = threadIdx.x; i < bin_words(nct * ncp) / 4; i += blockDim.x)
+    reinterpret_cast<uint4*>(bins)[i] = make_uint4(0u, 0u, 0u, 0u);
   if (LEI && threadIdx.x == 0) lei_next = 0;
-  // Shared address of this lane's first pair row; pair p adds p * 1 KiB.
+  // Shared address of this thread's first pair row; pair p adds p * 1 KiB.
   const uint32_t base = static_cast<uint32_t>(__cvta_generic_to_shared(bins)) +
-                        4u * static_cast<uint32_t>(Lay::row_word(4 * c));
+                        4u * static_cast<uint32_t>(row_word(4 * (ncp > 1 ? c + tok % ncp * nct : c)));
   uint32_t sel[4] = {0, 0, 0, 0};
   // internal high bytes (u ^ 0x80) of the selected bins, placed where the
   // internal keys carry them: bits 8-15 (even expert) and 24-31 (odd).
   auto load_sel = [&](const uint8_t* ub) {
 #pragma unroll
     for (int p = 0; p < 4; ++p) {
-      const uint32_t ue = ub[e0 + c * 8 + 2 * p] ^ 0x80u;
-      const uint32_t uo = ub[e0 + c * 8 + 2 * p + 1] ^ 0x80u;
+      const uint32_t ue = ub[c * 8 + 2 * p] ^ 0x80u;
+      const uint32_t uo = ub[c * 8 + 2 * p + 1] ^ 0x80u;
       sel[p] = (ue << 8) | (uo << 24);
     }
   };
   griddep_wait();  // the bins were zeroed above; global reads start here
-  if (PASS == 2 && !a.shard_off) load_sel(a.u);
+  if (PASS == 2 && !a.shard_off && !a.coarse) load_sel(a.u + e0);
   __syncthreads();
   if (LEI && wid >= nw) {
     stream_lei(ls, E, &lei_next);
     return;
   }
+  if (PASS == 2 && a.coarse) {
+    // Algorithm 1 step 3: every block selects u, rho for its own tile
+    select_tile<true>(a.coarse, e0, e0 + nct * 8, nw, wid, lane, a.sel_err,
+                      [&](int) { return a.r; },
+                      [&](int, int i, int bin, int32_t rest) {
+                        if (lane == 0) {
+                          su[i] = static_cast<uint8_t>(bin < 0 ? 255 : bin);
+                          srho[i] = rest;
+                        }
+                      });
+    sync_counting();
+    load_sel(su);
+  }
 
   // Token indices fit in 32 bits (T < 2^31 is checked on the host).
   const int tb = static_cast<int>(min((int64_t)blockIdx.y * tokens_per_cta, a.T));
   const int te = static_cast<int>(min((int64_t)tb + tokens_per_cta, a.T));
-  const int step = nw * Lay::TPS;  // tokens per warp round
+  const int step = slots;
   const size_t zstride = static_cast<size_t>(step) * E;
   const uint16_t* zlane = a.z + e0 + c * 8;
 
@@ -193,11 +207,11 @@ __global__ void __launch_bounds__(1024) hist_kernel(HistArgs a, int64_t tokens_p
       const int64_t send = __ldg(a.shard_off + sp + 1);
       if (send > cb && send < ce) ce = static_cast<int>(send);  // chunks end at shard boundaries
       hbase = (int64_t)sp * E * 256;
-      if (PASS == 2) load_sel(a.u + (int64_t)sp * E);
+      if (PASS == 2) load_sel(a.u + (int64_t)sp * E + e0);
     }
-    int t = cb + wid * Lay::TPS + tok;
+    int t = tok < slots ? cb + tok : ce;
     const uint16_t* zp = zlane + static_cast<size_t>(t) * E;
-    // full rounds of kUnroll tokens per lane, no guards
+    // full rounds of kUnroll tokens per thread, no guards
     for (; t + (kUnroll - 1) * step < ce; t += kUnroll * step, zp += kUnroll * zstride) {
       uint4 w[kUnroll];
       float tt[kUnroll];
@@ -209,15 +223,30 @@ __global__ void __launch_bounds__(1024) hist_kernel(HistArgs a, int64_t tokens_p
 #pragma unroll
       for (int u = 0; u < kUnroll; ++u) process(w[u], tt[u]);
     }
-    for (; t < ce; t += step, zp += zstride) process(__ldcs(reinterpret_cast<const uint4*>(zp)), __ldg(a.tau + t));
+    // the rest, two tokens in flight (a block of few tokens has only these)
+    for (; t < ce; t += 2 * step, zp += 2 * zstride) {
+      const bool two = t + step < ce;
+      const uint4 w0 = __ldcs(reinterpret_cast<const uint4*>(zp));
+      const float t0 = __ldg(a.tau + t);
+      const uint4 w1 = two ? __ldcs(reinterpret_cast<const uint4*>(zp + zstride)) : make_uint4(0u, 0u, 0u, 0u);
+      const float t1 = two ? __ldg(a.tau + t + step) : 0.f;
+      process(w0, t0);
+      if (two) process(w1, t1);
+    }
     sync_counting();
     // Flush: add every non-zero 16-bit counter to the global histogram.
-    for (int i = threadIdx.x; i < Lay::kRows * 256; i += nt) {
+    for (int i = threadIdx.x; i < nct * 1024; i += nt) {
       const int row = i >> 8, slot = i & 255;
-      const int wi = Lay::row_word(row) + slot;
-      const uint32_t v = bins[wi];
+      const int wi = row_word(row) + slot;
+      uint32_t v = bins[wi];
+      if (v) bins[wi] = 0u;
+      for (int k = 1; k < ncp; ++k) {  // the copies' halves add up to at most the tokens counted
+        const int wk = row_word(row + 4 * k * nct) + slot;
+        const uint32_t vk = bins[wk];
+        if (vk) bins[wk] = 0u;
+        v += vk;
+      }
       if (v) {
-        bins[wi] = 0u;
         const int bin = (PASS == 1) ? (slot ^ 0x80) : slot;  // pass 1 stores internal keys
         const int ee = e0 + 2 * row;
         if (v & 0xffffu) atomicAdd(a.hist + hbase + (int64_t)ee * 256 + bin, static_cast<int>(v & 0xffffu));
@@ -228,62 +257,87 @@ __global__ void __launch_bounds__(1024) hist_kernel(HistArgs a, int64_t tokens_p
     sync_counting();
     cb = ce;
   }
-  if (PASS != 3 && a.done && !a.shard_off) {
-    // The last block to get here selects.  After the barrier above (every
-    // flush of this block issued), one thread's fence releases the block's
-    // flushes before its count; the last block's fence after its count
-    // orders the other blocks' flushes before its reads.
-    __shared__ int sel_last;
-    if (threadIdx.x == 0) {
-      __threadfence();
-      const bool last = atomicAdd(a.done, 1) == (int)(gridDim.x * gridDim.y) - 1;
-      if (last) __threadfence();
-      sel_last = last;
-    }
-    sync_counting();
-    if (sel_last) {
-      // the bins are clear and no longer used: they hold the q_hat copy
-      last_block_select<PASS>(a, nw, wid, lane, reinterpret_cast<uint16_t*>(bins), sync_counting);
+  if (PASS == 2 && a.done) {
+    // Algorithm 1 steps 5-6 in the last block of this expert tile to get
+    // here, for the tile's experts, and Eq. (2) in the last tile to have
+    // selected.  After a barrier (every write of this block issued), one
+    // thread's fence releases the block's writes before its count; the last
+    // block's fence after its count orders the other blocks' writes before
+    // its reads.
+    __shared__ int last;
+    auto count_last = [&](int32_t* counter, int n) {
+      if (threadIdx.x == 0) {
+        __threadfence();
+        const bool l = atomicAdd(counter, 1) == n - 1;
+        if (l) __threadfence();
+        last = l;
+      }
+      sync_counting();
+      return last != 0;
+    };
+    if (count_last(a.done + blockIdx.x, gridDim.y)) {
+      select_tile<false>(a.hist, e0, e0 + nct * 8, nw, wid, lane, a.sel_err,
+                         [&](int i) { return srho[i]; },
+                         [&](int e, int i, int bin, int32_t) {
+                           if (lane == 0) a.q_hat[e] = static_cast<uint16_t>(quantile_bits(su[i], bin));
+                         });
+      sync_counting();  // this tile's q_hat are written, and `last` was read
+      if (count_last(a.done + kMaxHistTiles, gridDim.x)) block_bias_update(a.q_hat, E, a.b_next, nt, sync_counting);
     }
   }
   if (LEI) stream_lei(ls, E, &lei_next);
 }
 
-template <int PASS, int LPT, bool LEI>
-int launch_hist_t(const HistArgs& a, const LeiStream& ls, cudaStream_t s) {
-  using Lay = HistLayout<LPT>;
-  DeviceInfo di;
-  if (int rc = device_info(&di)) return rc;
-  const int smem = Lay::kWords * 4;
-  const int nE = a.E / Lay::ET;
-  int ctas_per_sm = (228 * 1024 - 1024) / (smem + 1024);
-  if (ctas_per_sm < 1) ctas_per_sm = 1;
-  // One 1024-thread block per SM whenever the bins are large: the same
-  // threads per SM as several smaller blocks, but a third of the zeroing and
-  // flushing of the block-local counters (E = 64, 128: 10-20% faster).
-  if (smem >= 32 * 1024) ctas_per_sm = 1;
-  const int threads = ctas_per_sm == 1 ? 1024 : 512;
-  if (ctas_per_sm > 2048 / threads) ctas_per_sm = 2048 / threads;
-  int64_t nT = ((int64_t)di.sm_count * ctas_per_sm + nE - 1) / nE;
-  const int64_t max_nT = (a.T + 2047) / 2048;  // keep >= ~2K tokens per CTA
-  if (nT > max_nT) nT = max_nT;
-  if (nT < 1) nT = 1;
-  const int64_t tpc = (a.T + nT - 1) / nT;
-  auto kern = hist_kernel<PASS, LPT, LEI>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
-    return kErrCuda;
-  dim3 grid((unsigned)nE, (unsigned)nT);
-  return launch_dependent(kern, grid, dim3(threads), smem, s, a, tpc, ls) == cudaSuccess ? kOk : kErrCuda;
+// How a pass is cut into blocks: expert tiles of `chunks` 8-expert chunks
+// times token ranges of `tpc` tokens, about one block per SM, each with
+// `copies` copies of its tile's bins.
+struct HistCut {
+  int tiles, chunks, copies, ranges;
+  int64_t tpc;
+};
+
+// A block's fixed cost (zeroing, flushing and selecting over its tile's bins)
+// grows with the tile; what narrow tiles cost is lanes of a warp that count
+// the same experts and meet in popular bins.  Measured on pass 1 / pass 2 /
+// the step without LEI, us, for tiles of 8, 16 and 32 chunks: T = 30,873,
+// E = 256 (6,500 chunks of z per SM) 9.2 / 6.3 / 40, 9.5 / 7.0 / 45 and
+// 12.0 / 8.2 / 74 (one 32-chunk tile on 2,048-token blocks before: 33.5 /
+// 27.1 / 93); T = 147,456 (31,000) 27 / 15 / 81, 21 / 16 / 76 and 22 / 17 /
+// 89; T = 1,048,576, E = 384 143 / 134 / 462 for 16, 162 / 136 / 487 for 24.
+// From 7,000 chunks per SM on, copies that give the 32 lanes of a warp bins
+// of their own pay for their zeroing: T = 1,000,000, E = 64 31 us against
+// 45 (pass 1), T = 60,000, E = 160 10.3 against 12.1; T = 65,536, E = 64
+// (3,400) 7.5 against 6.8.  Pass 2 counts few elements and takes one copy.
+HistCut cut_hist(int64_t T, int E, int pass, int sm_count) {
+  const int nch = E >> 3;
+  const int64_t per_sm = T * nch / sm_count;  // chunks of z to count per SM
+  const int want = per_sm < 10000 ? 8 : 16;
+  HistCut h;
+  h.tiles = (nch + want - 1) / want;
+  h.chunks = (nch + h.tiles - 1) / h.tiles;
+  h.tiles = (nch + h.chunks - 1) / h.chunks;
+  h.copies = pass != 2 && per_sm >= 7000 ? 32 / h.chunks : 1;
+  int64_t ranges = sm_count / h.tiles;
+  const int64_t most = (T * h.chunks + 1023) / 1024;  // a chunk for every thread
+  if (ranges > most) ranges = most;
+  if (ranges < 1) ranges = 1;
+  h.tpc = (T + ranges - 1) / ranges;
+  h.ranges = static_cast<int>((T + h.tpc - 1) / h.tpc);
+  return h;
 }
 
 template <int PASS, bool LEI>
 int launch_hist_pass(const HistArgs& a, const LeiStream& ls, cudaStream_t s) {
-  if (a.E % 256 == 0) return launch_hist_t<PASS, 32, LEI>(a, ls, s);
-  if (a.E % 128 == 0) return launch_hist_t<PASS, 16, LEI>(a, ls, s);
-  if (a.E % 64 == 0) return launch_hist_t<PASS, 8, LEI>(a, ls, s);
-  if (a.E % 32 == 0) return launch_hist_t<PASS, 4, LEI>(a, ls, s);
-  if (a.E % 16 == 0) return launch_hist_t<PASS, 2, LEI>(a, ls, s);
-  return launch_hist_t<PASS, 1, LEI>(a, ls, s);
+  DeviceInfo di;
+  if (int rc = device_info(&di)) return rc;
+  const HistCut h = cut_hist(a.T, a.E, PASS, di.sm_count);
+  const int smem = bin_words(h.chunks * h.copies) * 4;
+  auto kern = hist_kernel<PASS, LEI>;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
+    return kErrCuda;
+  dim3 grid((unsigned)h.tiles, (unsigned)h.ranges);
+  return launch_dependent(kern, grid, dim3(1024), smem, s, a, h.chunks, h.copies, h.tpc, ls) == cudaSuccess ? kOk
+                                                                                                      : kErrCuda;
 }
 
 }  // namespace

@@ -9,8 +9,6 @@
 //           q_hat_e = kappa^{-1}((u_e << 8) | v_e)   (a zero returned as +0)
 //   pass 3: pass 1 on a histogram of equal-width bins, whose edge bins hold
 //           ordinary (clamped) margins rather than non-finite ones
-//   pass 3: as pass 1 on a histogram of equal-width bins, where the edge bins
-//           hold ordinary (clamped) values rather than non-finite margins
 // The bias update reproduces the definition's fp64 sum in ascending expert
 // order bit for bit (see bias_update_kernel), divides by E and subtracts.
 #include "select_device.cuh"
@@ -51,13 +49,22 @@ __global__ void __launch_bounds__(256) select_kernel(const int32_t* __restrict__
 #pragma unroll
   for (int j = 0; j < 8; ++j) cnt[j] = h[j];
   const int64_t target = pass != 2 ? r : (int64_t)rho[e];
-  const uint32_t u_e = pass == 2 ? u[e] : 0u;
-  warp_select(cnt, e, pass, target, u_e, u, rho, q_hat, err, lane);
+  if (pass == 1 && ((lane == 0 && cnt[0] != 0) || (lane == 31 && cnt[7] != 0))) raise_flag(err, kErrNonfinite);
+  int64_t rest = 0;
+  const int bin = warp_pick<int64_t>(cnt, target, lane, rest);
+  if (lane != 0) return;
+  if (bin < 0) raise_flag(err, kErrRank);
+  if (pass != 2) {
+    u[e] = static_cast<uint8_t>(bin < 0 ? 255 : bin);
+    rho[e] = static_cast<int32_t>(rest);
+  } else {
+    q_hat[e] = static_cast<uint16_t>(quantile_bits(u[e], bin));
+  }
 }
 
 __global__ void bias_update_kernel(const uint16_t* __restrict__ q_hat, int E, float* __restrict__ b_next) {
   griddep_wait();
-  block_bias_update<false>(q_hat, E, b_next, blockDim.x, [] { __syncthreads(); });
+  block_bias_update(q_hat, E, b_next, blockDim.x, [] { __syncthreads(); });
 }
 
 }  // namespace

@@ -1,68 +1,52 @@
 // select_device.cuh -- the per-expert selection of Algorithm 1 (steps 3 and
 // 5-6) and the Eq. (2) centering (arXiv 2609.28053, Sec. 2 and App. C), as
-// device functions shared by the selection kernels (select.cu) and by the
-// histogram passes, whose last block to finish counting runs them in the
-// one-call step (hist.cu).
+// device functions shared by the selection kernels (select.cu) and the fine
+// histogram pass, which selects in its blocks in the one-call step
+// (hist.cu).
 #pragma once
 
 #include "eqb_device.cuh"
 
 namespace eqb {
 
-// One warp selects for expert e from its 256 counts, lane j holding bins
-// 8j..8j+7 (cnt): pass 1 writes u[e] and rho[e] for the rank `target`, pass 2
-// writes q_hat[e] (and *qs, when given) from u_e = u[e] and the rank target =
-// rho[e], both read by the caller beside the counts.  Flags a count in
-// high-byte bin 0x00 or 0xff (pass 1) and an unreachable rank.
-__device__ __forceinline__ void warp_select(const int64_t (&cnt)[8], int e, int pass, int64_t target,
-                                            uint32_t u_e, uint8_t* __restrict__ u, int32_t* __restrict__ rho,
-                                            uint16_t* __restrict__ q_hat, int32_t* err, int lane,
-                                            uint16_t* qs = nullptr) {
-  int64_t local = 0;
+// The first of 256 bins whose inclusive prefix count reaches `target`, lane j
+// of the warp holding the counts of bins 8j..8j+7: every lane gets the bin
+// (-1: the target is below 1 or above the total) and `rest` = target minus
+// the counts below that bin.  I is wide enough for the total count.
+template <class I>
+__device__ __forceinline__ int warp_pick(const I (&cnt)[8], I target, int lane, I& rest) {
+  I incl = 0;
 #pragma unroll
-  for (int j = 0; j < 8; ++j) local += cnt[j];
-  int64_t incl = local;
+  for (int j = 0; j < 8; ++j) incl += cnt[j];
+  I cum = -incl;  // becomes the count below this lane's bins
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
-    const int64_t o = __shfl_up_sync(kFull, incl, d);
+    const I o = __shfl_up_sync(kFull, incl, d);
     if (lane >= d) incl += o;
   }
-  const int64_t excl = incl - local;
-  const bool first = pass != 2;
-  const unsigned hit = __ballot_sync(kFull, excl < target && target <= incl);
-  if (pass == 1 && ((lane == 0 && cnt[0] != 0) || (lane == 31 && cnt[7] != 0)))
-    raise_flag(err, kErrNonfinite);
-  if (hit == 0u || target < 1) {
-    if (lane == 0) {
-      raise_flag(err, kErrRank);
-      if (first) { u[e] = 255; rho[e] = 0; }
-      else {
-        q_hat[e] = 0x7fc0;  // NaN marks an unreachable rank
-        if (qs) *qs = 0x7fc0;
-      }
-    }
-    return;
-  }
-  if (lane == __ffs(hit) - 1) {
-    int64_t below = excl;
+  cum += incl;
+  const unsigned hit = __ballot_sync(kFull, cum < target && target <= incl);
+  int bin = lane * 8;
+  I below = cum;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      if (below + cnt[j] >= target) {
-        const int bin = lane * 8 + j;
-        if (first) {
-          u[e] = static_cast<uint8_t>(bin);
-          rho[e] = static_cast<int32_t>(target - below);
-        } else {
-          uint32_t q = kappa16_inv((u_e << 8) | static_cast<uint32_t>(bin));
-          if (q == 0x8000u) q = 0u;
-          q_hat[e] = static_cast<uint16_t>(q);
-          if (qs) *qs = static_cast<uint16_t>(q);
-        }
-        break;
-      }
-      below += cnt[j];
-    }
+  for (int j = 0; j < 7; ++j) {  // the target lies in this lane's bins: not past the last
+    cum += cnt[j];
+    const bool past = cum < target;
+    bin += past ? 1 : 0;
+    below = past ? cum : below;
   }
+  if (hit == 0u || target < 1) return -1;
+  const int src = __ffs(hit) - 1;
+  rest = __shfl_sync(kFull, target - below, src);
+  return __shfl_sync(kFull, bin, src);
+}
+
+// bf16 pattern of the quantile with high key byte u_e and low byte v (a zero
+// is returned as +0; v < 0, an unreachable rank, as NaN).
+__device__ __forceinline__ uint32_t quantile_bits(uint32_t u_e, int v) {
+  if (v < 0) return 0x7fc0u;
+  const uint32_t q = kappa16_inv((u_e << 8) | static_cast<uint32_t>(v));
+  return q == 0x8000u ? 0u : q;
 }
 
 // Exponent range of a non-zero bf16 pattern: [ulp exponent, leading-bit exponent].
@@ -81,19 +65,19 @@ __device__ __forceinline__ void bf16_exp_range(uint32_t x, int& lo, int& hi) {
 // thread sums in ascending order.
 // Threads [0, nthreads) of the block compute b_next from q_hat (they share
 // the final subtraction; warp 0 forms the mean); sync() is their barrier.
-// SHARED_Q: q_hat is the block's shared-memory copy; otherwise the global
-// array, read through L2 (it may have been written earlier in the same
-// kernel).
-template <bool SHARED_Q, class Sync>
+// q_hat is read through L2 (it may have been written earlier in the same
+// kernel, by other blocks).
+template <class Sync>
 __device__ __forceinline__ void block_bias_update(const uint16_t* q_hat, int E, float* __restrict__ b_next,
                                                   int nthreads, Sync sync) {
   __shared__ double mean;
-  auto q_at = [&](int e) -> uint32_t { return SHARED_Q ? q_hat[e] : __ldcg(q_hat + e); };
+  auto q_at = [&](int e) -> uint32_t { return __ldcg(q_hat + e); };
 
   if (threadIdx.x < 32) {
     const int lane = threadIdx.x;
     double part = 0.0;
     int lo = 1 << 20, hi = -(1 << 20);
+#pragma unroll 4
     for (int e = lane; e < E; e += 32) {
       const uint32_t x = q_at(e);
       if ((x & 0x7fffu) != 0u) {

@@ -29,7 +29,7 @@ size_t carve_workspace(void* base, int E, StepWorkspace* w) {
   };
   w->H = reinterpret_cast<int32_t*>(take(static_cast<size_t>(E) * 256 * 4));
   w->L = reinterpret_cast<int32_t*>(take(static_cast<size_t>(E) * 256 * 4));
-  w->done = reinterpret_cast<int32_t*>(take(8));
+  w->done = reinterpret_cast<int32_t*>(take(kDoneBytes));
   w->u = take(static_cast<size_t>(E));
   w->rho = reinterpret_cast<int32_t*>(take(static_cast<size_t>(E) * 4));
   w->q = reinterpret_cast<uint16_t*>(take(static_cast<size_t>(E) * 2));
@@ -89,34 +89,26 @@ eqb_status clear(const Workspace& w, int32_t* loads, int32_t E, int32_t M, cudaS
   // H, L and the block counters are adjacent in the workspace (H and L each
   // E*1 KiB, a multiple of the 256-byte carve alignment): one memset clears
   // them.
-  if (cudaMemsetAsync(w.H, 0, 2 * eqb::carve_round(static_cast<size_t>(E) * 1024) + eqb::carve_round(8), s) !=
+  if (cudaMemsetAsync(w.H, 0, 2 * eqb::carve_round(static_cast<size_t>(E) * 1024) + eqb::carve_round(eqb::kDoneBytes), s) !=
           cudaSuccess ||
       cudaMemsetAsync(loads, 0, static_cast<size_t>(M) * E * 4, s) != cudaSuccess)
     return EQB_ERR_CUDA;
   return EQB_OK;
 }
 
-// The two histogram passes of the step, each with its selection run by the
-// pass's last block to finish counting (so neither selection is a launch of
-// its own, and each overlaps the other blocks' LEI streaming): pass 1 counts
-// H and selects u, rho at rank r; pass 2 counts L from u and selects q_hat,
-// then b_next (Eq. 2).
-eqb::HistArgs pass1_args(const Workspace& w, const eqb_bf16* z, const float* tau, int64_t T, int32_t E, int64_t r,
+// The two histogram passes of the step: pass 1 counts H; pass 2 selects u, rho
+// from H at rank r in every block, counts L, selects q_hat and forms b_next
+// (Eq. 2), so no selection is a launch of its own.
+eqb::HistArgs pass1_args(const Workspace& w, const eqb_bf16* z, const float* tau, int64_t T, int32_t E,
                          int32_t* err_flag) {
-  eqb::HistArgs h{z, tau, T, E, nullptr, w.H, err_flag};
-  h.done = w.done;
-  h.r = r;
-  h.sel_u = w.u;
-  h.rho = w.rho;
-  h.sel_err = err_flag;
-  return h;
+  return eqb::HistArgs{z, tau, T, E, nullptr, w.H, err_flag};
 }
-eqb::HistArgs pass2_args(const Workspace& w, const eqb_bf16* z, const float* tau, int64_t T, int32_t E,
+eqb::HistArgs pass2_args(const Workspace& w, const eqb_bf16* z, const float* tau, int64_t T, int32_t E, int64_t r,
                          float* b_next, int32_t* err_flag) {
-  eqb::HistArgs h{z, tau, T, E, w.u, w.L, nullptr};
-  h.done = w.done + 1;
-  h.sel_u = w.u;
-  h.rho = w.rho;
+  eqb::HistArgs h{z, tau, T, E, nullptr, w.L, nullptr};
+  h.coarse = w.H;
+  h.done = w.done;
+  h.r = static_cast<int32_t>(r < INT32_MAX ? r : INT32_MAX);  // T < INT32_MAX: a larger rank is as unreachable
   h.q_hat = w.q;
   h.b_next = b_next;
   h.sel_err = err_flag;
@@ -133,8 +125,8 @@ eqb_status after_routing(const Workspace& w, const eqb_bf16* z, int64_t T, int32
                          const int64_t* mb_offsets, int32_t M, int64_t r, const float* tau,
                          const int32_t* loads, float* b_next, float* grad_s, float eta, float c,
                          int32_t* err_flag, cudaStream_t s) {
-  const eqb::HistArgs h1 = pass1_args(w, z, tau, T, E, r, err_flag);
-  const eqb::HistArgs h2 = pass2_args(w, z, tau, T, E, b_next, err_flag);
+  const eqb::HistArgs h1 = pass1_args(w, z, tau, T, E, err_flag);
+  const eqb::HistArgs h2 = pass2_args(w, z, tau, T, E, r, b_next, err_flag);
   if (grad_s && static_cast<int64_t>(M) * E <= eqb::kLeiCoefCap) {
     eqb::LeiArgs la{grad_s, loads, mb_offsets, M, 0, T, E, K, eta, c};
     if (int rc = eqb::launch_lei_coef(la, w.coef, s)) return st(rc);
@@ -166,8 +158,7 @@ eqb_status after_coarse(const Workspace& w, const eqb_bf16* z, int64_t T, int32_
     eqb::LeiArgs la{grad_s, loads, mb_offsets, M, 0, T, E, K, eta, c};
     if (int rc = eqb::launch_lei_coef(la, w.coef, s)) return st(rc);
   }
-  if (int rc = eqb::launch_select(w.H, E, 1, r, w.u, w.rho, nullptr, err_flag, s)) return st(rc);
-  const eqb::HistArgs h2 = pass2_args(w, z, tau, T, E, b_next, err_flag);
+  const eqb::HistArgs h2 = pass2_args(w, z, tau, T, E, r, b_next, err_flag);
   if (lei) {
     eqb::LeiStream l2{grad_s, w.coef, mb_offsets, M, 0, T};
     if (int rc = eqb::launch_hist_lei(h2, 2, l2, s)) return st(rc);

@@ -10,7 +10,7 @@
 //
 // The scratch is one file-scope device array sized for the largest supported
 // E (256 experts): eqb_layer_workspace_bytes(256) = 788,480 bytes (the two
-// [256,256] histograms, two block counters, u, rho, q_hat and the
+// [256,256] histograms, block counters, u, rho, q_hat and the
 // 65,536-float LEI coefficient table).  Every GPU that loads this library
 // holds it until the process exits.  Host code cannot use the array's name as a
 // device address, so the first call on each device, with that device
