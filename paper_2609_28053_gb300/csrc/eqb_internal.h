@@ -133,6 +133,9 @@ constexpr size_t step_workspace_bytes(int E) {
 // Carves `base` (or, with base == nullptr, only measures); returns the bytes
 // used, step_workspace_bytes(E) by construction.
 size_t carve_workspace(void* base, int E, StepWorkspace* w);
+// Zeros the workspace's histograms and counters and the loads [n]: the first
+// kernel of a step.
+int launch_clear(const StepWorkspace& w, int E, int32_t* loads, int64_t n, cudaStream_t s);
 
 int launch_route(const RouteArgs& a, cudaStream_t s);
 bool route_wide_supported(int E, int K);
@@ -142,6 +145,9 @@ int launch_route_wide(const RouteArgs& a, cudaStream_t s);
 bool route_hist_supported(int E, int K);
 int launch_route_hist(const RouteArgs& a, int32_t* hist, cudaStream_t s);
 int launch_hist(const HistArgs& a, int pass, cudaStream_t s);
+// Pass 1 with a few of its blocks forming the [M,E] LEI coefficient table of
+// `la` (the step: the loads are complete, the fine pass injects).
+int launch_hist_coef(const HistArgs& a, const LeiArgs& la, float* coef, cudaStream_t s);
 // A histogram pass (1 or 2) with the injection `ls` streamed beside it.
 int launch_hist_lei(const HistArgs& a, int pass, const LeiStream& ls, cudaStream_t s);
 int launch_select(const int32_t* hist, int E, int pass, int64_t r, uint8_t* u, int32_t* rho,

@@ -27,8 +27,8 @@
 // most one per token, so the CTA flushes (adds its non-zero counters into
 // the global int32 [E,256] histogram) at least every 65,535 tokens; the
 // flush is also how token partitions are summed in device memory.
-// Each lane keeps eight 16-byte loads in flight (eight tokens per round),
-// which covers the DRAM latency without L2 prefetches.
+// Each thread keeps several 16-byte loads in flight (kUnroll tokens per
+// round), which covers the DRAM latency without L2 prefetches.
 //
 // Fused with Load-Error Injection (the one-call step): the passes are bound
 // by issue, not by DRAM, while LEI (Sec. 4) is a pure DRAM stream that needs
@@ -38,23 +38,37 @@
 // its counting is done; the stream is cut into chunks of about 8 KiB of
 // grad_s handed out by a shared counter, so no warp idles while the block
 // has work.  Each pass carries half of the step's tokens, which turns both
-// passes into DRAM-bound ones.
+// passes into DRAM-bound ones; where a pass is short, the fine pass carries
+// all of them and a few blocks of the coarse pass form the coefficients.
+#include "lei_device.cuh"
 #include "select_device.cuh"
 
 namespace eqb {
 
 namespace {
 
-constexpr int kUnroll = 8;  // 16-byte loads in flight per lane (64 registers at 1024 threads)
+// 16-byte loads in flight per thread (64 registers at 1024 threads).  Pass 1 /
+// pass 2 alone at T = 2,097,152, E = 256: 187 / 171 us with six, 185 / 185
+// with seven, 194 / 184 with eight, 221 / 181 with four.  Beside the injection
+// eight (the step at T = 1,048,576, E = 512 1229 us, 1241 with six).
+template <bool LEI>
+constexpr int kUnroll = LEI ? 8 : 6;
 constexpr int64_t kFlushTokens = 65535;
+
+// The LEI coefficient table formed by blocks of pass 1 (none: blocks == 0).
+struct CoefRows {
+  LeiArgs a = {};
+  float* coef = nullptr;
+  int blocks = 0;
+};
+
 // The injection share of a fused block (see above): chunks of about 8 KiB of
 // grad_s from this block's slice of [ls.t0, ls.t1), taken through the shared
 // counter *next.  Every element gets one fp32 addition (round to nearest) of
 // its microbatch's coefficient, as in lei.cu.
 __device__ __forceinline__ void stream_lei(const LeiStream& ls, int E, int* next) {
   int64_t q0, q1;
-  lei_block_slice(ls.t0, ls.t1, (int64_t)blockIdx.y * gridDim.x + blockIdx.x, (int64_t)gridDim.x * gridDim.y, &q0,
-                  &q1);
+  lei_block_slice(ls.t0, ls.t1, blockIdx.x, gridDim.x, &q0, &q1);
   int64_t mlo = 1, mhi = 0;  // token range of microbatch ml (none yet)
   int ml = 0;
   while (lei_warp_next_chunk(ls, E, q0, q1, next, mlo, mhi, ml)) {
@@ -103,35 +117,63 @@ __host__ __device__ constexpr int bin_words(int nct) { return (nct * 1024 + nct 
 constexpr int kMaxTileChunks = 16;
 static_assert(kMaxE / 64 <= kMaxHistTiles, "tiles of 8 chunks or more");
 
+// Where a thread stands in the pass's cut (cut_hist): read from the special
+// registers at every construction, never carried over from an earlier one.
+struct HistPlace {
+  int tid, lane, wid;
+  int tile, range;  // expert tile and token range of the block
+  int e0, nct;      // the tile's first expert and its chunks (the last tile may be narrower)
+  int nw, nt;       // counting warps and threads (a quarter of a fused block streams LEI)
+  __device__ __forceinline__ HistPlace(int tiles, int tile_chunks, int E, bool lei) {
+    int cta, n;
+    asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tid));
+    asm volatile("mov.u32 %0, %%ctaid.x;" : "=r"(cta));
+    asm volatile("mov.u32 %0, %%ntid.x;" : "=r"(n));
+    lane = tid & 31;
+    wid = tid >> 5;
+    tile = cta % tiles;
+    range = cta / tiles;
+    e0 = tile * tile_chunks * 8;
+    nct = min(tile_chunks, (E - e0) >> 3);
+    nw = lei ? (n >> 5) - (n >> 7) : n >> 5;
+    nt = nw * 32;
+  }
+};
+
 template <int PASS, bool LEI>
-__global__ void __launch_bounds__(1024) hist_kernel(HistArgs a, int tile_chunks, int copies,
-                                                    int64_t tokens_per_cta, LeiStream ls) {
+__global__ void __launch_bounds__(1024) hist_kernel(HistArgs a, int tiles, int tile_chunks, int copies,
+                                                    int64_t tokens_per_cta, LeiStream ls, CoefRows cr) {
+  constexpr int U = kUnroll<LEI>;
   extern __shared__ __align__(16) uint32_t bins[];
   __shared__ int lei_next;  // next injection chunk of this block (fused only)
   __shared__ uint8_t su[PASS == 2 ? kMaxTileChunks * 8 : 1];    // the tile's u and rho (the one-call step)
   __shared__ int32_t srho[PASS == 2 ? kMaxTileChunks * 8 : 1];
   const int E = a.E;
-  const int e0 = blockIdx.x * tile_chunks * 8;
-  const int nct = min(tile_chunks, (E - e0) >> 3);  // chunks of this tile (the last may be narrower)
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int nw = LEI ? (blockDim.x >> 5) - (blockDim.x >> 7) : (blockDim.x >> 5);  // counting warps
-  const int nt = nw * 32;
-  const int slots = nt / nct;                        // tokens per round of the block
-  const int tok = static_cast<int>(threadIdx.x) / nct;  // token slot (>= slots: no counting)
-  const int c = static_cast<int>(threadIdx.x) - tok * nct;  // 8-expert chunk of the tile owned by this thread
+  if (PASS == 1 && !LEI && blockIdx.x >= gridDim.x - cr.blocks) {
+    // the last cr.blocks blocks form the coefficient table meanwhile
+    griddep_wait();
+    for (int l = blockIdx.x - (gridDim.x - cr.blocks); l < cr.a.M; l += cr.blocks) {
+      const int64_t n = __ldg(cr.a.off + l + 1) - __ldg(cr.a.off + l);
+      block_lei_coef<1024>(cr.a.loads + (int64_t)l * E, n, E, cr.a.K, cr.a.eta, cr.a.c, cr.coef + (int64_t)l * E);
+    }
+    return;
+  }
+  const HistPlace pl(tiles, tile_chunks, E, LEI);
+  const int tok = pl.tid / pl.nct;           // token slot (>= slots: no counting)
+  const int c = pl.tid - tok * pl.nct;       // 8-expert chunk of the tile owned by this thread
   // Barrier of the counting warps (all warps unless fused).
   auto sync_counting = [&]() {
-    if (LEI) asm volatile("bar.sync 1, %0;" ::"r"(nt) : "memory");
+    if (LEI) asm volatile("bar.sync 1, %0;" ::"r"(pl.nt) : "memory");
     else __syncthreads();
   };
 
   const int ncp = PASS == 2 ? 1 : copies;
-  for (int i = threadIdx.x; i < bin_words(nct * ncp) / 4; i += blockDim.x)
+  for (int i = threadIdx.x; i < bin_words(pl.nct * ncp) / 4; i += blockDim.x)
     reinterpret_cast<uint4*>(bins)[i] = make_uint4(0u, 0u, 0u, 0u);
   if (LEI && threadIdx.x == 0) lei_next = 0;
   // Shared address of this thread's first pair row; pair p adds p * 1 KiB.
   const uint32_t base = static_cast<uint32_t>(__cvta_generic_to_shared(bins)) +
-                        4u * static_cast<uint32_t>(row_word(4 * (ncp > 1 ? c + tok % ncp * nct : c)));
+                        4u * static_cast<uint32_t>(row_word(4 * (ncp > 1 ? c + tok % ncp * pl.nct : c)));
   uint32_t sel[4] = {0, 0, 0, 0};
   // internal high bytes (u ^ 0x80) of the selected bins, placed where the
   // internal keys carry them: bits 8-15 (even expert) and 24-31 (odd).
@@ -144,18 +186,18 @@ __global__ void __launch_bounds__(1024) hist_kernel(HistArgs a, int tile_chunks,
     }
   };
   griddep_wait();  // the bins were zeroed above; global reads start here
-  if (PASS == 2 && !a.shard_off && !a.coarse) load_sel(a.u + e0);
+  if (PASS == 2 && !a.shard_off && !a.coarse) load_sel(a.u + pl.e0);
   __syncthreads();
-  if (LEI && wid >= nw) {
+  if (LEI && pl.wid >= pl.nw) {
     stream_lei(ls, E, &lei_next);
     return;
   }
   if (PASS == 2 && a.coarse) {
     // Algorithm 1 step 3: every block selects u, rho for its own tile
-    select_tile<true>(a.coarse, e0, e0 + nct * 8, nw, wid, lane, a.sel_err,
+    select_tile<true>(a.coarse, pl.e0, pl.e0 + pl.nct * 8, pl.nw, pl.wid, pl.lane, a.sel_err,
                       [&](int) { return a.r; },
                       [&](int, int i, int bin, int32_t rest) {
-                        if (lane == 0) {
+                        if (pl.lane == 0) {
                           su[i] = static_cast<uint8_t>(bin < 0 ? 255 : bin);
                           srho[i] = rest;
                         }
@@ -165,11 +207,10 @@ __global__ void __launch_bounds__(1024) hist_kernel(HistArgs a, int tile_chunks,
   }
 
   // Token indices fit in 32 bits (T < 2^31 is checked on the host).
-  const int tb = static_cast<int>(min((int64_t)blockIdx.y * tokens_per_cta, a.T));
+  const int tb = static_cast<int>(min((int64_t)pl.range * tokens_per_cta, a.T));
   const int te = static_cast<int>(min((int64_t)tb + tokens_per_cta, a.T));
-  const int step = slots;
-  const size_t zstride = static_cast<size_t>(step) * E;
-  const uint16_t* zlane = a.z + e0 + c * 8;
+  const int step = pl.nt / pl.nct;  // token slots: tokens per round of the block
+  const uint32_t zstep = static_cast<uint32_t>(step) * static_cast<uint32_t>(E) * 2u;  // bytes of z per round
 
   auto process = [&](const uint4& w4, float tv) {
     const uint32_t zw[4] = {w4.x, w4.y, w4.z, w4.w};
@@ -207,48 +248,52 @@ __global__ void __launch_bounds__(1024) hist_kernel(HistArgs a, int tile_chunks,
       const int64_t send = __ldg(a.shard_off + sp + 1);
       if (send > cb && send < ce) ce = static_cast<int>(send);  // chunks end at shard boundaries
       hbase = (int64_t)sp * E * 256;
-      if (PASS == 2) load_sel(a.u + (int64_t)sp * E + e0);
+      if (PASS == 2) load_sel(a.u + (int64_t)sp * E + pl.e0);
     }
-    int t = tok < slots ? cb + tok : ce;
-    const uint16_t* zp = zlane + static_cast<size_t>(t) * E;
-    // full rounds of kUnroll tokens per thread, no guards
-    for (; t + (kUnroll - 1) * step < ce; t += kUnroll * step, zp += kUnroll * zstride) {
-      uint4 w[kUnroll];
-      float tt[kUnroll];
+    int t = tok < step ? cb + tok : ce;
+    const char* zp = reinterpret_cast<const char*>(a.z + static_cast<size_t>(t) * E + pl.e0 + c * 8);
+    // full rounds of U tokens per thread, no guards
+    for (; t + (U - 1) * step < ce; t += U * step, zp += U * zstep) {
+      uint4 w[U];
+      float tt[U];
 #pragma unroll
-      for (int u = 0; u < kUnroll; ++u) {
-        w[u] = __ldcs(reinterpret_cast<const uint4*>(zp + u * zstride));
+      for (int u = 0; u < U; ++u) {
+        w[u] = __ldcs(reinterpret_cast<const uint4*>(zp + u * zstep));
         tt[u] = __ldg(a.tau + t + u * step);
       }
+      asm volatile("" ::: "memory");  // every load is issued before the first count
 #pragma unroll
-      for (int u = 0; u < kUnroll; ++u) process(w[u], tt[u]);
+      for (int u = 0; u < U; ++u) process(w[u], tt[u]);
     }
     // the rest, two tokens in flight (a block of few tokens has only these)
-    for (; t < ce; t += 2 * step, zp += 2 * zstride) {
+    for (; t < ce; t += 2 * step, zp += 2 * zstep) {
       const bool two = t + step < ce;
       const uint4 w0 = __ldcs(reinterpret_cast<const uint4*>(zp));
       const float t0 = __ldg(a.tau + t);
-      const uint4 w1 = two ? __ldcs(reinterpret_cast<const uint4*>(zp + zstride)) : make_uint4(0u, 0u, 0u, 0u);
+      const uint4 w1 = two ? __ldcs(reinterpret_cast<const uint4*>(zp + zstep)) : make_uint4(0u, 0u, 0u, 0u);
       const float t1 = two ? __ldg(a.tau + t + step) : 0.f;
       process(w0, t0);
       if (two) process(w1, t1);
     }
+    // from here on the thread's place is formed anew, so that the counting
+    // loop does not hold it in registers
+    const HistPlace fl(tiles, tile_chunks, E, LEI);
     sync_counting();
     // Flush: add every non-zero 16-bit counter to the global histogram.
-    for (int i = threadIdx.x; i < nct * 1024; i += nt) {
+    for (int i = fl.tid; i < fl.nct * 1024; i += fl.nt) {
       const int row = i >> 8, slot = i & 255;
       const int wi = row_word(row) + slot;
       uint32_t v = bins[wi];
       if (v) bins[wi] = 0u;
       for (int k = 1; k < ncp; ++k) {  // the copies' halves add up to at most the tokens counted
-        const int wk = row_word(row + 4 * k * nct) + slot;
+        const int wk = row_word(row + 4 * k * fl.nct) + slot;
         const uint32_t vk = bins[wk];
         if (vk) bins[wk] = 0u;
         v += vk;
       }
       if (v) {
         const int bin = (PASS == 1) ? (slot ^ 0x80) : slot;  // pass 1 stores internal keys
-        const int ee = e0 + 2 * row;
+        const int ee = fl.e0 + 2 * row;
         if (v & 0xffffu) atomicAdd(a.hist + hbase + (int64_t)ee * 256 + bin, static_cast<int>(v & 0xffffu));
         if (v >> 16) atomicAdd(a.hist + hbase + (int64_t)(ee + 1) * 256 + bin, static_cast<int>(v >> 16));
         if (PASS == 1 && (bin == 0 || bin == 255)) raise_flag(a.err, kErrNonfinite);
@@ -265,8 +310,9 @@ __global__ void __launch_bounds__(1024) hist_kernel(HistArgs a, int tile_chunks,
     // block's fence after its count orders the other blocks' writes before
     // its reads.
     __shared__ int last;
+    const HistPlace fl(tiles, tile_chunks, E, LEI);
     auto count_last = [&](int32_t* counter, int n) {
-      if (threadIdx.x == 0) {
+      if (fl.tid == 0) {
         __threadfence();
         const bool l = atomicAdd(counter, 1) == n - 1;
         if (l) __threadfence();
@@ -275,14 +321,14 @@ __global__ void __launch_bounds__(1024) hist_kernel(HistArgs a, int tile_chunks,
       sync_counting();
       return last != 0;
     };
-    if (count_last(a.done + blockIdx.x, gridDim.y)) {
-      select_tile<false>(a.hist, e0, e0 + nct * 8, nw, wid, lane, a.sel_err,
+    if (count_last(a.done + fl.tile, (int)gridDim.x / tiles)) {
+      select_tile<false>(a.hist, fl.e0, fl.e0 + fl.nct * 8, fl.nw, fl.wid, fl.lane, a.sel_err,
                          [&](int i) { return srho[i]; },
                          [&](int e, int i, int bin, int32_t) {
-                           if (lane == 0) a.q_hat[e] = static_cast<uint16_t>(quantile_bits(su[i], bin));
+                           if (fl.lane == 0) a.q_hat[e] = static_cast<uint16_t>(quantile_bits(su[i], bin));
                          });
       sync_counting();  // this tile's q_hat are written, and `last` was read
-      if (count_last(a.done + kMaxHistTiles, gridDim.x)) block_bias_update(a.q_hat, E, a.b_next, nt, sync_counting);
+      if (count_last(a.done + kMaxHistTiles, tiles)) block_bias_update(a.q_hat, E, a.b_next, fl.nt, sync_counting);
     }
   }
   if (LEI) stream_lei(ls, E, &lei_next);
@@ -308,16 +354,16 @@ struct HistCut {
 // of their own pay for their zeroing: T = 1,000,000, E = 64 31 us against
 // 45 (pass 1), T = 60,000, E = 160 10.3 against 12.1; T = 65,536, E = 64
 // (3,400) 7.5 against 6.8.  Pass 2 counts few elements and takes one copy.
-HistCut cut_hist(int64_t T, int E, int pass, int sm_count) {
+HistCut cut_hist(int64_t T, int E, int pass, int blocks) {
   const int nch = E >> 3;
-  const int64_t per_sm = T * nch / sm_count;  // chunks of z to count per SM
+  const int64_t per_sm = T * nch / blocks;  // chunks of z to count per SM
   const int want = per_sm < 10000 ? 8 : 16;
   HistCut h;
   h.tiles = (nch + want - 1) / want;
   h.chunks = (nch + h.tiles - 1) / h.tiles;
   h.tiles = (nch + h.chunks - 1) / h.chunks;
   h.copies = pass != 2 && per_sm >= 7000 ? 32 / h.chunks : 1;
-  int64_t ranges = sm_count / h.tiles;
+  int64_t ranges = blocks / h.tiles;
   const int64_t most = (T * h.chunks + 1023) / 1024;  // a chunk for every thread
   if (ranges > most) ranges = most;
   if (ranges < 1) ranges = 1;
@@ -326,31 +372,46 @@ HistCut cut_hist(int64_t T, int E, int pass, int sm_count) {
   return h;
 }
 
+// One block's rows of the coefficient table take about 2 us and 1 us for each
+// further one; a short pass gives it up to 16 SMs, a long one four.
+int coef_blocks(int64_t T, int E, int M, int sm_count) {
+  const int most = T * (E >> 3) / sm_count < 10000 ? 16 : 4;
+  return M < most ? M : most;
+}
+
 template <int PASS, bool LEI>
-int launch_hist_pass(const HistArgs& a, const LeiStream& ls, cudaStream_t s) {
+int launch_hist_pass(const HistArgs& a, const LeiStream& ls, CoefRows cr, cudaStream_t s) {
   DeviceInfo di;
   if (int rc = device_info(&di)) return rc;
-  const HistCut h = cut_hist(a.T, a.E, PASS, di.sm_count);
+  cr.blocks = cr.coef ? coef_blocks(a.T, a.E, cr.a.M, di.sm_count) : 0;
+  const HistCut h = cut_hist(a.T, a.E, PASS, di.sm_count - cr.blocks);
   const int smem = bin_words(h.chunks * h.copies) * 4;
   auto kern = hist_kernel<PASS, LEI>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
     return kErrCuda;
-  dim3 grid((unsigned)h.tiles, (unsigned)h.ranges);
-  return launch_dependent(kern, grid, dim3(1024), smem, s, a, h.chunks, h.copies, h.tpc, ls) == cudaSuccess ? kOk
-                                                                                                      : kErrCuda;
+  return launch_dependent(kern, dim3((unsigned)(h.tiles * h.ranges + cr.blocks)), dim3(1024), smem, s, a, h.tiles,
+                          h.chunks, h.copies, h.tpc, ls, cr) == cudaSuccess
+             ? kOk
+             : kErrCuda;
 }
 
 }  // namespace
 
 int launch_hist(const HistArgs& a, int pass, cudaStream_t s) {
   const LeiStream none;
-  if (pass == 3) return launch_hist_pass<3, false>(a, none, s);
-  return pass == 1 ? launch_hist_pass<1, false>(a, none, s) : launch_hist_pass<2, false>(a, none, s);
+  if (pass == 3) return launch_hist_pass<3, false>(a, none, CoefRows(), s);
+  return pass == 1 ? launch_hist_pass<1, false>(a, none, CoefRows(), s)
+                   : launch_hist_pass<2, false>(a, none, CoefRows(), s);
+}
+
+int launch_hist_coef(const HistArgs& a, const LeiArgs& la, float* coef, cudaStream_t s) {
+  if (la.M < 1 || !coef) return kErrInvalidArg;
+  return launch_hist_pass<1, false>(a, LeiStream(), CoefRows{la, coef, 0}, s);
 }
 
 int launch_hist_lei(const HistArgs& a, int pass, const LeiStream& ls, cudaStream_t s) {
   if (!ls.g || !ls.coef || !ls.off || ls.M < 1 || ls.t0 < 0 || ls.t1 < ls.t0) return kErrInvalidArg;
-  return pass == 1 ? launch_hist_pass<1, true>(a, ls, s) : launch_hist_pass<2, true>(a, ls, s);
+  return pass == 1 ? launch_hist_pass<1, true>(a, ls, CoefRows(), s) : launch_hist_pass<2, true>(a, ls, CoefRows(), s);
 }
 
 }  // namespace eqb

@@ -14,9 +14,10 @@
 // 16-byte loads and stores using evict-first cache hints.
 //
 // For the one-call step the coefficients are also formed once per microbatch
-// into an [M,E] table (lei_coef_kernel), from which the histogram passes
-// stream the injection beside their own work (hist.cu).
-#include "eqb_device.cuh"
+// into an [M,E] table (lei_coef_kernel, or blocks of the coarse histogram
+// pass), from which the fine pass streams the injection beside its own work
+// (hist.cu).
+#include "lei_device.cuh"
 
 namespace eqb {
 
@@ -24,57 +25,6 @@ namespace {
 
 constexpr int kLeiThreads = 256;
 constexpr int kLeiUnroll = 4;
-
-// Eq. (norm) coefficients eta * sigma * rho_e of one microbatch with n tokens
-// and loads f (one row of [M,E]), computed by a whole block of kLeiThreads
-// threads into out[0..E) (shared or global memory) and visible to the block
-// on return.  fp64 throughput is low on this part, so each thread does only
-// a multiply-add and a multiply per expert; the reciprocal of the target
-// load and tanh are formed once.
-__device__ void block_lei_coef(const int32_t* __restrict__ f, int64_t n, int E, int K, float eta, float c,
-                               float* out) {
-  __shared__ double red[kLeiThreads / 32];
-  __shared__ double scal[2];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  __syncthreads();  // a previous call has finished reading scal and out
-  if (threadIdx.x == 0) scal[0] = n > 0 ? (double)E / ((double)K * (double)n) : 0.0;  // 1 / fbar
-  __syncthreads();
-  const double inv_fbar = scal[0];
-  // each thread holds the rho of experts threadIdx.x + k * kLeiThreads
-  constexpr int kPer = kMaxE / kLeiThreads;
-  double rho[kPer];
-  double amax = 0.0;
-#pragma unroll
-  for (int k = 0; k < kPer; ++k) {
-    const int e = threadIdx.x + k * kLeiThreads;
-    rho[k] = (e < E && inv_fbar > 0.0) ? (double)__ldg(f + e) * inv_fbar - 1.0 : 0.0;
-    amax = fmax(amax, fabs(rho[k]));
-  }
-#pragma unroll
-  for (int d = 16; d > 0; d >>= 1) amax = fmax(amax, __shfl_xor_sync(kFull, amax, d));
-  if (lane == 0) red[wid] = amax;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double rmax = red[0];
-    for (int w = 1; w < kLeiThreads / 32; ++w) rmax = fmax(rmax, red[w]);
-    // sigma = tanh(xi) / xi in fp32: its relative error (a few ulp of fp32)
-    // stays far inside the LEI tolerance, and it spares the serial fp64
-    // division and tanh of this thread
-    float sigma = 1.0f;
-    if (c > 0.0f) {
-      const float xi = __fdiv_rn(static_cast<float>(rmax), c);
-      sigma = (xi == 0.0f) ? 1.0f : __fdiv_rn(tanhf(xi), xi);
-    }
-    scal[1] = (double)eta * (double)sigma;
-  }
-  __syncthreads();
-#pragma unroll
-  for (int k = 0; k < kPer; ++k) {
-    const int e = threadIdx.x + k * kLeiThreads;
-    if (e < E) out[e] = __double2float_rn(scal[1] * rho[k]);
-  }
-  __syncthreads();
-}
 
 __global__ void __launch_bounds__(kLeiThreads) lei_kernel(LeiArgs a, int64_t tokens_per_cta) {
   __shared__ __align__(16) float coef[kMaxE];
@@ -93,7 +43,7 @@ __global__ void __launch_bounds__(kLeiThreads) lei_kernel(LeiArgs a, int64_t tok
     // Malformed offsets (off[M] < T) must not stall the loop: tokens past
     // the last boundary are treated as the last microbatch's.
     const int64_t seg_end = (hi > t) ? min(te, hi) : te;
-    block_lei_coef(a.loads + (int64_t)l * E, hi - lo, E, a.K, a.eta, a.c, coef);
+    block_lei_coef<kLeiThreads>(a.loads + (int64_t)l * E, hi - lo, E, a.K, a.eta, a.c, coef);
 
     // ---- stream grad_s[t .. seg_end) in float4 units
     const int64_t i0 = t * E4, i1 = seg_end * E4;
@@ -142,7 +92,7 @@ __global__ void __launch_bounds__(kLeiThreads) lei_coef_kernel(LeiArgs a, float*
   griddep_launch();
   const int l = blockIdx.x;
   const int64_t n = __ldg(a.off + l + 1) - __ldg(a.off + l);
-  block_lei_coef(a.loads + (int64_t)l * a.E, n, a.E, a.K, a.eta, a.c, coef + (int64_t)l * a.E);
+  block_lei_coef<kLeiThreads>(a.loads + (int64_t)l * a.E, n, a.E, a.K, a.eta, a.c, coef + (int64_t)l * a.E);
 }
 
 }  // namespace

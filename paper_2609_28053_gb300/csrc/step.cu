@@ -5,9 +5,8 @@
 // pass, selection, fine pass, selection and the Eq. (2) bias update, and
 // Load-Error Injection (Sec. 4, Eqs. LEI and norm).  LEI needs only the
 // loads, so when its [M,E] coefficient table fits the workspace the
-// coefficients are formed right after routing and the two histogram passes
-// stream the injection, half of the tokens each; otherwise it runs last.
-// All on one stream.
+// coefficients are formed before or beside the coarse pass and the passes
+// stream the injection; otherwise it runs last.  All on one stream.
 // eqb_router_layer_step starts one step earlier, at the router projection
 // (Eq. 1), and routes from the projection's accumulators where it can; that
 // kernel also counts the coarse histogram, so the fine pass alone reads z
@@ -16,9 +15,38 @@
 #include <stdint.h>
 
 #include "eqb.h"
-#include "eqb_internal.h"
+#include "eqb_device.cuh"
 
 namespace eqb {
+
+namespace {
+
+// 16-byte words [0, n16) of the workspace's histograms and counters, then the
+// loads.  The successor may launch at once: it waits for this grid to
+// complete before it touches global memory.
+__global__ void __launch_bounds__(256) clear_kernel(uint4* w, int n16, int32_t* loads, int64_t n) {
+  griddep_wait();
+  griddep_launch();
+  const int stride = gridDim.x * blockDim.x, i0 = blockIdx.x * blockDim.x + threadIdx.x;
+  for (int i = i0; i < n16; i += stride) w[i] = make_uint4(0u, 0u, 0u, 0u);
+  for (int64_t i = i0; i < n; i += stride) loads[i] = 0;
+}
+
+}  // namespace
+
+// H, L and the counters are adjacent in the workspace (H and L each E KiB, a
+// multiple of the 256-byte carve alignment).  One kernel for both arrays in
+// place of a memset each: a memset neither starts early nor lets its
+// successor start early.
+int launch_clear(const StepWorkspace& w, int E, int32_t* loads, int64_t n, cudaStream_t s) {
+  const int n16 = static_cast<int>((2 * carve_round(static_cast<size_t>(E) * 1024) + carve_round(kDoneBytes)) / 16);
+  const int64_t work = n16 > n ? n16 : n;
+  const int64_t grid = (work + 511) / 512;
+  return launch_dependent(clear_kernel, dim3((unsigned)(grid < 608 ? grid : 608)), dim3(256), 0, s,
+                          reinterpret_cast<uint4*>(w.H), n16, loads, n) == cudaSuccess
+             ? kOk
+             : kErrCuda;
+}
 
 size_t carve_workspace(void* base, int E, StepWorkspace* w) {
   size_t off = 0;
@@ -85,17 +113,6 @@ eqb_status check_step(const eqb_bf16* z, const float* b, int64_t T, int32_t E, i
   return EQB_OK;
 }
 
-eqb_status clear(const Workspace& w, int32_t* loads, int32_t E, int32_t M, cudaStream_t s) {
-  // H, L and the block counters are adjacent in the workspace (H and L each
-  // E*1 KiB, a multiple of the 256-byte carve alignment): one memset clears
-  // them.
-  if (cudaMemsetAsync(w.H, 0, 2 * eqb::carve_round(static_cast<size_t>(E) * 1024) + eqb::carve_round(eqb::kDoneBytes), s) !=
-          cudaSuccess ||
-      cudaMemsetAsync(loads, 0, static_cast<size_t>(M) * E * 4, s) != cudaSuccess)
-    return EQB_ERR_CUDA;
-  return EQB_OK;
-}
-
 // The two histogram passes of the step: pass 1 counts H; pass 2 selects u, rho
 // from H at rank r in every block, counts L, selects q_hat and forms b_next
 // (Eq. 2), so no selection is a launch of its own.
@@ -117,10 +134,13 @@ eqb::HistArgs pass2_args(const Workspace& w, const eqb_bf16* z, const float* tau
 
 // Everything after routing: Algorithm 1's two passes with their selections,
 // the Eq. (2) bias update and LEI.  When the [M,E] coefficient table fits the
-// workspace, the coefficients are formed once and each histogram pass
-// streams the injection of half of the tokens beside its counting (the
-// passes are issue-bound, the injection DRAM-bound); the results are the
-// same bits as the separate LEI launch.
+// workspace, the passes stream the injection beside their counting (they are
+// issue-bound, it is DRAM-bound); the results are the same bits as the
+// separate LEI launch.  Up to 2^26 logits blocks of the coarse pass form the
+// table and the fine pass carries all of the injection, which spares a launch
+// (T = 65,536, E = 64 49 -> 39 us, T = 147,456, E = 256 118 -> 115); beyond,
+// each pass carries half of it (T = 2,097,152, E = 256 1196 us against 1222,
+// T = 524,288, E = 256 332 against 332).
 eqb_status after_routing(const Workspace& w, const eqb_bf16* z, int64_t T, int32_t E, int32_t K,
                          const int64_t* mb_offsets, int32_t M, int64_t r, const float* tau,
                          const int32_t* loads, float* b_next, float* grad_s, float eta, float c,
@@ -129,11 +149,15 @@ eqb_status after_routing(const Workspace& w, const eqb_bf16* z, int64_t T, int32
   const eqb::HistArgs h2 = pass2_args(w, z, tau, T, E, r, b_next, err_flag);
   if (grad_s && static_cast<int64_t>(M) * E <= eqb::kLeiCoefCap) {
     eqb::LeiArgs la{grad_s, loads, mb_offsets, M, 0, T, E, K, eta, c};
-    if (int rc = eqb::launch_lei_coef(la, w.coef, s)) return st(rc);
-    const int64_t th = T / 2;
-    eqb::LeiStream l1{grad_s, w.coef, mb_offsets, M, 0, th};
+    const int64_t th = T * E <= int64_t(1) << 26 ? 0 : T / 2;  // tokens carried by pass 1
+    if (th == 0) {
+      if (int rc = eqb::launch_hist_coef(h1, la, w.coef, s)) return st(rc);
+    } else {
+      if (int rc = eqb::launch_lei_coef(la, w.coef, s)) return st(rc);
+      eqb::LeiStream l1{grad_s, w.coef, mb_offsets, M, 0, th};
+      if (int rc = eqb::launch_hist_lei(h1, 1, l1, s)) return st(rc);
+    }
     eqb::LeiStream l2{grad_s, w.coef, mb_offsets, M, th, T};
-    if (int rc = eqb::launch_hist_lei(h1, 1, l1, s)) return st(rc);
     if (int rc = eqb::launch_hist_lei(h2, 2, l2, s)) return st(rc);
     return EQB_OK;
   }
@@ -187,7 +211,7 @@ eqb_status eqb_layer_step(const eqb_bf16* z, const float* b, int64_t T, int32_t 
   if (rs != EQB_OK) return rs;
   if (r <= 0) r = eqb_target_rank(T, E, K);
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  if ((rs = clear(w, loads, E, M, s)) != EQB_OK) return rs;
+  if (int rc = eqb::launch_clear(w, E, loads, static_cast<int64_t>(M) * E, s)) return st(rc);
   eqb::RouteArgs ra{z, b, T, E, K, mb_offsets, M, 0, topk_idx, tau, loads, err_flag};
   if (int rc = eqb::launch_route(ra, s)) return st(rc);
   return after_routing(w, z, T, E, K, mb_offsets, M, r, tau, loads, b_next, grad_s, eta, c, err_flag, s);
@@ -208,7 +232,7 @@ eqb_status eqb_router_layer_step(const eqb_bf16* x, const eqb_bf16* W_r, int64_t
   if (rs != EQB_OK) return rs;
   if (r <= 0) r = eqb_target_rank(T, E, K);
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  if ((rs = clear(w, loads, E, M, s)) != EQB_OK) return rs;
+  if (int rc = eqb::launch_clear(w, E, loads, static_cast<int64_t>(M) * E, s)) return st(rc);
   if ((E == 64 || E == 128) && K <= 8) {
     // projection, routing and the coarse histogram in one kernel
     if (int rc = eqb::launch_router_route(x, W_r, T, d, E, K, b, mb_offsets, M, z, topk_idx, tau, loads, w.H,
