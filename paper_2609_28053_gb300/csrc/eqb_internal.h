@@ -138,8 +138,12 @@ size_t carve_workspace(void* base, int E, StepWorkspace* w);
 int launch_clear(const StepWorkspace& w, int E, int32_t* loads, int64_t n, cudaStream_t s);
 
 int launch_route(const RouteArgs& a, cudaStream_t s);
-bool route_wide_supported(int E, int K);
+// The routing kernels of compile-time row widths (K + 1 <= 16): E <= 128 and
+// E <= 512.
+int launch_route_narrow(const RouteArgs& a, cudaStream_t s);
 int launch_route_wide(const RouteArgs& a, cudaStream_t s);
+// One warp per token (any E, K + 1 <= 32).
+int launch_route_warp(const RouteArgs& a, cudaStream_t s);
 // Routing and the coarse histogram (hist, [E,256] +=) in one pass over z
 // (route_hist.cu; E = 128 or 256, K + 1 <= 16).
 bool route_hist_supported(int E, int K);

@@ -1,5 +1,6 @@
 // route.cu -- top-K routing, cutoff tau_t and per-microbatch loads
-// (Sec. 2, Eq. 1 and the QB paragraph of arXiv 2609.28053).
+// (Sec. 2, Eq. 1 and the QB paragraph of arXiv 2609.28053): the choice of the
+// routing kernel, and the kernel of runtime row width for 17 <= K + 1 <= 32.
 //
 // One thread owns one token.  A warp stages a tile of 32 consecutive token
 // rows of z (one contiguous block of 32 * E bf16) in shared memory with
@@ -46,7 +47,8 @@ __host__ __device__ inline int warp_region_bytes(int E, int nbuf) {
   return align16(nbuf * 32 * row_stride_bytes(E) + (E / 8) * 32 * 2 + 4 * E);  // tile, chunk lists, loads
 }
 
-template <int KP1, int G>
+constexpr int KP1 = 32, G = 32;  // list length, groups of the bound
+
 __global__ void __launch_bounds__(512) route_kernel(RouteArgs a, int64_t tiles_per_warp, int nbuf) {
   extern __shared__ __align__(16) uint8_t smem[];
   const int E = a.E, K = a.K;
@@ -294,9 +296,7 @@ __global__ void __launch_bounds__(512) route_kernel(RouteArgs a, int64_t tiles_p
   if (a.loads) flush_loads();
 }
 
-template <int KP1>
-int launch_route_kp1(const RouteArgs& a, cudaStream_t s) {
-  constexpr int G = KP1 <= 16 ? 16 : 32;
+int launch_route_many(const RouteArgs& a, cudaStream_t s) {
   DeviceInfo di;
   if (int rc = device_info(&di)) return rc;
   const int head = head_bytes(a.E);
@@ -317,7 +317,7 @@ int launch_route_kp1(const RouteArgs& a, cudaStream_t s) {
   if (grid > max_grid) grid = max_grid;
   const int64_t total_warps = grid * nw;
   const int64_t tpw = (ntiles + total_warps - 1) / total_warps;
-  auto kern = route_kernel<KP1, G>;
+  auto kern = route_kernel;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
     return kErrCuda;
   return launch_dependent(kern, dim3((unsigned)grid), dim3(nw * 32), smem, s, a, tpw, nbuf) == cudaSuccess
@@ -327,18 +327,18 @@ int launch_route_kp1(const RouteArgs& a, cudaStream_t s) {
 
 }  // namespace
 
+// A warp per token up to 32 E tokens, where tiles leave SMs idle and a tile's
+// serial work is the call's time (T = 4,096: E = 128 4.3 us against 4.5, 256
+// 4.1 against 6.9, 512 5.0 against 10.4; above, tiles: T = 16,411, E = 256 5.9
+// against 9.8, T = 30,000, E = 512 15 against 21; below E = 128 tiles take
+// under 4 us), and for rows too wide for a tile with enough warps beside it
+// (T = 300,000, E = 1024 248 us against 598).
 int launch_route(const RouteArgs& a, cudaStream_t s) {
-  if (route_wide_supported(a.E, a.K)) return launch_route_wide(a, s);
   const int kp1 = a.K + 1;
-  if (kp1 <= 2) return launch_route_kp1<2>(a, s);
-  if (kp1 <= 3) return launch_route_kp1<3>(a, s);
-  if (kp1 <= 4) return launch_route_kp1<4>(a, s);
-  if (kp1 <= 7) return launch_route_kp1<7>(a, s);
-  if (kp1 <= 8) return launch_route_kp1<8>(a, s);
-  if (kp1 <= 9) return launch_route_kp1<9>(a, s);
-  if (kp1 <= 16) return launch_route_kp1<16>(a, s);
-  if (kp1 <= 32) return launch_route_kp1<32>(a, s);
-  return kErrUnsupported;
+  if (kp1 > 32) return kErrUnsupported;
+  if (a.E > 512 || (a.E >= 128 && a.E >= 8 * kp1 && a.T <= 32 * (int64_t)a.E)) return launch_route_warp(a, s);
+  if (kp1 > 16) return launch_route_many(a, s);
+  return a.E <= 128 ? launch_route_narrow(a, s) : launch_route_wide(a, s);
 }
 
 }  // namespace eqb

@@ -81,7 +81,7 @@ __global__ void __launch_bounds__(32 * NW, 1)
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   griddep_wait();
-  load_bias_tables<E>(a.b, bs, bdn, bup, a.err);
+  load_bias_tables<E>(a.b, E, bs, bdn, bup, a.err);
   __syncthreads();
 
   const uint4* bdn4 = reinterpret_cast<const uint4*>(bdn);

@@ -1,17 +1,19 @@
 // route_wide.cu -- top-K routing, cutoff tau_t and per-microbatch loads
-// (Sec. 2, Eq. 1 and the QB paragraph of arXiv 2609.28053) for the wide rows
-// E = 128, 256, 384 and 512 with K + 1 <= 16, the row width fixed at compile
-// time.
+// (Sec. 2, Eq. 1 and the QB paragraph of arXiv 2609.28053) for rows of 136 to
+// 512 experts with K + 1 <= 16, at a compile-time row width of 160, 192, 256,
+// 320, 384 or 512 experts (narrower rows padded with -inf).
 //
 // One thread owns one token; a warp owns a tile of 32 consecutive tokens,
 // which each lane brings into shared memory with one bulk copy of its row
 // (completion on a per-warp mbarrier) while the next tile is prefetched into
 // L2.  Rows are padded to a stride of 4 (mod 8) words so the 32 lanes reading
 // the same 16-byte chunk of their own rows hit distinct banks.  The per-token
-// work (bound from packed chunk maxima, candidate masks, exact insertion of
-// the candidates) is route_row() in route_wide.cuh.
-// Loads are counted in per-warp shared counters for the warp's current
-// microbatch and flushed when it changes.
+// work (bound from packed group maxima, candidate masks, exact insertion of
+// the candidates) is route_row() in route_wide.cuh.  It is bound by the ALU
+// pipe and by the latency of its dependent instructions (12 warps an SM at
+// E = 256): T = 2,097,152, E = 256, K = 8 takes 211 us (169 at the copy
+// peak), T = 1,000,000, E = 264 152 us (219 with the runtime-width kernel it
+// replaced there), E = 160 91 (139).
 #include "route_wide.cuh"
 
 namespace eqb {
@@ -26,12 +28,14 @@ constexpr int wide_max_warps() {
              : 16;
 }
 
-template <int E, int KP1>
+// EXACT: the row has E experts, so that the copies' addresses and sizes are
+// constants too (T = 2,097,152, E = 256, K = 8 214 us, 224 without).
+template <int E, int KP1, bool EXACT>
 __global__ void __launch_bounds__(32 * wide_max_warps<E>(), 1)
     route_wide_kernel(RouteArgs a, int64_t tiles_per_warp) {
   using L = WideLayout<E>;
+  const int real = EXACT ? E : a.E;
   extern __shared__ __align__(16) uint8_t smem[];
-  const int K = a.K;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int nw = blockDim.x >> 5;
 
@@ -41,17 +45,18 @@ __global__ void __launch_bounds__(32 * wide_max_warps<E>(), 1)
   uint8_t* wreg = smem + L::HEAD + wid * L::WARP;
   uint8_t* tile = wreg;
   uint32_t* mw = reinterpret_cast<uint32_t*>(wreg + L::TILE);  // [NCH/4][32 lanes]
-  int* wl = reinterpret_cast<int*>(wreg + L::TILE + L::ENT);
+  TileLoads loads{reinterpret_cast<int*>(wreg + L::TILE + L::ENT)};
   const uint32_t bar = saddr(wreg + L::TILE + L::ENT + L::WL);
 
-  griddep_wait();
-  load_bias_tables<E>(a.b, bs, bdn, bup, a.err);
-  for (int e = lane; e < E; e += 32) wl[e] = 0;
+  if (!EXACT) pad_rows<E>(tile, 32, L::RS, real, lane);
+  for (int e = lane; e < E; e += 32) loads.wl[e] = 0;
   if (lane == 0) {
     bar_init(bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
+  griddep_wait();
+  load_bias_tables<E>(a.b, real, bs, bdn, bup, a.err);
   __syncthreads();
 
   const int64_t ntiles = (a.T + 31) >> 5;
@@ -68,33 +73,19 @@ __global__ void __launch_bounds__(32 * wide_max_warps<E>(), 1)
   auto load_tile = [&](int64_t tl) {
     const int64_t t0 = tl << 5;
     const int rows = static_cast<int>(min((int64_t)32, a.T - t0));
-    if (lane == 0) bar_expect_tx(bar, static_cast<uint32_t>(rows * E * 2));
+    if (lane == 0) bar_expect_tx(bar, static_cast<uint32_t>(rows * real * 2));
     __syncwarp();
     if (lane < rows) {
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      bulk_copy(saddr(tile + lane * L::RS), a.z + (t0 + lane) * E, E * 2, bar);
+      bulk_copy(saddr(tile + lane * L::RS), a.z + (t0 + lane) * real, real * 2, bar);
     }
   };
   auto prefetch = [&](int64_t tl) {
     if (lane == 0 && tl < te) {
       const int64_t t0 = tl << 5;
-      const uint32_t bytes = static_cast<uint32_t>(min((int64_t)32, a.T - t0) * E * 2);
-      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.z + t0 * E), "r"(bytes) : "memory");
+      const uint32_t bytes = static_cast<uint32_t>(min((int64_t)32, a.T - t0) * real * 2);
+      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.z + t0 * real), "r"(bytes) : "memory");
     }
-  };
-
-  int cur_mb = -1;
-  int64_t mb_lo = 0, mb_hi = 0;  // token range of cur_mb
-  auto flush_loads = [&]() {
-    __syncwarp();
-    if (cur_mb >= 0) {
-      for (int e = lane; e < E; e += 32) {
-        const int v = wl[e];
-        if (v) atomicAdd(a.loads + (int64_t)cur_mb * E + e, v);
-        wl[e] = 0;
-      }
-    }
-    __syncwarp();
   };
 
   uint32_t phase = 0;
@@ -122,100 +113,68 @@ __global__ void __launch_bounds__(32 * wide_max_warps<E>(), 1)
       load_tile(tl + 1);
       prefetch(tl + 2);
     }
-
-    // ---- outputs
-    if (valid) {
-      const float tau_t = list_tau<KP1>(v, K);
-      a.tau[t] = tau_t;
-      if (!isfinite(tau_t)) raise_flag(a.err, kErrNonfinite);
-      if (a.idx) {
-        int32_t* out = a.idx + t * K;
-#pragma unroll
-        for (int j = 0; j < KP1; ++j)
-          if (j < K) out[j] = id[j];
-      }
-    }
-    if (a.loads) {
-      const int64_t t0 = tl << 5;
-      const int64_t t_last = min(t0 + 31, a.T - 1) + a.tbase;
-      if (!(t0 + a.tbase >= mb_lo && t_last < mb_hi)) {
-        // the tile leaves the current microbatch: per-lane lookup
-        const int l = valid ? microbatch_of(a.off, a.M, t + a.tbase) : -1;
-        const int l0 = __shfl_sync(kFull, l, 0);
-        if (l0 != cur_mb) {
-          flush_loads();
-          cur_mb = l0;
-          mb_lo = __ldg(a.off + l0);
-          mb_hi = __ldg(a.off + l0 + 1);
-        }
-        if (valid) {
-#pragma unroll
-          for (int j = 0; j < KP1; ++j) {
-            if (j < K) {
-              if (l == cur_mb) atomicAdd(wl + id[j], 1);
-              else atomicAdd(a.loads + (int64_t)l * E + id[j], 1);
-            }
-          }
-        }
-      } else if (valid) {
-#pragma unroll
-        for (int j = 0; j < KP1; ++j)
-          if (j < K) atomicAdd(wl + id[j], 1);
-      }
-    }
+    if (valid) store_route<KP1>(a, t, v, id);
+    if (a.loads) loads.count<KP1>(a, tl << 5, valid, id, lane);
   }
-  if (a.loads) flush_loads();
+  if (a.loads) loads.flush(a, lane);
 }
 
-template <int E, int KP1>
+template <int E, int KP1, bool EXACT>
 int launch_wide_t(const RouteArgs& a, cudaStream_t s) {
   using L = WideLayout<E>;
   DeviceInfo di;
   if (int rc = device_info(&di)) return rc;
-  int nw = (di.max_smem_optin - L::HEAD) / L::WARP;
-  if (nw > wide_max_warps<E>()) nw = wide_max_warps<E>();
-  if (nw < 1) return kErrUnsupported;
-  const int smem = L::HEAD + nw * L::WARP;
-  int ctas_per_sm = (228 * 1024 - 1024) / (smem + 1024);
-  if (ctas_per_sm < 1) ctas_per_sm = 1;
-  if (ctas_per_sm > 4) ctas_per_sm = 4;
+  constexpr int nw_max = wide_max_warps<E>();
   const int64_t ntiles = (a.T + 31) / 32;
-  int64_t grid = (int64_t)di.sm_count * ctas_per_sm;
+  // few tiles: as few warps a block as leave none idle, over all SMs
+  int64_t nw = (ntiles + di.sm_count - 1) / di.sm_count;
+  if (nw > nw_max) nw = nw_max;
+  const int smem = L::HEAD + static_cast<int>(nw) * L::WARP;
+  if (smem > di.max_smem_optin) return kErrUnsupported;
+  int64_t grid = di.sm_count;
   const int64_t max_grid = (ntiles + nw - 1) / nw;
   if (grid > max_grid) grid = max_grid;
-  const int64_t total_warps = grid * nw;
-  const int64_t tpw = (ntiles + total_warps - 1) / total_warps;
-  auto kern = route_wide_kernel<E, KP1>;
+  const int64_t tpw = (ntiles + grid * nw - 1) / (grid * nw);
+  auto kern = route_wide_kernel<E, KP1, EXACT>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
     return kErrCuda;
-  return launch_dependent(kern, dim3((unsigned)grid), dim3(nw * 32), smem, s, a, tpw) == cudaSuccess ? kOk
-                                                                                         : kErrCuda;
+  return launch_dependent(kern, dim3((unsigned)grid), dim3((unsigned)nw * 32), smem, s, a, tpw) == cudaSuccess
+             ? kOk
+             : kErrCuda;
 }
 
 template <int E>
 int launch_wide_e(const RouteArgs& a, cudaStream_t s) {
   const int kp1 = a.K + 1;
-  if (kp1 <= 2) return launch_wide_t<E, 2>(a, s);
-  if (kp1 <= 3) return launch_wide_t<E, 3>(a, s);
-  if (kp1 <= 4) return launch_wide_t<E, 4>(a, s);
-  if (kp1 <= 7) return launch_wide_t<E, 7>(a, s);
-  if (kp1 <= 8) return launch_wide_t<E, 8>(a, s);
-  if (kp1 <= 9) return launch_wide_t<E, 9>(a, s);
-  if (kp1 <= 16) return launch_wide_t<E, 16>(a, s);
-  return kErrUnsupported;
+  if (kp1 <= 3) return launch_wide_t<E, 3, true>(a, s);
+  if (kp1 <= 5) return launch_wide_t<E, 5, true>(a, s);
+  if (kp1 <= 7) return launch_wide_t<E, 7, true>(a, s);
+  if (kp1 <= 9) return launch_wide_t<E, 9, true>(a, s);
+  return launch_wide_t<E, 16, true>(a, s);
+}
+
+// A row of fewer than E experts.
+template <int E>
+int launch_wide_padded(const RouteArgs& a, cudaStream_t s) {
+  const int kp1 = a.K + 1;
+  if (kp1 <= 5) return launch_wide_t<E, 5, false>(a, s);
+  if (kp1 <= 9) return launch_wide_t<E, 9, false>(a, s);
+  return launch_wide_t<E, 16, false>(a, s);
 }
 
 }  // namespace
 
-bool route_wide_supported(int E, int K) {
-  return (E == 128 || E == 256 || E == 384 || E == 512) && K + 1 <= 16;
-}
-
 int launch_route_wide(const RouteArgs& a, cudaStream_t s) {
+  if (a.K + 1 > 16) return kErrUnsupported;
   if (a.E == 256) return launch_wide_e<256>(a, s);
-  if (a.E == 128) return launch_wide_e<128>(a, s);
-  if (a.E == 512) return launch_wide_e<512>(a, s);
   if (a.E == 384) return launch_wide_e<384>(a, s);
+  if (a.E == 512) return launch_wide_e<512>(a, s);
+  if (a.E <= 160) return launch_wide_padded<160>(a, s);
+  if (a.E <= 192) return launch_wide_padded<192>(a, s);
+  if (a.E <= 256) return launch_wide_padded<256>(a, s);
+  if (a.E <= 320) return launch_wide_padded<320>(a, s);
+  if (a.E <= 384) return launch_wide_padded<384>(a, s);
+  if (a.E <= 512) return launch_wide_padded<512>(a, s);
   return kErrUnsupported;
 }
 

@@ -1,22 +1,27 @@
-// route_wide.cuh -- the per-token part of wide-row routing (Sec. 2, Eq. 1
-// and the QB paragraph of arXiv 2609.28053), shared by the routing kernel
-// (route_wide.cu) and the routing + coarse-histogram kernel (route_hist.cu).
+// route_wide.cuh -- the per-token part of routing by tiles (Sec. 2, Eq. 1
+// and the QB paragraph of arXiv 2609.28053), shared by the routing kernels
+// (route_wide.cu, route_narrow.cu) and the routing + coarse-histogram kernel
+// (route_hist.cu).
 //
 // One thread owns one token whose row of z sits in shared memory (rows of a
-// 32-token tile padded to a stride of 4 (mod 8) words, so the 32 lanes
-// reading the same 16-byte chunk of their own rows hit distinct banks).  The
-// row width E is a compile-time constant, so every loop over the row unrolls:
-//   A. packed bf16x2 maxima of L_e = bf16(z_e + RD(b_e)) per 8-expert chunk,
-//      the chunks c and c + NCH/2 sharing one word.  Sorting the words
-//      (bf16x2 max/min network) sorts both half-rows' chunk maxima at once,
-//      and the KP1-th largest of all chunk maxima is
-//      min_{i<KP1} max(A[i], B[KP1-1-i]) for the two sorted lists A, B.
-//      KP1 >= K+1 chunks each hold an element with L at or above it, so one
-//      bf16 step below it is <= tau_t and bounds every expert that can be
-//      selected; two steps below it is the filter threshold.
-//   B. per-chunk masks of U_e = bf16(z_e + RU(b_e)) >= threshold, every one
-//      of the experts with s_e >= tau_t among them, kept in shared memory,
-//      with the set of non-zero mask words (32 experts each).
+// 32-token tile padded to a stride of 4 (mod 8) words, so the 32 lanes reading
+// the same 16-byte chunk of their own rows hit distinct banks).  The row
+// width E is a compile-time multiple of 32, so every loop over the row
+// unrolls; a narrower row is padded to it with z = -inf, which is never
+// selected:
+//   A. packed bf16x2 maxima of L_e = bf16(z_e + RD(b_e)) over the row's words
+//      congruent mod 16: 32 groups, 16 of even and 16 of odd experts.  One
+//      bf16x2 max/min network sorts both halves at once, and the KP1-th
+//      largest group maximum is min_{i<KP1} max(A[i], B[KP1-1-i]) for the two
+//      sorted lists A, B.  KP1 >= K+1 groups each hold an element with L at
+//      or above it, so one bf16 step below it is <= tau_t and bounds every
+//      expert that can be selected; two steps below it is the filter
+//      threshold.  (Groups of E/32 experts leave 9.7, 10.1, 10.3 and 10.5
+//      candidates of 64, 128, 256 and 512 for K + 1 = 9; more groups cost
+//      more in the network than the fewer candidates save.)
+//   B. masks of U_e = bf16(z_e + RU(b_e)) >= threshold, 32 experts to a word,
+//      every one of the experts with s_e >= tau_t among them, with the set of
+//      non-zero words.
 //   C. the listed experts, in ascending index, are inserted into a sorted
 //      (K+1)-list by their exact fp32 score s_e = fp32(z_e) + b_e; a new
 //      element goes after equal scores, so ties keep the lower index first.
@@ -40,12 +45,6 @@ __device__ __forceinline__ uint32_t lds_u16(const void* p) {
   return *reinterpret_cast<const uint16_t*>(p);
 }
 
-// (max of the even experts, max of the odd experts) of one chunk of L.
-__device__ __forceinline__ uint32_t chunk_max(const uint4& w, const uint4& bd) {
-  return hmax2_nan_bf16(hmax2_nan_bf16(hadd2_bf16(w.x, bd.x), hadd2_bf16(w.y, bd.y)),
-                        hmax2_nan_bf16(hadd2_bf16(w.z, bd.z), hadd2_bf16(w.w, bd.w)));
-}
-
 __host__ __device__ constexpr int wide_row_stride(int E) { return 4 * (E / 2 + ((4 - E / 2) & 7)); }
 
 template <int E>
@@ -59,21 +58,29 @@ struct WideLayout {
   static constexpr int HEAD = 4 * E + 2 * (2 * E);               // b, RD(b), RU(b)
 };
 
-// The block's copy of the bias: b as fp32, and RD(b), RU(b) as packed bf16
+// The block's copy of the bias (0 for the experts [real, E) of a padded row):
+// b as fp32, and RD(b), RU(b) as packed bf16
 // pairs (the bounds of phases A and B).  A non-finite b raises the flag.
 template <int E>
-__device__ __forceinline__ void load_bias_tables(const float* __restrict__ b, float* bs, uint32_t* bdn, uint32_t* bup,
-                                                 int32_t* err) {
+__device__ __forceinline__ void load_bias_tables(const float* __restrict__ b, int real, float* bs, uint32_t* bdn,
+                                                 uint32_t* bup, int32_t* err) {
   for (int e = threadIdx.x; e < E; e += blockDim.x) {
-    const float v = b[e];
+    const float v = e < real ? b[e] : 0.f;
     bs[e] = v;
     if (!isfinite(v)) raise_flag(err, kErrNonfinite);
   }
   for (int q = threadIdx.x; q < E / 2; q += blockDim.x) {
-    const float b0 = b[2 * q], b1 = b[2 * q + 1];
+    const float b0 = 2 * q < real ? b[2 * q] : 0.f, b1 = 2 * q < real ? b[2 * q + 1] : 0.f;
     bdn[q] = bf16_round_down(b0) | (bf16_round_down(b1) << 16);
     bup[q] = bf16_round_up(b0) | (bf16_round_up(b1) << 16);
   }
+}
+
+// x >> n, 0 for n >= 32.
+__device__ __forceinline__ uint32_t shr_clamp(uint32_t x, int n) {
+  uint32_t r;
+  asm("shr.u32 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(n));
+  return r;
 }
 
 // Phases A-C for the token whose row starts at rowp: on return v[0..KP1)
@@ -85,35 +92,35 @@ template <int E, int KP1>
 __device__ __forceinline__ void route_row(const uint8_t* rowp, const float* bs, const uint4* bdn4, const uint4* bup4,
                                           uint32_t* mw, int lane, bool valid, int32_t* err, float (&v)[KP1],
                                           int (&id)[KP1]) {
-  constexpr int NCH = E / 8, NH = NCH / 2;
-  constexpr int NP = NH <= 8 ? 8 : NH <= 16 ? 16 : 32;  // sorted length (a power of two)
+  constexpr int NCH = E / 8;
 
-  // ---- A: chunk maxima of L, chunks c and c + NH in one word (words past
-  // NH, when NH is not a power of two, hold -inf in both halves)
-  uint32_t cm[NP];
+  // ---- A: maxima of L over the words congruent mod 16, both halves
+  uint32_t cm[16];
 #pragma unroll
-  for (int c = NH; c < NP; ++c) cm[c] = 0xff80ff80u;
-#pragma unroll
-  for (int c = 0; c < NH; ++c) {
+  for (int c = 0; c < NCH; ++c) {
     // From E = 256 on the unrolled loads do not fit in registers if all are
     // hoisted (at E = 256 the 168 registers of a 12-warp block spilled):
-    // let at most eight pairs of chunks be in flight.
-    if (NH > 8 && c > 0 && (c & 7) == 0) asm volatile("" ::: "memory");
-    const uint32_t qa = chunk_max(lds128(rowp + 16 * c), bdn4[c]);
-    const uint32_t qb = chunk_max(lds128(rowp + 16 * (c + NH)), bdn4[c + NH]);
-    cm[c] = hmax2_nan_bf16(prmt(qa, qb, 0x5410u), prmt(qa, qb, 0x7632u));
+    // let at most sixteen chunks be in flight.
+    if (NCH > 16 && c > 0 && (c & 15) == 0) asm volatile("" ::: "memory");
+    const uint4 w = lds128(rowp + 16 * c), bd = bdn4[c];
+    const uint32_t q[4] = {hadd2_bf16(w.x, bd.x), hadd2_bf16(w.y, bd.y), hadd2_bf16(w.z, bd.z),
+                           hadd2_bf16(w.w, bd.w)};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int g = (c & 3) * 4 + i;
+      cm[g] = c < 4 ? q[i] : hmax2_nan_bf16(cm[g], q[i]);
+    }
   }
   uint32_t anynan = cm[0];
 #pragma unroll
-  for (int c = 1; c < NH; ++c) anynan = hmax2_nan_bf16(anynan, cm[c]);
+  for (int c = 1; c < 16; ++c) anynan = hmax2_nan_bf16(anynan, cm[c]);
   if (valid && ((anynan & 0x7fffu) > 0x7f80u || (anynan >> 16 & 0x7fffu) > 0x7f80u)) raise_flag(err, kErrNonfinite);
-  sort_desc_bf16x2<NP>(cm);
+  sort_desc_bf16x2<16>(cm);
   float theta = INFINITY;
 #pragma unroll
   for (int i = 0; i < KP1; ++i) {
     const int j = KP1 - 1 - i;
-    const float x = i < NP ? bf16_lo(cm[i < NP ? i : 0]) : -INFINITY;
-    const float y = j < NP ? bf16_hi(cm[j < NP ? j : 0]) : -INFINITY;
+    const float x = bf16_lo(cm[i]), y = bf16_hi(cm[j]);  // KP1 <= 16
     theta = fminf(theta, fmaxf(x, y));
   }
   // Near zero, flushing of subnormal bf16 sums could move L by up to
@@ -130,9 +137,12 @@ __device__ __forceinline__ void route_row(const uint8_t* rowp, const float* bs, 
   const uint32_t thf = bf16_steps_down(__float_as_uint(theta) >> 16, 2u);
   const uint32_t thf2 = thf | (thf << 16);
 
-  // ---- B: per-chunk masks of U >= threshold, stored four to a word (bit
-  // 8u + j of word k is expert 32k + 8u + j), and the set of non-zero words
+  // ---- B: per-chunk masks of U >= threshold, four to a word (bit 31 -
+  // 8u - j of word k is expert 32k + 8u + j: the first expert is the highest
+  // bit, one count of leading zeros away), and the set of non-zero words.
+  // Up to 64 experts the words stay in registers, else in shared memory.
   uint32_t hits = 0u;
+  uint32_t m = 0u, m1 = 0u;  // the current mask word; E <= 64: the words themselves
 #pragma unroll
   for (int k = 0; k < NCH / 4; ++k) {
     uint32_t word = 0u;
@@ -145,12 +155,17 @@ __device__ __forceinline__ void route_row(const uint8_t* rowp, const float* bs, 
       const uint32_t r1 = hge2_bf16(hadd2_bf16(w.y, bu.y), thf2);
       const uint32_t r2 = hge2_bf16(hadd2_bf16(w.z, bu.z), thf2);
       const uint32_t r3 = hge2_bf16(hadd2_bf16(w.w, bu.w), thf2);
-      // element 2q -> bit 2q (low half of r_q), element 2q+1 -> bit 16+2q
-      const uint32_t y = (r0 & 0x00010001u) | (r1 & 0x00040004u) | (r2 & 0x00100010u) | (r3 & 0x00400040u);
-      word |= ((y | (y >> 15)) & 0xffu) << (8 * u);
+      // element 2q -> bit 7 - 2q (low half of r_q), element 2q+1 -> bit 22 - 2q
+      const uint32_t y = (r0 & 0x00400080u) | (r1 & 0x00100020u) | (r2 & 0x00040008u) | (r3 & 0x00010002u);
+      word |= ((y | (y >> 16)) & 0xffu) << (24 - 8 * u);
     }
-    mw[(k << 5) | lane] = word;
-    hits |= (word != 0u ? 1u : 0u) << k;
+    if (E <= 64) {
+      if (k == 0) m = word;
+      else m1 = word;
+    } else {
+      mw[(k << 5) | lane] = word;
+      hits |= (word != 0u ? 0x80000000u : 0u) >> k;
+    }
   }
 
   // ---- C: exact top-(K+1) of the experts with a hit, in ascending index,
@@ -161,16 +176,28 @@ __device__ __forceinline__ void route_row(const uint8_t* rowp, const float* bs, 
 #pragma unroll
   for (int j = 0; j < KP1; ++j) { v[j] = -INFINITY; id[j] = 0; }
   int wb = 0;  // first expert of the current mask word
-  uint32_t m = 0u;
   auto fetch = [&]() -> int {
+    if constexpr (E <= 64) {
+      if constexpr (E > 32) {
+        const bool need = m == 0u;
+        m = need ? m1 : m;
+        wb = need ? 32 : wb;
+        m1 = need ? 0u : m1;
+      }
+      const int p = __clz(m);
+      const int e = m != 0u ? wb + p : -1;
+      m &= shr_clamp(0x7fffffffu, p);
+      return e;
+    }
     const bool need = m == 0u && hits != 0u;
-    const int k = __ffs(hits) - 1;
+    const int k = __clz(hits);  // 32 when there is none
     const uint32_t word = mw[((need ? k : 0) << 5) | lane];
     m = need ? word : m;
     wb = need ? k << 5 : wb;
-    hits = need ? hits & (hits - 1u) : hits;
-    const int e = m != 0u ? wb + __ffs(m) - 1 : -1;
-    m &= m - 1u;
+    hits = need ? hits ^ shr_clamp(0x80000000u, k) : hits;
+    const int p = __clz(m);
+    const int e = m != 0u ? wb + p : -1;
+    m &= shr_clamp(0x7fffffffu, p);  // experts before p are already gone
     return e;
   };
   int e0 = fetch();
@@ -194,6 +221,83 @@ __device__ __forceinline__ float list_tau(const float (&v)[KP1], int K) {
 #pragma unroll
   for (int j = 1; j < KP1; ++j) tau_t = (j == K) ? v[j] : tau_t;
   return tau_t;
+}
+
+// Per-warp load counters (E ints in shared memory) of the warp's current
+// microbatch, flushed when it changes; every warp owns a contiguous range of
+// tiles, so flushes are rare.  A tile inside the current microbatch skips the
+// lookup.
+struct TileLoads {
+  int* wl;
+  int cur = -1;
+  int64_t lo = 0, hi = 0;  // token range of cur
+
+  __device__ __forceinline__ void flush(const RouteArgs& a, int lane) {
+    __syncwarp();
+    if (cur >= 0) {
+      for (int e = lane; e < a.E; e += 32) {
+        const int v = wl[e];
+        if (v) atomicAdd(a.loads + (int64_t)cur * a.E + e, v);
+        wl[e] = 0;
+      }
+    }
+    __syncwarp();
+  }
+
+  // Counts the top-K experts id[0..K) of this lane's token t (if valid) of
+  // the tile starting at t0.  Called by all lanes.
+  template <int KP1>
+  __device__ __forceinline__ void count(const RouteArgs& a, int64_t t0, bool valid, const int (&id)[KP1], int lane) {
+    const int K = a.K;
+    const int64_t t_last = min(t0 + 31, a.T - 1) + a.tbase;
+    int l = cur;
+    if (!(t0 + a.tbase >= lo && t_last < hi)) {
+      // the tile leaves the current microbatch: per-lane lookup
+      l = valid ? microbatch_of(a.off, a.M, t0 + lane + a.tbase) : -1;
+      const int l0 = __shfl_sync(kFull, l, 0);
+      if (l0 != cur) {
+        flush(a, lane);
+        cur = l0;
+        lo = __ldg(a.off + l0);
+        hi = __ldg(a.off + l0 + 1);
+      }
+    }
+    if (!valid) return;
+    if (l == cur) {
+#pragma unroll
+      for (int j = 0; j < KP1; ++j)
+        if (j < K) atomicAdd(wl + id[j], 1);
+    } else {
+#pragma unroll
+      for (int j = 0; j < KP1; ++j)
+        if (j < K) atomicAdd(a.loads + (int64_t)l * a.E + id[j], 1);
+    }
+  }
+};
+
+// tau and the top-K list of token t.
+template <int KP1>
+__device__ __forceinline__ void store_route(const RouteArgs& a, int64_t t, const float (&v)[KP1],
+                                            const int (&id)[KP1]) {
+  const float tau_t = list_tau<KP1>(v, a.K);
+  a.tau[t] = tau_t;
+  if (!isfinite(tau_t)) raise_flag(a.err, kErrNonfinite);
+  if (a.idx) {
+    int32_t* out = a.idx + t * a.K;
+#pragma unroll
+    for (int j = 0; j < KP1; ++j)
+      if (j < a.K) out[j] = id[j];
+  }
+}
+
+// Columns [a.E, E) of `rows` staged rows set to -inf by a warp (copies of a
+// row never reach them).
+template <int E>
+__device__ __forceinline__ void pad_rows(uint8_t* rows, int n, int stride, int real, int lane) {
+  for (int c = real / 8; c < E / 8; ++c)
+    for (int r = lane; r < n; r += 32)
+      *reinterpret_cast<uint4*>(rows + r * stride + 16 * c) =
+          make_uint4(0xff80ff80u, 0xff80ff80u, 0xff80ff80u, 0xff80ff80u);
 }
 
 }  // namespace eqb

@@ -1,0 +1,91 @@
+"""GPU parity of routing at the edges of its kernels: row widths on both sides
+of every compile-time width, token counts on both sides of the line between a
+warp per token and tiles, list lengths on both sides of theirs, and rows with
+more candidates than a warp collects (all scores equal).  tau, indices and
+loads equal the oracle's bit for bit."""
+import numpy as np
+import pytest
+import torch
+
+import brute
+import oracle
+import paper_2609_28053_gb300 as eqb
+from eqb_workloads import ragged_offsets
+from gpu_harness import Guarded, bits_f32, to_dev_bf16
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib(cuda_ok):
+    eqb.load()
+
+
+def check(z, b, K, M, seed):
+    T, E = z.shape
+    off = ragged_offsets(T, M, seed=seed) if M > 1 else np.array([0, T], np.int64)
+    idx_ref, tau_ref, loads_ref = oracle.route(z, b, K, off)
+    idx, tau, loads = Guarded((T, K), torch.int32), Guarded((T,), torch.float32), Guarded((M, E), torch.int32)
+    err = torch.zeros(1, dtype=torch.int32, device="cuda")
+    eqb.eqb_route_topk(to_dev_bf16(z), torch.from_numpy(b).cuda(), K, torch.from_numpy(off).cuda(), idx.view,
+                       tau.view, loads.view, err_flag=err)
+    torch.cuda.synchronize()
+    assert idx.intact() and tau.intact() and loads.intact() and err.item() == 0
+    assert np.array_equal(idx.view.cpu().numpy(), idx_ref)
+    assert np.array_equal(bits_f32(tau.view.cpu().numpy()), bits_f32(tau_ref))
+    assert np.array_equal(loads.view.cpu().numpy(), loads_ref)
+
+
+WIDTHS = [8, 32, 40, 64, 72, 96, 104, 128, 136, 160, 168, 192, 200, 256, 264, 320, 328, 384, 392, 512, 520, 1024]
+
+
+@pytest.mark.parametrize("E", WIDTHS)
+@pytest.mark.parametrize("side", ["one", "warp", "tile"])
+def test_row_widths(E, side):
+    K = min(8, E // 4)
+    T = {"one": 1, "warp": 32 * E, "tile": 32 * E + 1}[side]
+    rng = np.random.default_rng(E)
+    z = brute.bf16_bits_from_f32(rng.standard_normal((T, E), dtype=np.float32))
+    check(z, (rng.standard_normal(E) * 0.3).astype(np.float32), K, 1 if T < 3 else 5, seed=E)
+
+
+@pytest.mark.parametrize("E", [8, 64, 256, 1024])
+@pytest.mark.parametrize("K", [1, 2, 3, 4, 5, 6, 7, 8, 15, 16, 31])
+def test_list_lengths(E, K):
+    if K >= E:
+        pytest.skip("K < E")
+    rng = np.random.default_rng(K)
+    for T in (70, 32 * E + 40):
+        z = brute.bf16_bits_from_f32(rng.standard_normal((T, E), dtype=np.float32))
+        check(z, (rng.standard_normal(E) * 0.3).astype(np.float32), K, 3, seed=K)
+
+
+@pytest.mark.parametrize("E,K", [(24, 4), (72, 8), (128, 8), (264, 12), (512, 8), (1024, 15)])
+@pytest.mark.parametrize("kind", ["constant", "two values", "zeros"])
+def test_equal_scores(E, K, kind):
+    rng = np.random.default_rng(E)
+    for T in (9, 32 * E + 3):
+        z = np.full((T, E), 1.5, np.float32)
+        if kind == "two values":
+            z = np.where(rng.random((T, E)) < 0.5, np.float32(0.25), np.float32(-0.75))
+        if kind == "zeros":  # -0 and +0 are equal scores
+            z = np.where(rng.random((T, E)) < 0.5, np.float32(0.0), np.float32(-0.0))
+        b = np.where(np.arange(E) % 3 == 0, np.float32(-0.0), np.float32(0.0)).astype(np.float32)
+        check(brute.bf16_bits_from_f32(z), b, K, 2, seed=E)
+
+
+def test_microbatches_of_a_warp():
+    """More boundaries than a warp loads at once, most of them equal, and
+    enough tokens of a wide row for the loads to be counted by segments."""
+    E, K = 520, 4
+    for T, M in ((700, 200), (130000, 90)):
+        rng = np.random.default_rng(M)
+        z = brute.bf16_bits_from_f32(rng.standard_normal((T, E), dtype=np.float32))
+        b = (rng.standard_normal(E) * 0.3).astype(np.float32)
+        off = np.sort(np.concatenate([[0] * 40, rng.integers(0, T, M - 79), [T] * 40])).astype(np.int64)
+        _, _, ref = oracle.route(z, b, K, off)
+        loads = torch.zeros((len(off) - 1, E), dtype=torch.int32, device="cuda")
+        eqb.eqb_route_topk(to_dev_bf16(z), torch.from_numpy(b).cuda(), K, torch.from_numpy(off).cuda(), None, None,
+                           loads)
+        torch.cuda.synchronize()
+        assert np.array_equal(loads.cpu().numpy(), ref)
