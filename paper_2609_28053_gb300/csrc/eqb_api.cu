@@ -210,7 +210,7 @@ eqb_status eqb_router_logits(const eqb_bf16* x, const eqb_bf16* W_r, int64_t T, 
   if (!aligned(x, 16) || !aligned(W_r, 16) || !aligned(z, 16) || !aligned(err_flag, 4))
     return EQB_ERR_INVALID_ARG;
   if (T == 0) return EQB_OK;
-  return to_status(eqb::launch_router_gemm(x, W_r, T, d, E, z, err_flag, as_stream(stream)));
+  return to_status(eqb::launch_router_gemm(x, W_r, T, d, E, z, err_flag, true, as_stream(stream)));
 }
 
 eqb_status eqb_router_route(const eqb_bf16* x, const eqb_bf16* W_r, int64_t T, int32_t d, int32_t E,
@@ -228,7 +228,7 @@ eqb_status eqb_router_route(const eqb_bf16* x, const eqb_bf16* W_r, int64_t T, i
     return EQB_ERR_INVALID_ARG;
   if (T == 0) return EQB_OK;
   return to_status(eqb::launch_router_route(x, W_r, T, d, E, K, b, mb_offsets, M, z, topk_idx, tau, loads,
-                                            hist_hi, err_flag, as_stream(stream)));
+                                            hist_hi, err_flag, true, as_stream(stream)));
 }
 
 eqb_status eqb_maxvio(const int32_t* loads, const int64_t* mb_offsets, int32_t M, int32_t E, int32_t K,

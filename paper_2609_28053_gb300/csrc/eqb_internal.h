@@ -166,17 +166,33 @@ int launch_lei(const LeiArgs& a, cudaStream_t s);
 // The [M,E] fp32 table of Eq. (norm) coefficients, row l for microbatch l
 // (bit-identical to the coefficients launch_lei forms).
 int launch_lei_coef(const LeiArgs& a, float* coef, cudaStream_t s);
+// z = bf16(x W^T).  With `split`, few tokens take the split kernel below.
 int launch_router_gemm(const uint16_t* x, const uint16_t* W, int64_t T, int d, int E, uint16_t* z,
-                       int32_t* err, cudaStream_t s);
+                       int32_t* err, bool split, cudaStream_t s);
+// Few tokens (router_split.cu): a cluster of n blocks shares each 128-token
+// tile, every block a part of the columns of x; router_splits says how many
+// pay (1: the persistent kernel).  With ro.b the tokens are routed too.
+struct SplitRoute {
+  const float* b = nullptr;
+  int K = 0;
+  const int64_t* off = nullptr;
+  int M = 0;
+  int32_t* idx = nullptr;
+  float* tau = nullptr;
+  int32_t* loads = nullptr;
+};
+int router_splits(int64_t T, int d, int sm_count);
+int launch_router_split(const uint16_t* x, const uint16_t* W, int64_t T, int d, int E, int n, uint16_t* z,
+                        const SplitRoute& ro, int32_t* err, cudaStream_t s);
 int launch_gshard(const GshardArgs& a, cudaStream_t s);
 int launch_maxvio(const int32_t* loads, const int64_t* off, int M, int E, int K, double* out, double* per_mb,
                   cudaStream_t s);
 // The router projection routing each token from its accumulators (E = 64 or
 // 128, K <= 8); with hist (nullable) also the coarse histogram ([E,256] +=),
 // counted in the epilogue when no block routes more than 65,535 tokens, else
-// by the coarse pass over z after it.
+// by the coarse pass over z after it.  `split` as for launch_router_gemm.
 int launch_router_route(const uint16_t* x, const uint16_t* W, int64_t T, int d, int E, int K, const float* b,
                         const int64_t* off, int M, uint16_t* z, int32_t* idx, float* tau, int32_t* loads,
-                        int32_t* hist, int32_t* err, cudaStream_t s);
+                        int32_t* hist, int32_t* err, bool split, cudaStream_t s);
 
 }  // namespace eqb

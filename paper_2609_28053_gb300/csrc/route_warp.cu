@@ -4,17 +4,11 @@
 // a tile's serial work is what a call takes, and for rows too wide for tiles
 // in shared memory.
 //
-// Lane j holds the 16-byte chunks j, j + 32, ... of the row (read straight
-// into registers, the next token's while this one is routed) and forms their
-// exact scores s_e = fp32(z_e) + b_e.  The (K+1)st largest of the 32 lane
-// maxima, found by K + 1 warp reductions (lanes with equal maxima leave
-// together, which only lowers it), is <= tau_t, so the scores >= it hold the
-// top K + 1; about K + 3 of them do.  They are collected in shared memory, one
-// per lane, each lane counts the ones that come before its own (higher score,
-// ties to the lower index), and the lane of rank r stores entry r.  More than
-// 32 of them (many equal scores, or fewer than K + 1 chunks) are selected one
-// by one over the whole row instead.
-#include "eqb_device.cuh"
+// Lanes read the row straight into registers, the next token's while this one
+// is routed, as in warp_route (route_warp.cuh).  The steps are written out
+// here: called as that function, the same steps compile to a schedule that
+// takes 12% longer (T = 300,000, E = 1024 277 us against 248).
+#include "route_warp.cuh"
 
 namespace eqb {
 
@@ -24,26 +18,6 @@ constexpr int kWarps = 8;  // per block
 // Blocks that an SM holds (47, 59 and 94 registers a thread).
 template <int CPL>
 constexpr int kResident = CPL == 1 ? 5 : CPL == 2 ? 4 : 2;
-
-// Order-preserving key of a score; -0 and +0 get the same key (they are equal
-// scores).
-__device__ __forceinline__ uint32_t score_key(float s) {
-  const uint32_t u = __float_as_uint(__fadd_rn(s, 0.0f));
-  return u ^ ((u & 0x80000000u) ? 0xffffffffu : 0x80000000u);
-}
-
-// Microbatch of token t, as microbatch_of, by a whole warp in one round of
-// loads for every 32 boundaries.
-__device__ __forceinline__ int warp_microbatch_of(const int64_t* __restrict__ off, int M, int64_t t, int lane) {
-  int l = 0;
-  for (int j0 = 0; j0 < M - 1; j0 += 32) {
-    const int j = j0 + lane;
-    const unsigned below = __ballot_sync(kFull, j < M - 1 && __ldg(off + j + 1) <= t);
-    l += __popc(below);
-    if (below != kFull) break;
-  }
-  return l;
-}
 
 // CPL chunks per lane: rows of up to 256 * CPL experts.
 template <int CPL>

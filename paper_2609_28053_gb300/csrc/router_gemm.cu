@@ -24,122 +24,12 @@
 // makes all roles leave their loops, the MMA thread drains its outstanding
 // tensor-core work through one more commit, TMEM is freed, and the kernel
 // reports EQB_ERR_CUDA through the error word.
-#include <cuda.h>
-
 #include "coarse_window.cuh"
-#include "eqb_device.cuh"
+#include "tcgen05.cuh"
 
 namespace eqb {
 
 namespace {
-
-constexpr int kBM = 128;  // rows of x per tile (UMMA M)
-constexpr int kBK = 64;   // bf16 columns per stage: one 128-byte swizzle atom
-constexpr uint32_t kSpinLimit = 1u << 20;  // polls of at most ~1 us: about a second
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity), "r"(1000u)
-      : "memory");
-  return ok != 0;
-}
-// Bounded wait for the phase of parity `parity`; false if it timed out or
-// another role aborted.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
-  for (uint32_t i = 0; i < kSpinLimit; ++i) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if ((i & 63u) == 63u && *abort_flag) return false;
-  }
-  *abort_flag = 1;
-  return false;
-}
-
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0,
-                                            int c1) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%3, %4}], [%2];" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(bar), "r"(c0), "r"(c1)
-      : "memory");
-}
-
-__device__ __forceinline__ void tc_fence_before() {
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-}
-__device__ __forceinline__ void tc_fence_after() {
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-}
-
-// UMMA shared-memory descriptor of a K-major tile stored as 128-byte swizzled
-// rows (8-row atoms of 1 KiB): start address >> 4 (bits 0-13), leading byte
-// offset 16 B (unused for this layout), stride byte offset 1 KiB between
-// 8-row groups (bits 32-45), descriptor version 1 (bit 46), swizzle mode
-// 128B (value 2 in bits 61-63).
-__device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
-  uint64_t d = static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4);
-  d |= static_cast<uint64_t>(16u >> 4) << 16;
-  d |= static_cast<uint64_t>(1024u >> 4) << 32;
-  d |= static_cast<uint64_t>(1u) << 46;
-  d |= static_cast<uint64_t>(2u) << 61;
-  return d;
-}
-
-// Instruction descriptor, kind::f16: fp32 accumulator (bits 4-5 = 1), A and
-// B bf16 (bits 7-9 = 1, 10-12 = 1), both K-major, N >> 3 in bits 17-22,
-// M >> 4 in bits 24-28.
-__host__ __device__ constexpr uint32_t umma_idesc_bf16(int M, int N) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((static_cast<uint32_t>(N) >> 3) << 17) |
-         ((static_cast<uint32_t>(M) >> 4) << 24);
-}
-
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                          uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-__device__ __forceinline__ void umma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar)
-               : "memory");
-}
-
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
-        "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]),
-        "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]),
-        "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
-constexpr uint32_t kTmemCols = 512;  // the whole TMEM of the SM: one CTA per SM
 
 struct GemmArgs {
   uint16_t* z;
@@ -492,42 +382,6 @@ __global__ void __launch_bounds__(192, 1)
   if (threadIdx.x == 0 && *abort_flag) raise_flag(err, kErrCuda);
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*,
-                                  CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
-                                  CUtensorMapFloatOOBfill);
-
-EncodeTiledFn encode_fn() {
-  static EncodeTiledFn fn = nullptr;
-  if (!fn) {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-            cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<EncodeTiledFn>(p);
-  }
-  return fn;
-}
-
-// 2-D bf16 tensor map over a row-major [rows, cols] matrix, box [box_rows, 64]
-// (64 bf16 = one 128-byte swizzle atom per row).
-bool make_map(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t cols, uint32_t box_rows) {
-  EncodeTiledFn fn = encode_fn();
-  if (!fn) return false;
-  const cuuint64_t dims[2] = {cols, rows};
-  const cuuint64_t strides[1] = {cols * 2};
-  const cuuint32_t box[2] = {static_cast<cuuint32_t>(kBK), box_rows};
-  const cuuint32_t estr[2] = {1, 1};
-  return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-}  // namespace
-
-namespace {
-
 template <int EC, int KP1, bool HIST>
 int launch_gemm(const uint16_t* x, const uint16_t* W, GemmArgs a, cudaStream_t s) {
   DeviceInfo di;
@@ -557,7 +411,15 @@ int launch_gemm(const uint16_t* x, const uint16_t* W, GemmArgs a, cudaStream_t s
 }  // namespace
 
 int launch_router_gemm(const uint16_t* x, const uint16_t* W, int64_t T, int d, int E, uint16_t* z,
-                       int32_t* err, cudaStream_t s) {
+                       int32_t* err, bool split, cudaStream_t s) {
+  if (split) {
+    DeviceInfo di;
+    if (int rc = device_info(&di)) return rc;
+    if (const int n = router_splits(T, d, di.sm_count); n > 1) {
+      const SplitRoute none;
+      return launch_router_split(x, W, T, d, E, n, z, none, err, s);
+    }
+  }
   GemmArgs a{z, static_cast<int>(T), d, E, 0, err, nullptr, 0, nullptr, 0, nullptr, nullptr, nullptr, nullptr};
   return launch_gemm<0, 1, false>(x, W, a, s);
 }
@@ -573,9 +435,20 @@ int launch_route_ec(const uint16_t* x, const uint16_t* W, const GemmArgs& a, cud
 
 int launch_router_route(const uint16_t* x, const uint16_t* W, int64_t T, int d, int E, int K, const float* b,
                         const int64_t* off, int M, uint16_t* z, int32_t* idx, float* tau, int32_t* loads,
-                        int32_t* hist, int32_t* err, cudaStream_t s) {
-  GemmArgs a{z, static_cast<int>(T), d, E, 0, err, b, K, off, M, idx, tau, loads, hist};
+                        int32_t* hist, int32_t* err, bool split, cudaStream_t s) {
   if (E != 64 && E != 128) return kErrUnsupported;
+  if (split) {
+    DeviceInfo di;
+    if (int rc = device_info(&di)) return rc;
+    if (const int n = router_splits(T, d, di.sm_count); n > 1) {
+      const SplitRoute ro{b, K, off, M, idx, tau, loads};
+      const int rc = launch_router_split(x, W, T, d, E, n, z, ro, err, s);
+      if (rc || !hist) return rc;
+      HistArgs h{z, tau, T, E, nullptr, hist, err};
+      return launch_hist(h, 1, s);
+    }
+  }
+  GemmArgs a{z, static_cast<int>(T), d, E, 0, err, b, K, off, M, idx, tau, loads, hist};
   bool in_epilogue = false;
   if (hist) {
     // the epilogue's 16-bit window counters are added into H once, at the

@@ -236,11 +236,11 @@ eqb_status eqb_router_layer_step(const eqb_bf16* x, const eqb_bf16* W_r, int64_t
   if ((E == 64 || E == 128) && K <= 8) {
     // projection, routing and the coarse histogram in one kernel
     if (int rc = eqb::launch_router_route(x, W_r, T, d, E, K, b, mb_offsets, M, z, topk_idx, tau, loads, w.H,
-                                          err_flag, s))
+                                          err_flag, false, s))
       return st(rc);
     return after_coarse(w, z, T, E, K, mb_offsets, M, r, tau, loads, b_next, grad_s, eta, c, err_flag, s);
   } else {
-    if (int rc = eqb::launch_router_gemm(x, W_r, T, d, E, z, err_flag, s)) return st(rc);
+    if (int rc = eqb::launch_router_gemm(x, W_r, T, d, E, z, err_flag, false, s)) return st(rc);
     eqb::RouteArgs ra{z, b, T, E, K, mb_offsets, M, 0, topk_idx, tau, loads, err_flag};
     if (int rc = eqb::launch_route(ra, s)) return st(rc);
   }

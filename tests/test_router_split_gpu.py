@@ -1,0 +1,62 @@
+"""GPU parity of the router projection for few tokens, where a cluster of 2, 4
+or 8 blocks shares each 128-token tile: on integer-valued inputs (every sum is
+exact in fp32, in any order) z equals the rounded exact product bit for bit,
+and the routed outputs equal routing those logits; T lies on both sides of the
+lines between cluster sizes."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2609_28053_gb300 as eqb
+from eqb_workloads import ragged_offsets
+from gpu_harness import Guarded
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib(cuda_ok):
+    eqb.load()
+
+
+def inputs(T, d, E, seed):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    x = torch.randint(-8, 9, (T, d), generator=g, device="cuda").to(torch.bfloat16)
+    W = torch.randint(-4, 5, (E, d), generator=g, device="cuda").to(torch.bfloat16)
+    z = (x.double() @ W.double().t()).to(torch.float32).to(torch.bfloat16)  # |sums| < 2^17: exact in fp32
+    return x, W, z
+
+
+@pytest.mark.parametrize("T", [1, 8, 127, 129, 1024, 1025, 1153, 4096, 4225, 8192, 8449])
+@pytest.mark.parametrize("d,E", [(1024, 128), (4096, 64)])
+def test_route(T, d, E):
+    K, M = (8, 5) if T > 8 else (3, 1)
+    x, W, z_ref = inputs(T, d, E, seed=T + E)
+    b = torch.randn(E, device="cuda") * 30.0
+    off = torch.from_numpy(ragged_offsets(T, M, seed=T) if M > 1 else np.array([0, T], np.int64)).cuda()
+    z, idx, tau, loads = (Guarded((T, E), torch.bfloat16), Guarded((T, K), torch.int32), Guarded((T,), torch.float32),
+                          Guarded((M, E), torch.int32))
+    hist, err = Guarded((E, 256), torch.int32), torch.zeros(1, dtype=torch.int32, device="cuda")
+    eqb.eqb_router_route(x, W, b, K, off, z=z.view, topk_idx=idx.view, tau=tau.view, loads=loads.view, err_flag=err,
+                         hist_hi=hist.view)
+    idx2, tau2 = torch.empty((T, K), dtype=torch.int32, device="cuda"), torch.empty(T, device="cuda")
+    loads2, hist2 = torch.zeros((M, E), dtype=torch.int32, device="cuda"), torch.zeros((E, 256), dtype=torch.int32,
+                                                                                     device="cuda")
+    eqb.eqb_route_topk(z_ref, b, K, off, idx2, tau2, loads2, hist_hi=hist2)
+    torch.cuda.synchronize()
+    assert all(g.intact() for g in (z, idx, tau, loads, hist)) and err.item() == 0
+    assert torch.equal(z.view.view(torch.int16), z_ref.view(torch.int16))
+    assert torch.equal(idx.view, idx2) and torch.equal(tau.view, tau2)
+    assert torch.equal(loads.view, loads2) and torch.equal(hist.view, hist2)
+
+
+@pytest.mark.parametrize("T,d,E", [(5, 1024, 16), (300, 1088, 48), (130, 2048, 240), (1100, 1024, 256), (4300, 1600, 256)])
+def test_logits(T, d, E):
+    """Expert counts that fill no whole run of lanes, columns that the blocks
+    of a cluster share unevenly."""
+    x, W, z_ref = inputs(T, d, E, seed=T)
+    z, err = Guarded((T, E), torch.bfloat16), torch.zeros(1, dtype=torch.int32, device="cuda")
+    eqb.eqb_router_logits(x, W, z=z.view, err_flag=err)
+    torch.cuda.synchronize()
+    assert z.intact() and err.item() == 0
+    assert torch.equal(z.view.view(torch.int16), z_ref.view(torch.int16))
