@@ -39,17 +39,22 @@ __all__ = [
 
 
 def _p(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream):
+    """The raw stream handle; the current stream of the current device by
+    default (the tensors of a call are on the GPU, so CUDA is initialised)."""
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    return stream.cuda_stream
 
 
 def _need(t, dtype, name, shape=None):
-    if t is None:
+    # one line for a tensor that fits, the reasons below for one that does not:
+    # a call checks up to ten tensors, which takes longer than its launches
+    if t is None or (type(t) is torch.Tensor and t.dtype is dtype and t.is_cuda and t.is_contiguous()
+                     and (shape is None or t.shape == shape)):
         return
     if not isinstance(t, torch.Tensor):
         raise TypeError(f"{name} must be a torch.Tensor")

@@ -37,6 +37,8 @@ class EqbError(RuntimeError):
 
 def load(path: str | None = None) -> ctypes.CDLL:
     global _lib
+    if _lib is not None and path is None:
+        return _lib
     with _lock:
         if _lib is not None and path is None:
             return _lib
