@@ -353,11 +353,21 @@ struct HistCut {
 // From 7,000 chunks per SM on, copies that give the 32 lanes of a warp bins
 // of their own pay for their zeroing: T = 1,000,000, E = 64 31 us against
 // 45 (pass 1), T = 60,000, E = 160 10.3 against 12.1; T = 65,536, E = 64
-// (3,400) 7.5 against 6.8.  Pass 2 counts few elements and takes one copy.
+// (3,400) 7.5 against 6.8.  Pass 2 counts few elements, so that its lanes
+// rarely meet: one copy, and narrower tiles, whose selections take one round
+// of the block's warps and whose flushes (nearly every low byte occurs) add
+// fewer counters to the global histogram.  The step with tiles of 4, 8 and 16
+// chunks: T = 30,873, E = 256 35 / 37 / 42 us, T = 65,536, E = 64 31 / 35 /
+// 35, T = 524,288, E = 128 185 / 187 / 190, E = 256 321 / 321 / 325, T =
+// 1,048,576, E = 512 1220 / 1219 / 1211.
 HistCut cut_hist(int64_t T, int E, int pass, int blocks) {
   const int nch = E >> 3;
   const int64_t per_sm = T * nch / blocks;  // chunks of z to count per SM
-  const int want = per_sm < 10000 ? 8 : 16;
+  int want = per_sm < 10000 ? 8 : 16;
+  if (pass == 2) {
+    want = per_sm < 64000 ? 4 : per_sm < 200000 ? 8 : 16;
+    if (want * kMaxHistTiles < nch) want = (nch + kMaxHistTiles - 1) / kMaxHistTiles;
+  }
   HistCut h;
   h.tiles = (nch + want - 1) / want;
   h.chunks = (nch + h.tiles - 1) / h.tiles;

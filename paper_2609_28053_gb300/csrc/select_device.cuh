@@ -72,27 +72,29 @@ __device__ __forceinline__ void block_bias_update(const uint16_t* q_hat, int E, 
                                                   int nthreads, Sync sync) {
   __shared__ double mean;
   auto q_at = [&](int e) -> uint32_t { return __ldcg(q_hat + e); };
+  const uint32_t mine = threadIdx.x < E ? q_at(threadIdx.x) : 0u;  // in flight beside warp 0's
 
   if (threadIdx.x < 32) {
     const int lane = threadIdx.x;
     double part = 0.0;
     int lo = 1 << 20, hi = -(1 << 20);
-#pragma unroll 4
-    for (int e = lane; e < E; e += 32) {
-      const uint32_t x = q_at(e);
-      if ((x & 0x7fffu) != 0u) {
-        int l, h;
-        bf16_exp_range(x, l, h);
-        lo = min(lo, l);
-        hi = max(hi, h);
-      }
-      part = __dadd_rn(part, (double)bf16_bits_to_f32(x));
-    }
+    for (int e0 = lane; e0 < E; e0 += 256) {
+      uint32_t x[8];  // eight loads in flight; +0 past E changes neither the sum nor its range
 #pragma unroll
-    for (int d = 16; d > 0; d >>= 1) {
-      lo = min(lo, __shfl_xor_sync(kFull, lo, d));
-      hi = max(hi, __shfl_xor_sync(kFull, hi, d));
+      for (int k = 0; k < 8; ++k) x[k] = e0 + 32 * k < E ? q_at(e0 + 32 * k) : 0u;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        if ((x[k] & 0x7fffu) != 0u) {
+          int l, h;
+          bf16_exp_range(x[k], l, h);
+          lo = min(lo, l);
+          hi = max(hi, h);
+        }
+        part = __dadd_rn(part, (double)bf16_bits_to_f32(x[k]));
+      }
     }
+    lo = __reduce_min_sync(kFull, lo);
+    hi = __reduce_max_sync(kFull, hi);
     double sum;
     const int lg = 32 - __clz(E - 1);  // ceil(log2 E)
     if (hi - lo + 1 + lg <= 52 || hi < lo) {
@@ -107,7 +109,8 @@ __device__ __forceinline__ void block_bias_update(const uint16_t* q_hat, int E, 
     if (lane == 0) mean = __ddiv_rn(sum, (double)E);
   }
   sync();
-  for (int e = threadIdx.x; e < E; e += nthreads)
+  if (threadIdx.x < E) b_next[threadIdx.x] = __double2float_rn(__dsub_rn((double)bf16_bits_to_f32(mine), mean));
+  for (int e = threadIdx.x + nthreads; e < E; e += nthreads)
     b_next[e] = __double2float_rn(__dsub_rn((double)bf16_bits_to_f32(q_at(e)), mean));
 }
 
