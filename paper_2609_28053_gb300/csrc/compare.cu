@@ -27,7 +27,13 @@ __device__ void center_store(double* x, int E, float* b) {
   __syncthreads();
   if (threadIdx.x == 0) {
     double acc = 0.0;
-    for (int e = 0; e < E; ++e) acc += x[e];
+    for (int e = 0; e < E; e += 8) {  // E is a multiple of 8: eight reads ahead of the chain of sums
+      double v[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) v[k] = x[e + k];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) acc += v[k];
+    }
     mean = acc / (double)E;
   }
   __syncthreads();
@@ -39,18 +45,58 @@ __device__ void center_store(double* x, int E, float* b) {
 __global__ void __launch_bounds__(256) shard_average_kernel(const uint16_t* q, const int64_t* off, int P, int E,
                                                             float* b) {
   __shared__ double x[kMaxE];
+  griddep_wait();
   for (int e = threadIdx.x; e < E; e += blockDim.x) {
     double acc = 0.0;
     int cnt = 0;
-    for (int p = 0; p < P; ++p) {
-      if (off[p + 1] > off[p]) {
-        acc += (double)bf16_bits_to_f32(q[(int64_t)p * E + e]);
-        ++cnt;
+    for (int p0 = 0; p0 < P; p0 += 8) {  // eight shards' loads in flight
+      uint32_t v[8];
+      bool some[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const int p = min(p0 + k, P - 1);
+        v[k] = q[(int64_t)p * E + e];
+        some[k] = p0 + k < P && off[p + 1] > off[p];
       }
+#pragma unroll
+      for (int k = 0; k < 8; ++k)
+        if (some[k]) {
+          acc += (double)bf16_bits_to_f32(v[k]);
+          ++cnt;
+        }
     }
     x[e] = acc / (double)cnt;
   }
   center_store(x, E, b);
+}
+
+// The first kernel of a comparison: zeros n16 16-byte words of its histograms
+// and, up to kParamShards shards, writes the shard offsets, which come as an
+// argument (in place of two memsets and a copy from pageable memory, none of
+// which overlap anything).
+constexpr int kParamShards = 128;
+struct ShardOffsets {
+  int64_t v[kParamShards + 1];
+};
+__global__ void __launch_bounds__(256) setup_kernel(uint4* w, int64_t n16, int64_t* off, int n,
+                                                    const __grid_constant__ ShardOffsets so) {
+  griddep_wait();
+  griddep_launch();
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n16; i += stride)
+    w[i] = make_uint4(0u, 0u, 0u, 0u);
+  if (blockIdx.x == 0)
+    for (int i = threadIdx.x; i < n; i += blockDim.x) off[i] = so.v[i];
+}
+int launch_setup(void* w, size_t bytes, int64_t* off, const int64_t* off_host, int n, cudaStream_t s) {
+  ShardOffsets so;
+  for (int i = 0; i < n; ++i) so.v[i] = off_host[i];
+  const int64_t n16 = static_cast<int64_t>(bytes / 16);
+  const int64_t grid = (n16 + 1023) / 1024;
+  return launch_dependent(setup_kernel, dim3((unsigned)(grid < 608 ? grid : 608)), dim3(256), 0, s,
+                          static_cast<uint4*>(w), n16, off, n, so) == cudaSuccess
+             ? kOk
+             : kErrCuda;
 }
 
 // Scratch of the rank average: per-shard histograms H and L [P,E,256],
@@ -81,6 +127,7 @@ size_t carve_shards(void* base, int E, int P, ShardWs* w) {
 __global__ void __launch_bounds__(256) bin_edge_kernel(const uint8_t* u, int E, float lo, float w, float* b,
                                                        double* est) {
   __shared__ double x[kMaxE];
+  griddep_wait();
   for (int e = threadIdx.x; e < E; e += blockDim.x) {
     x[e] = (double)lo + (double)(u[e] + 1) * (double)w;
     if (est) est[e] = x[e];
@@ -129,10 +176,13 @@ eqb_status eqb_rank_averaged_bias(const eqb_bf16* z, const float* tau, int64_t T
   eqb::ShardWs w;
   if (eqb::carve_shards(workspace, E, P, &w) > workspace_bytes) return EQB_ERR_INVALID_ARG;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  const size_t hb = (size_t)P * (size_t)E * 256 * 4;
-  if (cudaMemsetAsync(w.H, 0, hb, s) != cudaSuccess || cudaMemsetAsync(w.L, 0, hb, s) != cudaSuccess ||
-      cudaMemcpyAsync(w.off, shard_offsets_host, ((size_t)P + 1) * 8, cudaMemcpyHostToDevice, s) != cudaSuccess)
+  // H and L are adjacent (each a multiple of 256 bytes)
+  const size_t hb = 2 * (size_t)P * (size_t)E * 256 * 4;
+  const int n = P <= eqb::kParamShards ? P + 1 : 0;
+  if (n == 0 && cudaMemcpyAsync(w.off, shard_offsets_host, ((size_t)P + 1) * 8, cudaMemcpyHostToDevice, s) !=
+                    cudaSuccess)
     return EQB_ERR_CUDA;
+  if (int rc = eqb::launch_setup(w.H, hb, w.off, shard_offsets_host, n, s)) return eqb::st(rc);
   // Both radix passes over all tokens at once, each shard counted into its
   // own histogram, then one selection per (shard, expert).
   eqb::HistArgs h1{z, tau, T, E, nullptr, w.H, err_flag};
@@ -147,8 +197,11 @@ eqb_status eqb_rank_averaged_bias(const eqb_bf16* z, const float* tau, int64_t T
   if (int rc = eqb::launch_hist(h2, 2, s)) return eqb::st(rc);
   if (int rc = eqb::launch_select_sharded(w.L, E, 2, w.off, P, K, w.u, w.rho, q_shards, err_flag, s))
     return eqb::st(rc);
-  eqb::shard_average_kernel<<<1, 256, 0, s>>>(q_shards, w.off, P, E, b_out);
-  return cudaGetLastError() == cudaSuccess ? EQB_OK : EQB_ERR_CUDA;
+  return eqb::launch_dependent(eqb::shard_average_kernel, dim3(1), dim3(256), 0, s,
+                               static_cast<const uint16_t*>(q_shards), static_cast<const int64_t*>(w.off), (int)P,
+                               (int)E, b_out) == cudaSuccess
+             ? EQB_OK
+             : EQB_ERR_CUDA;
 }
 
 eqb_status eqb_fixed_hist_bias(const eqb_bf16* z, const float* tau, int64_t T, int32_t E, int32_t K, float lo,
@@ -162,15 +215,17 @@ eqb_status eqb_fixed_hist_bias(const eqb_bf16* z, const float* tau, int64_t T, i
   eqb::StepWorkspace w;
   if (eqb::carve_workspace(workspace, E, &w) > workspace_bytes) return EQB_ERR_INVALID_ARG;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  if (cudaMemsetAsync(w.H, 0, (size_t)E * 1024, s) != cudaSuccess) return EQB_ERR_CUDA;
+  if (int rc = eqb::launch_setup(w.H, (size_t)E * 1024, nullptr, nullptr, 0, s)) return eqb::st(rc);
   eqb::HistArgs h{z, tau, T, E, nullptr, w.H, err_flag};
   h.lo = lo;
   h.inv_w = 1.0f / width;
   if (int rc = eqb::launch_hist(h, 3, s)) return eqb::st(rc);
   const int64_t r = eqb_target_rank(T, E, K);
   if (int rc = eqb::launch_select(w.H, E, 3, r, w.u, w.rho, nullptr, err_flag, s)) return eqb::st(rc);
-  eqb::bin_edge_kernel<<<1, 256, 0, s>>>(w.u, E, lo, width, b_out, estimate);
-  return cudaGetLastError() == cudaSuccess ? EQB_OK : EQB_ERR_CUDA;
+  return eqb::launch_dependent(eqb::bin_edge_kernel, dim3(1), dim3(256), 0, s, static_cast<const uint8_t*>(w.u),
+                               (int)E, lo, width, b_out, estimate) == cudaSuccess
+             ? EQB_OK
+             : EQB_ERR_CUDA;
 }
 
 }  // extern "C"

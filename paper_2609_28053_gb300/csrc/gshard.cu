@@ -22,9 +22,13 @@ constexpr int kGsThreads = 256;
 template <int LPT, int CPL>
 __global__ void __launch_bounds__(kGsThreads) gshard_kernel(GshardArgs a, int64_t tokens_per_cta) {
   constexpr int TPW = 32 / LPT;  // tokens per warp step
+  // four chunks a lane leave registers for one token (E = 1024, T = 200,000
+  // 367 us with one, 584 with two); fewer are faster with two
+  constexpr int U = CPL < 4 ? 2 : 1;
   __shared__ __align__(16) float Rs[kMaxE];
   __shared__ float cs;
   const int E = a.E, nch = E >> 3;
+  griddep_wait();
   const int64_t tb = (int64_t)blockIdx.x * tokens_per_cta;
   const int64_t te = min(tb + tokens_per_cta, a.T);
   if (tb >= te) return;
@@ -61,16 +65,16 @@ __global__ void __launch_bounds__(kGsThreads) gshard_kernel(GshardArgs a, int64_
     }
     const float c0 = cs;
 
-    // Two tokens per lane per round, every load issued before any use, so
-    // the z and grad loads of both overlap.
+    // U tokens per lane per round, every load issued before any use, so the
+    // z and grad loads of all overlap.
     const int64_t stride = (int64_t)nw * TPW;
-    for (int64_t base = t + (int64_t)wid * TPW; base < seg_end; base += 2 * stride) {
-      int64_t tok[2];
-      bool ok[2];
-      uint4 w[2][CPL];
-      float4 g0[2][CPL], g1[2][CPL];
+    for (int64_t base = t + (int64_t)wid * TPW; base < seg_end; base += U * stride) {
+      int64_t tok[U];
+      bool ok[U];
+      uint4 w[U][CPL];
+      float4 g0[U][CPL], g1[U][CPL];
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
+      for (int u = 0; u < U; ++u) {
         tok[u] = base + u * stride + slot;
         ok[u] = tok[u] < seg_end;
 #pragma unroll
@@ -85,7 +89,7 @@ __global__ void __launch_bounds__(kGsThreads) gshard_kernel(GshardArgs a, int64_
         }
       }
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
+      for (int u = 0; u < U; ++u) {
         float d = 0.f, num = 0.f;
 #pragma unroll
         for (int k = 0; k < CPL; ++k) {
@@ -139,12 +143,15 @@ int launch_gs(const GshardArgs& a, cudaStream_t s) {
   DeviceInfo di;
   if (int rc = device_info(&di)) return rc;
   int64_t grid = (int64_t)di.sm_count * 8;
-  const int64_t max_grid = (a.T + 255) / 256;  // at least 256 tokens per CTA
+  // at least 64 tokens per CTA (T = 11,409, E = 512 28 us; 69 with 256, which
+  // left most SMs idle)
+  const int64_t max_grid = (a.T + 63) / 64;
   if (grid > max_grid) grid = max_grid;
   if (grid < 1) grid = 1;
   const int64_t tpc = (a.T + grid - 1) / grid;
-  gshard_kernel<LPT, CPL><<<(unsigned)grid, kGsThreads, 0, s>>>(a, tpc);
-  return cudaGetLastError() == cudaSuccess ? kOk : kErrCuda;
+  return launch_dependent(gshard_kernel<LPT, CPL>, dim3((unsigned)grid), dim3(kGsThreads), 0, s, a, tpc) == cudaSuccess
+             ? kOk
+             : kErrCuda;
 }
 
 }  // namespace
@@ -157,6 +164,7 @@ int launch_gshard(const GshardArgs& a, cudaStream_t s) {
   if (nch <= 8) return launch_gs<8, 1>(a, s);
   if (nch <= 16) return launch_gs<16, 1>(a, s);
   if (nch <= 32) return launch_gs<32, 1>(a, s);
+  if (nch <= 48) return launch_gs<16, 3>(a, s);  // E = 264, T = 241,812 172 us; 272 with half of 32 x 2 idle
   if (nch <= 64) return launch_gs<32, 2>(a, s);
   if (nch <= 96) return launch_gs<32, 3>(a, s);
   if (nch <= 128) return launch_gs<32, 4>(a, s);

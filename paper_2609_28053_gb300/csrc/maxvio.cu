@@ -25,6 +25,7 @@ __global__ void __launch_bounds__(kThreads) maxvio_kernel(const int32_t* __restr
   extern __shared__ double sv[];
   __shared__ long long wmax[kThreads / 32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  griddep_wait();
 
   // Largest load of every microbatch (warps take microbatches).
   for (int l = wid; l < M; l += nw) {
@@ -99,8 +100,10 @@ int launch_maxvio(const int32_t* loads, const int64_t* off, int M, int E, int K,
   if (smem > 48 * 1024 &&
       cudaFuncSetAttribute(maxvio_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
     return kErrCuda;
-  maxvio_kernel<<<1, kThreads, smem, s>>>(loads, off, M, E, K, out, per_mb);
-  return cudaGetLastError() == cudaSuccess ? kOk : kErrCuda;
+  return launch_dependent(maxvio_kernel, dim3(1), dim3(kThreads), smem, s, loads, off, M, E, K, out, per_mb) ==
+                 cudaSuccess
+             ? kOk
+             : kErrCuda;
 }
 
 }  // namespace eqb
