@@ -168,6 +168,10 @@ __device__ __forceinline__ void route_row(const uint8_t* rowp, const float* bs, 
     }
   }
 
+  // a lane past the end of the batch has no candidates (its row is zeros or
+  // left over, often all equal: the warp would walk every expert of it)
+  if (!valid) hits = m = m1 = 0u;
+
   // ---- C: exact top-(K+1) of the experts with a hit, in ascending index,
   // one per lane per step, taken from the mask words 32 experts at a time;
   // the next candidate's z and b are read one step ahead.  Refills are
@@ -212,6 +216,10 @@ __device__ __forceinline__ void route_row(const uint8_t* rowp, const float* bs, 
     z0 = z1;
     b0 = b1;
   }
+  // after a NaN score (flagged) a finished lane's -1 can enter the list: the
+  // loads are counted by these numbers
+#pragma unroll
+  for (int j = 0; j < KP1; ++j) id[j] = max(id[j], 0);
 }
 
 // tau_t = v[K] of the sorted list (K < KP1 chosen at run time).
