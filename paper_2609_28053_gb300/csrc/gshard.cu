@@ -19,14 +19,17 @@ namespace {
 
 constexpr int kGsThreads = 256;
 
+// At most 128 registers where a lane holds several chunks: with one block an
+// SM instead of two, E = 264, T = 241,812 takes 286 us instead of 172.
 template <int LPT, int CPL>
-__global__ void __launch_bounds__(kGsThreads) gshard_kernel(GshardArgs a, int64_t tokens_per_cta) {
+__global__ void __launch_bounds__(kGsThreads, CPL > 1 ? 2 : 4) gshard_kernel(GshardArgs a, int64_t tokens_per_cta) {
   constexpr int TPW = 32 / LPT;  // tokens per warp step
   // four chunks a lane leave registers for one token (E = 1024, T = 200,000
   // 367 us with one, 584 with two); fewer are faster with two
   constexpr int U = CPL < 4 ? 2 : 1;
   __shared__ __align__(16) float Rs[kMaxE];
   __shared__ float cs;
+  __shared__ double inv[2];  // 1 / (K n) and 1 / E
   const int E = a.E, nch = E >> 3;
   griddep_wait();
   const int64_t tb = (int64_t)blockIdx.x * tokens_per_cta;
@@ -40,13 +43,18 @@ __global__ void __launch_bounds__(kGsThreads) gshard_kernel(GshardArgs a, int64_
     const int l = microbatch_of(a.off, a.M, t);
     const int64_t lo = __ldg(a.off + l), hi = __ldg(a.off + l + 1);
     const int64_t seg_end = (hi > t) ? min(te, hi) : te;
-    __syncthreads();  // the previous segment is done with Rs and cs
+    __syncthreads();  // the previous segment is done with Rs, cs and inv
     const int64_t n = hi - lo;
+    if (threadIdx.x == 0) {
+      inv[0] = n > 0 ? 1.0 / ((double)a.K * (double)n) : 0.0;
+      inv[1] = 1.0 / (double)E;
+      cs = n > 0 ? __double2float_rn((double)a.alpha / (double)n) : 0.f;
+    }
+    __syncthreads();
+    // the divisions once per segment: fp64 runs at two lanes a clock here, and
+    // one per expert took 12 of 115 us at T = 524,288, E = 128
     for (int e = threadIdx.x; e < E; e += blockDim.x)
-      Rs[e] = n > 0 ? __double2float_rn((double)__ldg(a.loads + (int64_t)l * E + e) / ((double)a.K * (double)n) -
-                                        1.0 / (double)E)
-                    : 0.f;
-    if (threadIdx.x == 0) cs = n > 0 ? __double2float_rn((double)a.alpha / (double)n) : 0.f;
+      Rs[e] = n > 0 ? __double2float_rn((double)__ldg(a.loads + (int64_t)l * E + e) * inv[0] - inv[1]) : 0.f;
     __syncthreads();
     // this lane's chunks: sub, sub + LPT, ... (CPL of them, past nch unused)
     float r[CPL][8];
@@ -164,7 +172,7 @@ int launch_gshard(const GshardArgs& a, cudaStream_t s) {
   if (nch <= 8) return launch_gs<8, 1>(a, s);
   if (nch <= 16) return launch_gs<16, 1>(a, s);
   if (nch <= 32) return launch_gs<32, 1>(a, s);
-  if (nch <= 48) return launch_gs<16, 3>(a, s);  // E = 264, T = 241,812 172 us; 272 with half of 32 x 2 idle
+  if (nch <= 48) return launch_gs<16, 3>(a, s);  // E = 264: half of 32 x 2 would be idle
   if (nch <= 64) return launch_gs<32, 2>(a, s);
   if (nch <= 96) return launch_gs<32, 3>(a, s);
   if (nch <= 128) return launch_gs<32, 4>(a, s);

@@ -109,8 +109,11 @@ int launch_lei(const LeiArgs& a, cudaStream_t s) {
   DeviceInfo di;
   if (int rc = device_info(&di)) return rc;
   int64_t grid = (int64_t)di.sm_count * 8;
-  // at least 256 tokens per CTA so the per-microbatch prologue stays small
-  const int64_t max_grid = (a.T + 255) / 256;
+  // At least 256 tokens per CTA, so that the per-microbatch prologue stays
+  // small, but no fewer CTAs than SMs while they have 16 tokens.
+  int64_t least = a.T / di.sm_count;
+  least = least < 16 ? 16 : least > 256 ? 256 : least;
+  const int64_t max_grid = (a.T + least - 1) / least;
   if (grid > max_grid) grid = max_grid;
   if (grid < 1) grid = 1;
   const int64_t tpc = (a.T + grid - 1) / grid;
