@@ -34,6 +34,7 @@ struct LeiStream {
   const int64_t* off = nullptr;
   int M = 0;
   int64_t t0 = 0, t1 = 0;
+  int warps = 0;  // of a block that only stream (set at the launch)
 };
 
 struct RouteArgs {

@@ -32,7 +32,7 @@
 //
 // Fused with Load-Error Injection (the one-call step): the passes are bound
 // by issue, not by DRAM, while LEI (Sec. 4) is a pure DRAM stream that needs
-// only the loads.  A fused block gives a quarter of its warps to streaming
+// only the loads.  A fused block gives some of its warps to streaming
 // grad_s[t, e] += coef[mb(t), e] over its slice of a token range from the
 // start, the other warps count, and each counting warp joins the stream when
 // its counting is done; the stream is cut into chunks of about 8 KiB of
@@ -123,8 +123,8 @@ struct HistPlace {
   int tid, lane, wid;
   int tile, range;  // expert tile and token range of the block
   int e0, nct;      // the tile's first expert and its chunks (the last tile may be narrower)
-  int nw, nt;       // counting warps and threads (a quarter of a fused block streams LEI)
-  __device__ __forceinline__ HistPlace(int tiles, int tile_chunks, int E, bool lei) {
+  int nw, nt;       // counting warps and threads (the last lei_warps of a fused block stream LEI)
+  __device__ __forceinline__ HistPlace(int tiles, int tile_chunks, int E, int lei_warps) {
     int cta, n;
     asm volatile("mov.u32 %0, %%tid.x;" : "=r"(tid));
     asm volatile("mov.u32 %0, %%ctaid.x;" : "=r"(cta));
@@ -135,7 +135,7 @@ struct HistPlace {
     range = cta / tiles;
     e0 = tile * tile_chunks * 8;
     nct = min(tile_chunks, (E - e0) >> 3);
-    nw = lei ? (n >> 5) - (n >> 7) : n >> 5;
+    nw = (n >> 5) - lei_warps;
     nt = nw * 32;
   }
 };
@@ -158,7 +158,7 @@ __global__ void __launch_bounds__(1024) hist_kernel(HistArgs a, int tiles, int t
     }
     return;
   }
-  const HistPlace pl(tiles, tile_chunks, E, LEI);
+  const HistPlace pl(tiles, tile_chunks, E, LEI ? ls.warps : 0);
   const int tok = pl.tid / pl.nct;           // token slot (>= slots: no counting)
   const int c = pl.tid - tok * pl.nct;       // 8-expert chunk of the tile owned by this thread
   // Barrier of the counting warps (all warps unless fused).
@@ -277,7 +277,7 @@ __global__ void __launch_bounds__(1024) hist_kernel(HistArgs a, int tiles, int t
     }
     // from here on the thread's place is formed anew, so that the counting
     // loop does not hold it in registers
-    const HistPlace fl(tiles, tile_chunks, E, LEI);
+    const HistPlace fl(tiles, tile_chunks, E, LEI ? ls.warps : 0);
     sync_counting();
     // Flush: add every non-zero 16-bit counter to the global histogram.
     for (int i = fl.tid; i < fl.nct * 1024; i += fl.nt) {
@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(1024) hist_kernel(HistArgs a, int tiles, int t
     // block's fence after its count orders the other blocks' writes before
     // its reads.
     __shared__ int last;
-    const HistPlace fl(tiles, tile_chunks, E, LEI);
+    const HistPlace fl(tiles, tile_chunks, E, LEI ? ls.warps : 0);
     auto count_last = [&](int32_t* counter, int n) {
       if (fl.tid == 0) {
         __threadfence();
@@ -419,7 +419,16 @@ int launch_hist_coef(const HistArgs& a, const LeiArgs& la, float* coef, cudaStre
   return launch_hist_pass<1, false>(a, LeiStream(), CoefRows{la, coef, 0}, s);
 }
 
-int launch_hist_lei(const HistArgs& a, int pass, const LeiStream& ls, cudaStream_t s) {
+int launch_hist_lei(const HistArgs& a, int pass, const LeiStream& lei, cudaStream_t s) {
+  LeiStream ls = lei;
+  // of 32: the passes are DRAM-bound, and the more warps stream from the start
+  // the sooner they are, until counting is what takes longest.  A pass that
+  // carries every token, 8 / 14 / 16 / 18 / 20 / 24: T = 524,288, E = 128 184 /
+  // 182 / 180 / 182 / 182 / 198 us a step, T = 65,536, E = 64 31.4 / 31.2 /
+  // 31.0 / 34.1 / 32.9 / 34.7; half of them each, 8 / 12 / 13 / 14 / 16: T =
+  // 2,097,152, E = 256 1198 / 1180 / 1177 / 1175 / 1191, T = 1,048,576, E =
+  // 512 1209 / 1191 / 1188 / 1185 / 1199.
+  ls.warps = ls.t1 - ls.t0 == a.T ? 16 : 14;
   if (!ls.g || !ls.coef || !ls.off || ls.M < 1 || ls.t0 < 0 || ls.t1 < ls.t0) return kErrInvalidArg;
   return pass == 1 ? launch_hist_pass<1, true>(a, ls, CoefRows(), s) : launch_hist_pass<2, true>(a, ls, CoefRows(), s);
 }
