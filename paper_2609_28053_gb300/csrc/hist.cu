@@ -152,9 +152,12 @@ __global__ void __launch_bounds__(1024) hist_kernel(HistArgs a, int tiles, int t
   if (PASS == 1 && !LEI && blockIdx.x >= gridDim.x - cr.blocks) {
     // the last cr.blocks blocks form the coefficient table meanwhile
     griddep_wait();
-    for (int l = blockIdx.x - (gridDim.x - cr.blocks); l < cr.a.M; l += cr.blocks) {
+    // a warp per row, the rows dealt out to the blocks first
+    const int first = (threadIdx.x >> 5) * cr.blocks + blockIdx.x - (gridDim.x - cr.blocks);
+    for (int l = first; l < cr.a.M; l += 32 * cr.blocks) {
       const int64_t n = __ldg(cr.a.off + l + 1) - __ldg(cr.a.off + l);
-      block_lei_coef<1024>(cr.a.loads + (int64_t)l * E, n, E, cr.a.K, cr.a.eta, cr.a.c, cr.coef + (int64_t)l * E);
+      warp_lei_coef(cr.a.loads + (int64_t)l * E, n, E, cr.a.K, cr.a.eta, cr.a.c, cr.coef + (int64_t)l * E,
+                    threadIdx.x & 31);
     }
     return;
   }
@@ -382,8 +385,9 @@ HistCut cut_hist(int64_t T, int E, int pass, int blocks) {
   return h;
 }
 
-// One block's rows of the coefficient table take about 2 us and 1 us for each
-// further one; a short pass gives it up to 16 SMs, a long one four.
+// A warp forms a row of the coefficient table in 2-3 us; a short pass gives
+// the rows up to 16 SMs, so that few share the fp64 pipe of one, a long one
+// four.
 int coef_blocks(int64_t T, int E, int M, int sm_count) {
   const int most = T * (E >> 3) / sm_count < 10000 ? 16 : 4;
   return M < most ? M : most;

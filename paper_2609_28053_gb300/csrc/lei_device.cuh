@@ -70,4 +70,31 @@ __device__ __forceinline__ void block_lei_coef(const int32_t* __restrict__ f, in
   __syncthreads();
 }
 
+// The same coefficients by one warp (bit for bit: the same operations per
+// expert, and exact reductions), for blocks that form several rows at once.
+__device__ __forceinline__ void warp_lei_coef(const int32_t* __restrict__ f, int64_t n, int E, int K, float eta,
+                                              float c, float* out, int lane) {
+  int lo = INT_MAX, hi = INT_MIN;
+#pragma unroll 8
+  for (int e = lane; e < E; e += 32) {
+    const int v = __ldg(f + e);
+    lo = min(lo, v);
+    hi = max(hi, v);
+  }
+  lo = __reduce_min_sync(kFull, lo);
+  hi = __reduce_max_sync(kFull, hi);
+  const double inv_fbar = n > 0 ? (double)E / ((double)K * (double)n) : 0.0;
+  const double rmax =
+      inv_fbar > 0.0 ? fmax(fabs((double)lo * inv_fbar - 1.0), fabs((double)hi * inv_fbar - 1.0)) : 0.0;
+  float sigma = 1.0f;
+  if (c > 0.0f) {
+    const float xi = __fdiv_rn(static_cast<float>(rmax), c);
+    sigma = (xi == 0.0f) ? 1.0f : __fdiv_rn(tanhf(xi), xi);
+  }
+  const double es = (double)eta * (double)sigma;
+#pragma unroll 4
+  for (int e = lane; e < E; e += 32)
+    out[e] = inv_fbar > 0.0 ? __double2float_rn(es * ((double)__ldg(f + e) * inv_fbar - 1.0)) : 0.f;
+}
+
 }  // namespace eqb
