@@ -478,17 +478,20 @@ class EqbWorkspace:
 
     def __init__(self, E: int, device="cuda"):
         self.E = E
-        self.hist_hi = torch.zeros((E, 256), dtype=torch.int32, device=device)
-        self.hist_lo = torch.zeros((E, 256), dtype=torch.int32, device=device)
+        # what zero_() clears lies in one buffer: one fill in place of three
+        self._cleared = torch.zeros(2 * E * 256 + 1, dtype=torch.int32, device=device)
+        self.hist_hi = self._cleared[:E * 256].view(E, 256)
+        self.hist_lo = self._cleared[E * 256:2 * E * 256].view(E, 256)
+        self.err = self._cleared[2 * E * 256:]
         self.u = torch.zeros(E, dtype=torch.uint8, device=device)
         self.rho = torch.zeros(E, dtype=torch.int32, device=device)
         self.q_hat = torch.zeros(E, dtype=torch.bfloat16, device=device)
-        self.err = torch.zeros(1, dtype=torch.int32, device=device)
 
     def zero_(self):
-        self.hist_hi.zero_()
-        self.hist_lo.zero_()
-        self.err.zero_()
+        self._cleared.zero_()
+        for t in (self.hist_hi, self.hist_lo, self.err):
+            if t._base is not self._cleared:  # replaced by the caller
+                t.zero_()
 
 
 def eqb_layer_forward(z, b, K, mb_offsets, ws: EqbWorkspace, topk_idx, tau, loads, b_next,
