@@ -207,11 +207,11 @@ class Step:
         self.r_global = None
         self.off_h = even_offsets(T, self.M)
         self.workspace = torch.zeros(eqb.eqb_layer_workspace_bytes(E), dtype=torch.uint8, device=dev)
-        # The one-call step streams LEI inside the two histogram passes when
-        # the [M,E] coefficient table fits its workspace (M * E <= 65,536),
-        # and each pass's last block runs that pass's selection; the
-        # per-kernel breakdown issues the same work through the separate
-        # entry points (the selections as kernels of their own).
+        # The one-call step streams LEI inside the histogram passes when the
+        # [M,E] coefficient table fits its workspace (M * E <= 65,536), and
+        # selects inside the fine pass; the per-kernel breakdown issues the
+        # same work through the separate entry points (the selections as
+        # kernels of their own).
         self.fused = self.M * E <= 65536
         self.coef = torch.empty((self.M, E), dtype=torch.float32, device=dev)
         if workload == "router":
@@ -314,17 +314,20 @@ class Step:
             rec(6, lambda: eqb.lei_inject_grad(g, self.loads, self.off, self.K, ETA, C_NORM, stream))
 
     def launches_per_step(self):
-        """Kernels of this library launched by one timed one-call step
-        (memsets and torch copies excluded).  Each histogram pass runs its
-        own selection in its last block (the fine pass also the bias update).
-        Router workload: the projection with routing and the coarse
-        histogram, the LEI coefficient table, the pass-1 selection and the
-        fine pass carrying LEI: 4.  Otherwise: routing, the coefficient
-        table and the two histogram passes carrying the injection: 4.
-        Without the table, LEI in its own launch instead: still 4.  (With
-        several ranks the histograms are summed between the passes, so the
-        step runs as the separate calls of `names`, one kernel each.)"""
-        return 4
+        """Kernels of this library launched by one timed one-call step (torch
+        copies excluded; with several ranks the step runs as the separate
+        calls of `names`, one kernel each).  The clearing kernel, routing (or
+        the projection with routing and the coarse histogram) and the fine
+        pass, which selects and updates the bias; the coarse pass unless the
+        projection counted it; the LEI coefficient table unless the coarse
+        pass forms it (T E <= 2^26), or LEI itself where the table does not
+        fit the workspace."""
+        n = 3
+        if self.workload != "router":
+            n += 1
+        if not self.fused or self.workload == "router" or self.T * self.E > 1 << 26:
+            n += 1
+        return n
 
     def algorithmic_bytes(self):
         """Bytes the two-pass method must move per step (see the design notes):
