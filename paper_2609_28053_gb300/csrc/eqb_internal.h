@@ -73,13 +73,15 @@ struct HistArgs {
   int P = 0;
   // Algorithm 1's selections inside pass 2 (the one-call step; no shards):
   // with `coarse` (pass 1's [E,256] counts) every block selects u, rho of its
-  // experts at rank r itself.  With `done` (zero before the pass), done[i]
-  // counts the blocks of expert tile i that finished, the tile's last one
-  // selects its q_hat, done[kMaxHistTiles] counts the tiles selected, and the
-  // last one forms b_next (Eq. 2).  Selection flags go to sel_err.
+  // experts at rank r itself (one of them also into sel_u, sel_rho).  With
+  // `done` (zero before the pass), done[i] counts the blocks of expert tile i
+  // that finished, the tile's last one selects its q_hat, done[kMaxHistTiles]
+  // counts the tiles selected, and the last one forms b_next (Eq. 2).  Selection flags go to sel_err.
   const int32_t* coarse = nullptr;
   int32_t* done = nullptr;
   int32_t r = 0;
+  uint8_t* sel_u = nullptr;
+  int32_t* sel_rho = nullptr;
   uint16_t* q_hat = nullptr;
   float* b_next = nullptr;
   int32_t* sel_err = nullptr;
@@ -113,8 +115,8 @@ constexpr int64_t kLeiCoefCap = 65536;
 
 // The step's scratch, carved from one caller-provided buffer (256-byte
 // aligned pieces): the two [E,256] histograms and the fine pass's block
-// counters (adjacent, cleared together before every step), u and rho of the
-// separate selections, q_hat and the [M,E] LEI coefficient table.
+// counters (adjacent, cleared together before every step), u, rho, q_hat and
+// the [M,E] LEI coefficient table.
 struct StepWorkspace {
   int32_t* H;
   int32_t* L;

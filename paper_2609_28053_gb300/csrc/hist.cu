@@ -199,10 +199,14 @@ __global__ void __launch_bounds__(1024) hist_kernel(HistArgs a, int tiles, int t
     // Algorithm 1 step 3: every block selects u, rho for its own tile
     select_tile<true>(a.coarse, pl.e0, pl.e0 + pl.nct * 8, pl.nw, pl.wid, pl.lane, a.sel_err,
                       [&](int) { return a.r; },
-                      [&](int, int i, int bin, int32_t rest) {
+                      [&](int e, int i, int bin, int32_t rest) {
                         if (pl.lane == 0) {
                           su[i] = static_cast<uint8_t>(bin < 0 ? 255 : bin);
                           srho[i] = rest;
+                          if (pl.range == 0) {
+                            a.sel_u[e] = su[i];
+                            a.sel_rho[e] = rest;
+                          }
                         }
                       });
     sync_counting();

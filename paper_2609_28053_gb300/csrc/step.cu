@@ -126,6 +126,8 @@ eqb::HistArgs pass2_args(const Workspace& w, const eqb_bf16* z, const float* tau
   h.coarse = w.H;
   h.done = w.done;
   h.r = static_cast<int32_t>(r < INT32_MAX ? r : INT32_MAX);  // T < INT32_MAX: a larger rank is as unreachable
+  h.sel_u = w.u;
+  h.sel_rho = w.rho;
   h.q_hat = w.q;
   h.b_next = b_next;
   h.sel_err = err_flag;

@@ -59,3 +59,11 @@ def test_passes_and_step_match_oracle(T, E, K):
     torch.cuda.synchronize()
     assert bn.intact() and err.item() == 0
     assert np.array_equal(bits_f32(bn.view.cpu().numpy()), bits_f32(b_ref))
+    # what the step leaves in its workspace: H, L, 256 bytes of counters, u, rho
+    wb = ws.cpu().numpy()
+    at = 2 * E * 1024 + 256
+    assert np.array_equal(wb[:E * 1024].view(np.int32).reshape(E, 256), H_ref)
+    assert np.array_equal(wb[E * 1024:2 * E * 1024].view(np.int32).reshape(E, 256), L_ref)
+    assert np.array_equal(wb[at:at + E], u)
+    at += (E + 255) // 256 * 256
+    assert np.array_equal(wb[at:at + 4 * E].view(np.int32), rho)
