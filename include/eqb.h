@@ -213,13 +213,13 @@ size_t eqb_layer_workspace_bytes(int32_t E);
  * routing (Sec. 2), Algorithm 1's coarse pass, selection, fine pass,
  * selection, the Eq. (2) bias update, then Load-Error Injection (Sec. 4,
  * Eqs. LEI and norm) on grad_s when grad_s is given.  Results are identical
- * to the individual calls above.  When M * E <= 65,536 the LEI coefficients
- * are formed right after routing (lei_coefficients) and the injection is
- * streamed by the two histogram passes, half of the tokens each
- * (eqb_margin_hist_lei); otherwise LEI runs last (lei_inject_grad).  Each
- * histogram pass's selection (eqb_select_quantile; after the fine pass also
- * eqb_bias_update) runs in the pass's own last block to finish counting,
- * while the other blocks are still streaming LEI.
+ * to the individual calls above.  When M * E <= 65,536 the injection is
+ * streamed by the histogram passes (eqb_margin_hist_lei): all of it by the
+ * fine pass up to T E = 2^26, with the coefficients formed beside the coarse
+ * pass, half by each above, with the coefficients formed right after routing
+ * (lei_coefficients); otherwise LEI runs last (lei_inject_grad).  The
+ * selections (eqb_select_quantile) and eqb_bias_update run inside the fine
+ * pass.
  *   z, b, mb_offsets, M, topk_idx (nullable), tau, eta, c: as in
  *             eqb_route_topk / lei_inject_grad;
  *   mb_offsets_host host copy of mb_offsets (nullable; validated when given)

@@ -23,11 +23,11 @@ constexpr unsigned kFull = 0xffffffffu;
 // previous grid has completed and its writes are visible; a no-op for a grid
 // not launched as a dependent).  The implicit trigger at completion saves
 // 17 us on the global step against plain launches.  Only the short kernels
-// that precede a histogram pass (the LEI coefficient table, a selection)
-// trigger their successor early, at their start: the pass's blocks take the
-// SMs those leave idle and zero their bins meanwhile (1-3 us per step on
-// every workload).  Early triggers in every kernel cost 60 us on the global
-// step.
+// (the clearing and set-up kernels, the LEI coefficient table, a selection)
+// trigger their successor early, at their start: its blocks take the SMs
+// those leave idle and do their block-local set-up meanwhile (1-3 us per step
+// on every workload).  Early triggers in routing and the coarse pass cost
+// 11-32 us at 0.04-0.2 ms, in every kernel 60 us on the global step.
 __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // Let the next kernel in the stream launch now (it still waits, in
 // griddep_wait, for this grid to complete).
