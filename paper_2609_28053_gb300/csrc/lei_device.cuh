@@ -65,7 +65,7 @@ __device__ __forceinline__ void block_lei_coef(const int32_t* __restrict__ f, in
 #pragma unroll
   for (int k = 0; k < kPer; ++k) {
     const int e = threadIdx.x + k * NT;
-    if (e < E) out[e] = inv_fbar > 0.0 ? __double2float_rn(es * ((double)load[k] * inv_fbar - 1.0)) : 0.f;
+    if (e < E) out[e] = __double2float_rn(es * (inv_fbar > 0.0 ? (double)load[k] * inv_fbar - 1.0 : 0.0));
   }
   __syncthreads();
 }
@@ -94,7 +94,7 @@ __device__ __forceinline__ void warp_lei_coef(const int32_t* __restrict__ f, int
   const double es = (double)eta * (double)sigma;
 #pragma unroll 4
   for (int e = lane; e < E; e += 32)
-    out[e] = inv_fbar > 0.0 ? __double2float_rn(es * ((double)__ldg(f + e) * inv_fbar - 1.0)) : 0.f;
+    out[e] = __double2float_rn(es * (inv_fbar > 0.0 ? (double)__ldg(f + e) * inv_fbar - 1.0 : 0.0));
 }
 
 }  // namespace eqb
