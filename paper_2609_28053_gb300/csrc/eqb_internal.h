@@ -185,6 +185,10 @@ struct SplitRoute {
   int32_t* loads = nullptr;
 };
 int router_splits(int64_t T, int d, int sm_count);
+// Many experts, columns and tokens (router_pair.cu; E a multiple of 32, at
+// most 256): pairs of SMs.
+int launch_router_pair(const uint16_t* x, const uint16_t* W, int64_t T, int d, int E, uint16_t* z, int32_t* err,
+                       cudaStream_t s);
 int launch_router_split(const uint16_t* x, const uint16_t* W, int64_t T, int d, int E, int n, uint16_t* z,
                         const SplitRoute& ro, int32_t* err, cudaStream_t s);
 int launch_gshard(const GshardArgs& a, cudaStream_t s);

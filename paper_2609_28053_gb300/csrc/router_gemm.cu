@@ -429,6 +429,12 @@ int launch_router_gemm(const uint16_t* x, const uint16_t* W, int64_t T, int d, i
       return launch_router_split(x, W, T, d, E, n, z, none, err, s);
     }
   }
+  // Pairs of SMs (us, with routing after it, one SM a tile / pairs): T = 16,411,
+  // E = 256 18.4 / 19.4 at d = 1,024, 26.2 / 25.9 at 2,048, 44.8 / 38.4 at 4,096;
+  // T = 131,072 92.4 / 91.3, 143.7 / 130.9 and 262.4 / 218.7; T = 9,000, d =
+  // 2,048 22.5 / 23.4; d = 4,096, E = 224 38.5 / 38.3 and 224.2 / 213.4, E = 160
+  // 35.5 / 36.1 and 203.3 / 200.2.
+  if (E >= 224 && E % 32 == 0 && d >= 2048 && T >= 16384) return launch_router_pair(x, W, T, d, E, z, err, s);
   GemmArgs a{z, static_cast<int>(T), d, E, 0, err, nullptr, 0, nullptr, 0, nullptr, nullptr, nullptr, nullptr};
   return launch_gemm<0, 1, false>(x, W, a, s);
 }
