@@ -207,9 +207,9 @@ class Step:
         self.r_global = None
         self.off_h = even_offsets(T, self.M)
         self.workspace = torch.zeros(eqb.eqb_layer_workspace_bytes(E), dtype=torch.uint8, device=dev)
-        # The one-call step streams LEI inside the histogram passes when the
-        # [M,E] coefficient table fits its workspace (M * E <= 65,536), and
-        # selects inside the fine pass; the per-kernel breakdown issues the
+        # The one-call step streams LEI inside the fine pass when the [M,E]
+        # coefficient table, formed beside the coarse pass, fits its workspace
+        # (M * E <= 65,536), and selects inside the fine pass; the per-kernel breakdown issues the
         # same work through the separate entry points (the selections as
         # kernels of their own).
         self.fused = self.M * E <= 65536
@@ -217,13 +217,13 @@ class Step:
         if workload == "router":
             # projection, routing and the coarse histogram in one kernel; the
             # fine pass carries all of LEI
-            self.names = (["router_route", "lei_coefficients", "select_pass1", "margin_hist_lei_pass2",
+            self.names = (["router_route", "lei_coefficients", "select_pass1", "margin_hist_lei_all",
                            "select_pass2", "bias_update"] if self.fused else
                           ["router_route", "select_pass1", "margin_hist_pass2", "select_pass2", "bias_update",
                            "lei_inject_grad"])
         elif self.fused:
-            self.names = ["route_topk", "lei_coefficients", "margin_hist_lei_pass1", "select_pass1",
-                          "margin_hist_lei_pass2", "select_pass2", "bias_update"]
+            self.names = ["route_topk", "lei_coefficients", "margin_hist_pass1", "select_pass1",
+                          "margin_hist_lei_all", "select_pass2", "bias_update"]
         else:
             self.names = ["route_topk", "margin_hist_pass1", "select_pass1", "margin_hist_pass2",
                           "select_pass2", "bias_update", "lei_inject_grad"]
@@ -289,18 +289,14 @@ class Step:
         rec(0, lambda: eqb.eqb_route_topk(z, self.b, self.K, self.off, self.idx, self.tau,
                                           self.loads, None, ws.err, stream))
         if self.fused:
-            th = self.T // 2
             rec(1, lambda: eqb.lei_coefficients(self.loads, self.off, self.K, ETA, C_NORM, self.coef, stream))
-            rec(2, lambda: eqb.eqb_margin_hist_lei(z, self.tau, 1, ws.hist_hi, g, self.coef, self.off, 0, th,
-                                                   err_flag=ws.err, stream=stream))
-        else:
-            rec(1, lambda: eqb.eqb_margin_hist_pass1(z, self.tau, ws.hist_hi, ws.err, stream))
+        rec(2 if self.fused else 1, lambda: eqb.eqb_margin_hist_pass1(z, self.tau, ws.hist_hi, ws.err, stream))
         if world > 1:
             allreduce_(ws.hist_hi)
         k = 3 if self.fused else 2
         rec(k, lambda: eqb.eqb_select_quantile(ws.hist_hi, 1, r, ws.u, ws.rho, None, ws.err, stream))
         if self.fused:
-            rec(4, lambda: eqb.eqb_margin_hist_lei(z, self.tau, 2, ws.hist_lo, g, self.coef, self.off, th,
+            rec(4, lambda: eqb.eqb_margin_hist_lei(z, self.tau, 2, ws.hist_lo, g, self.coef, self.off, 0,
                                                    self.T, u=ws.u, stream=stream))
         else:
             rec(3, lambda: eqb.eqb_margin_hist_pass2(z, self.tau, ws.u, ws.hist_lo, stream))
@@ -320,12 +316,12 @@ class Step:
         the projection with routing and the coarse histogram) and the fine
         pass, which selects and updates the bias; the coarse pass unless the
         projection counted it; the LEI coefficient table unless the coarse
-        pass forms it (T E <= 2^26), or LEI itself where the table does not
-        fit the workspace."""
+        pass forms it, or LEI itself where the table does not fit the
+        workspace."""
         n = 3
         if self.workload != "router":
             n += 1
-        if not self.fused or self.workload == "router" or self.T * self.E > 1 << 26:
+        if not self.fused or self.workload == "router":
             n += 1
         return n
 
@@ -337,15 +333,12 @@ class Step:
         routing and the coarse histogram in its epilogue leaves only pass 2
         and LEI to read z.  Per kernel:"""
         T, E, K = self.T, self.E, self.K
-        th = T // 2
         d = {"route_topk": 2 * T * E + 4 * T * K + 4 * T,
              "margin_hist_pass1": 2 * T * E + 4 * T,
              "margin_hist_pass2": 2 * T * E + 4 * T,
              "lei_inject_grad": 8 * T * E,
-             # the fused passes: the pass's z and tau plus its share of grad
-             "margin_hist_lei_pass1": 2 * T * E + 4 * T + 8 * th * E,
-             "margin_hist_lei_pass2": (2 * T * E + 4 * T + 8 * T * E if self.workload == "router"
-                                       else 2 * T * E + 4 * T + 8 * (T - th) * E),
+             # the fine pass carrying LEI of every token
+             "margin_hist_lei_all": 2 * T * E + 4 * T + 8 * T * E,
              "path": 12 * T * E + 8 * T + 4 * T * K}
         if self.workload == "router":
             # the projection reads x and W_r and writes z; routing from its

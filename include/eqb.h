@@ -192,7 +192,7 @@ eqb_status lei_coefficients(const int32_t *loads, const int64_t *mb_offsets,
  * microbatch of t (Sec. 4, Eq. LEI).  The counting is issue-bound and the
  * injection DRAM-bound, so the two share the GPU better than back to back.
  * Results are bit-identical to the separate calls; the one-call step runs
- * pass 1 with the first half of the tokens and pass 2 with the rest.
+ * pass 2 with all of the tokens.
  *   grad_s  device fp32 [T,E], 16-byte aligned, updated in place on [lei_t0, lei_t1)
  *   coef    device fp32 [M,E] from lei_coefficients, 16-byte aligned
  *   0 <= lei_t0 <= lei_t1 <= T, else EQB_ERR_INVALID_ARG. */
@@ -214,12 +214,10 @@ size_t eqb_layer_workspace_bytes(int32_t E);
  * selection, the Eq. (2) bias update, then Load-Error Injection (Sec. 4,
  * Eqs. LEI and norm) on grad_s when grad_s is given.  Results are identical
  * to the individual calls above.  When M * E <= 65,536 the injection is
- * streamed by the histogram passes (eqb_margin_hist_lei): all of it by the
- * fine pass up to T E = 2^26, with the coefficients formed beside the coarse
- * pass, half by each above, with the coefficients formed right after routing
- * (lei_coefficients); otherwise LEI runs last (lei_inject_grad).  The
- * selections (eqb_select_quantile) and eqb_bias_update run inside the fine
- * pass.
+ * streamed by the fine pass (eqb_margin_hist_lei), with the coefficients
+ * formed beside the coarse pass; otherwise LEI runs last (lei_inject_grad).
+ * The selections (eqb_select_quantile) and eqb_bias_update run inside the
+ * fine pass.
  *   z, b, mb_offsets, M, topk_idx (nullable), tau, eta, c: as in
  *             eqb_route_topk / lei_inject_grad;
  *   mb_offsets_host host copy of mb_offsets (nullable; validated when given)

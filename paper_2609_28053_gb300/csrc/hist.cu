@@ -20,26 +20,34 @@
 // one z word share a word, the even one in the low half, so the increment is
 // a constant.  512 bytes per expert: 64 KiB for 128 experts.  Thread i owns
 // chunk i mod nct (8 experts) of token slot i / nct, so a warp reads
-// contiguous pieces of rows whatever the expert count; chunk c's rows start
-// c words past a 1 KiB boundary so equal bins of different chunks fall in
-// different banks.  Where a warp holds several tokens of a tile, the tile can
-// have as many copies of its bins (added at the flush).  A counter gains at
-// most one per token, so the CTA flushes (adds its non-zero counters into
+// contiguous pieces of rows whatever the expert count.
+// Two layouts.  Banked (BANK, from 5,000 chunks of z per SM on, passes 1 and
+// 3): 32 columns, a warp's lanes each in their own (chunk, and where the warp
+// holds several tokens of the tile, copy), the bank of every word of a column
+// the same, so no two lanes of an increment meet: word (bin * 4 + pair) * 32 +
+// column.  What bounds these passes otherwise is the banks in which random
+// bins meet: 2.8 to 3.7 clocks an increment of a warp, against 1.4 or less.
+// T = 2,097,152, E = 256 202 -> 160 us (the copy rate), T = 524,288, E = 128
+// 34 -> 26, T = 147,456, E = 256 21 -> 16.6; pass 3 260 -> 192 and 49 -> 40 (a
+// comparison).  It takes 128 KiB to zero and flush whatever the tile: small
+// batches, and pass 2, which counts few elements, use rows of 256 bins, chunk
+// c's c words past a 1 KiB boundary so equal bins of different chunks fall in
+// different banks.
+// A counter gains at most one per token, so the CTA flushes (adds its non-zero counters into
 // the global int32 [E,256] histogram) at least every 65,535 tokens; the
 // flush is also how token partitions are summed in device memory.
 // Each thread keeps several 16-byte loads in flight (kUnroll tokens per
 // round), which covers the DRAM latency without L2 prefetches.
 //
-// Fused with Load-Error Injection (the one-call step): the passes are bound
-// by issue, not by DRAM, while LEI (Sec. 4) is a pure DRAM stream that needs
-// only the loads.  A fused block gives some of its warps to streaming
+// Fused with Load-Error Injection (the one-call step): counting takes issue
+// slots beside DRAM, while LEI (Sec. 4) is a pure DRAM stream that needs only
+// the loads.  A fused block gives some of its warps to streaming
 // grad_s[t, e] += coef[mb(t), e] over its slice of a token range from the
 // start, the other warps count, and each counting warp joins the stream when
 // its counting is done; the stream is cut into chunks of about 8 KiB of
 // grad_s handed out by a shared counter, so no warp idles while the block
-// has work.  Each pass carries half of the step's tokens, which turns both
-// passes into DRAM-bound ones; where a pass is short, the fine pass carries
-// all of them and a few blocks of the coarse pass form the coefficients.
+// has work.  The step's fine pass carries all of the tokens, and a few blocks
+// of its coarse pass form the coefficients.
 #include "lei_device.cuh"
 #include "select_device.cuh"
 
@@ -47,8 +55,8 @@ namespace eqb {
 
 namespace {
 
-// 16-byte loads in flight per thread (64 registers at 1024 threads).  Pass 1 /
-// pass 2 alone at T = 2,097,152, E = 256: 187 / 171 us with six, 185 / 185
+// 16-byte loads in flight per thread (64 registers at 1024 threads).  Pass 1
+// (before its banked bins) / pass 2 alone at T = 2,097,152, E = 256: 187 / 171 us with six, 185 / 185
 // with seven, 194 / 184 with eight, 221 / 181 with four.  Beside the injection
 // eight (the step at T = 1,048,576, E = 512 1229 us, 1241 with six).
 template <bool LEI>
@@ -113,6 +121,8 @@ __device__ __forceinline__ void select_tile(const int32_t* hist, int ea, int eb,
 __device__ __forceinline__ int row_word(int row) { return row * 256 + (row >> 2); }
 // Words of the bins of nct chunks, a multiple of four.
 __host__ __device__ constexpr int bin_words(int nct) { return (nct * 1024 + nct + 3) & ~3; }
+// The banked bins: (slot * 4 + pair) * 32 + column.
+constexpr int kBankWords = 256 * 4 * 32;
 // Widest tile of a block, in 8-expert chunks.
 constexpr int kMaxTileChunks = 16;
 static_assert(kMaxE / 64 <= kMaxHistTiles, "tiles of 8 chunks or more");
@@ -140,7 +150,7 @@ struct HistPlace {
   }
 };
 
-template <int PASS, bool LEI>
+template <int PASS, bool LEI, bool BANK>
 __global__ void __launch_bounds__(1024) hist_kernel(HistArgs a, int tiles, int tile_chunks, int copies,
                                                     int64_t tokens_per_cta, LeiStream ls, CoefRows cr) {
   constexpr int U = kUnroll<LEI>;
@@ -170,13 +180,15 @@ __global__ void __launch_bounds__(1024) hist_kernel(HistArgs a, int tiles, int t
     else __syncthreads();
   };
 
-  const int ncp = PASS == 2 ? 1 : copies;
-  for (int i = threadIdx.x; i < bin_words(pl.nct * ncp) / 4; i += blockDim.x)
+  for (int i = threadIdx.x; i < (BANK ? kBankWords : bin_words(pl.nct)) / 4; i += blockDim.x)
     reinterpret_cast<uint4*>(bins)[i] = make_uint4(0u, 0u, 0u, 0u);
   if (LEI && threadIdx.x == 0) lei_next = 0;
-  // Shared address of this thread's first pair row; pair p adds p * 1 KiB.
+  // Shared address of this thread's bin 0 of its first pair; pair p adds
+  // p * kPairBytes, bin j j << kBinShift.
+  constexpr uint32_t kPairBytes = BANK ? 128u : 1024u;
+  constexpr int kBinShift = BANK ? 9 : 2;
   const uint32_t base = static_cast<uint32_t>(__cvta_generic_to_shared(bins)) +
-                        4u * static_cast<uint32_t>(row_word(4 * (ncp > 1 ? c + tok % ncp * pl.nct : c)));
+                        4u * static_cast<uint32_t>(BANK ? c + tok % copies * pl.nct : row_word(4 * c));
   uint32_t sel[4] = {0, 0, 0, 0};
   // internal high bytes (u ^ 0x80) of the selected bins, placed where the
   // internal keys carry them: bits 8-15 (even expert) and 24-31 (odd).
@@ -226,19 +238,29 @@ __global__ void __launch_bounds__(1024) hist_kernel(HistArgs a, int tiles, int t
     for (int p = 0; p < 4; ++p) {
       const uint32_t m = margins_bf16x2(tt, zw[p]);
       const uint32_t k = kappa2_internal(m);
-      const uint32_t row = base + 1024u * p;
+      const uint32_t row = base + kPairBytes * p;
       if (PASS == 1) {
         const uint32_t he = prmt(k, 0u, 0x4441u), ho = k >> 24;  // internal high bytes
-        const bool same = he == ho;
-        red_shared_add(row + 4u * he, same ? 0x10001u : 1u);
-        if (!same) red_shared_add(row + 4u * ho, 0x10000u);
+        if (BANK) {
+          red_shared_add(row + (he << kBinShift), 1u);
+          red_shared_add(row + (ho << kBinShift), 0x10000u);
+        } else {
+          const bool same = he == ho;
+          red_shared_add(row + (he << kBinShift), same ? 0x10001u : 1u);
+          if (!same) red_shared_add(row + (ho << kBinShift), 0x10000u);
+        }
       } else if (PASS == 3) {
         // equal-width bins: j = floor((m - lo) * inv_w), clamped to [0, 255]
         const uint32_t he = static_cast<uint32_t>(min(max(__float2int_rd(__fmul_rn(__fsub_rn(bf16_lo(m), a.lo), a.inv_w)), 0), 255));
         const uint32_t ho = static_cast<uint32_t>(min(max(__float2int_rd(__fmul_rn(__fsub_rn(bf16_hi(m), a.lo), a.inv_w)), 0), 255));
-        const bool same = he == ho;
-        red_shared_add(row + 4u * he, same ? 0x10001u : 1u);
-        if (!same) red_shared_add(row + 4u * ho, 0x10000u);
+        if (BANK) {
+          red_shared_add(row + (he << kBinShift), 1u);
+          red_shared_add(row + (ho << kBinShift), 0x10000u);
+        } else {
+          const bool same = he == ho;
+          red_shared_add(row + (he << kBinShift), same ? 0x10001u : 1u);
+          if (!same) red_shared_add(row + (ho << kBinShift), 0x10000u);
+        }
       } else {
         const uint32_t d = (k ^ sel[p]) & 0xff00ff00u;
         if ((d & 0x0000ff00u) == 0u) red_shared_add(row + 4u * (k & 0xffu), 1u);
@@ -287,23 +309,49 @@ __global__ void __launch_bounds__(1024) hist_kernel(HistArgs a, int tiles, int t
     const HistPlace fl(tiles, tile_chunks, E, LEI ? ls.warps : 0);
     sync_counting();
     // Flush: add every non-zero 16-bit counter to the global histogram.
-    for (int i = fl.tid; i < fl.nct * 1024; i += fl.nt) {
-      const int row = i >> 8, slot = i & 255;
-      const int wi = row_word(row) + slot;
-      uint32_t v = bins[wi];
-      if (v) bins[wi] = 0u;
-      for (int k = 1; k < ncp; ++k) {  // the copies' halves add up to at most the tokens counted
-        const int wk = row_word(row + 4 * k * fl.nct) + slot;
-        const uint32_t vk = bins[wk];
-        if (vk) bins[wk] = 0u;
-        v += vk;
+    auto add = [&](uint32_t v, int row, int slot) {
+      const int bin = (PASS == 1) ? (slot ^ 0x80) : slot;  // pass 1 stores internal keys
+      const int ee = fl.e0 + 2 * row;
+      if (v & 0xffffu) atomicAdd(a.hist + hbase + (int64_t)ee * 256 + bin, static_cast<int>(v & 0xffffu));
+      if (v >> 16) atomicAdd(a.hist + hbase + (int64_t)(ee + 1) * 256 + bin, static_cast<int>(v >> 16));
+      if (PASS == 1 && (bin == 0 || bin == 255)) raise_flag(a.err, kErrNonfinite);
+    };
+    if constexpr (BANK) {
+      // A warp takes 32 slots of one pair: read with a lane per column, turned
+      // in place (element (slot, column) to row `column`), read back with a lane
+      // per slot, so that neither the reads meet in a bank nor the global
+      // additions of a warp scatter.
+#pragma unroll 1
+      for (int blk = fl.wid; blk < 32; blk += fl.nw) {
+        uint32_t* const w = bins + (blk >> 2) * 4096 + (blk & 3) * 32;  // 32 rows, 128 words apart
+        uint32_t v[32], some = 0;
+#pragma unroll
+        for (int j = 0; j < 32; ++j) {
+          v[j] = w[j * 128 + fl.lane];
+          some |= v[j];
+        }
+        if (!__any_sync(kFull, some != 0u)) continue;  // (every lane has read)
+#pragma unroll
+        for (int j = 0; j < 32; ++j) w[fl.lane * 128 + ((j + fl.lane) & 31)] = v[j];
+        __syncwarp();
+        for (int ch = 0; ch < fl.nct; ++ch) {
+          uint32_t sum = 0;  // the copies' halves add up to at most the tokens counted
+          for (int r = ch; r < fl.nct * copies; r += fl.nct) sum += w[r * 128 + ((fl.lane + r) & 31)];
+          if (sum) add(sum, 4 * ch + (blk & 3), (blk >> 2) * 32 + fl.lane);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < 32; ++j) w[j * 128 + fl.lane] = 0u;
       }
-      if (v) {
-        const int bin = (PASS == 1) ? (slot ^ 0x80) : slot;  // pass 1 stores internal keys
-        const int ee = fl.e0 + 2 * row;
-        if (v & 0xffffu) atomicAdd(a.hist + hbase + (int64_t)ee * 256 + bin, static_cast<int>(v & 0xffffu));
-        if (v >> 16) atomicAdd(a.hist + hbase + (int64_t)(ee + 1) * 256 + bin, static_cast<int>(v >> 16));
-        if (PASS == 1 && (bin == 0 || bin == 255)) raise_flag(a.err, kErrNonfinite);
+    } else {
+      for (int i = fl.tid; i < fl.nct * 1024; i += fl.nt) {
+        const int row = i >> 8, slot = i & 255;
+        const int wi = row_word(row) + slot;
+        const uint32_t v = bins[wi];
+        if (v) {
+          bins[wi] = 0u;
+          add(v, row, slot);
+        }
       }
     }
     sync_counting();
@@ -342,8 +390,8 @@ __global__ void __launch_bounds__(1024) hist_kernel(HistArgs a, int tiles, int t
 }
 
 // How a pass is cut into blocks: expert tiles of `chunks` 8-expert chunks
-// times token ranges of `tpc` tokens, about one block per SM, each with
-// `copies` copies of its tile's bins.
+// times token ranges of `tpc` tokens, about one block per SM, with `copies`
+// columns for each chunk of the banked layout (1: rows of bins).
 struct HistCut {
   int tiles, chunks, copies, ranges;
   int64_t tpc;
@@ -357,13 +405,15 @@ struct HistCut {
 // 12.0 / 8.2 / 74 (one 32-chunk tile on 2,048-token blocks before: 33.5 /
 // 27.1 / 93); T = 147,456 (31,000) 27 / 15 / 81, 21 / 16 / 76 and 22 / 17 /
 // 89; T = 1,048,576, E = 384 143 / 134 / 462 for 16, 162 / 136 / 487 for 24.
-// From 7,000 chunks per SM on, copies that give the 32 lanes of a warp bins
-// of their own pay for their zeroing: T = 1,000,000, E = 64 31 us against
-// 45 (pass 1), T = 60,000, E = 160 10.3 against 12.1; T = 65,536, E = 64
-// (3,400) 7.5 against 6.8.  Pass 2 counts few elements, so that its lanes
-// rarely meet: one copy, and narrower tiles, whose selections take one round
-// of the block's warps and whose flushes (nearly every low byte occurs) add
-// fewer counters to the global histogram.  The step with tiles of 4, 8 and 16
+// From 5,000 chunks per SM on the banked layout, `copies` columns a chunk,
+// pays for its zeroing and flush: the step at T = 30,873, E = 256 36.5 -> 35.6
+// us, T = 40,000, E = 96 (3,200) 29.5 against 29.9 with it.  Tiles of 32
+// chunks with it: pass 1 at T = 147,456, E = 256 18.3 us against 16.6, T =
+// 524,288 48.5 against 45.7, T = 2,097,152 159.9 against 159.7.  Pass 2 counts
+// few elements, so that its lanes rarely meet: rows of bins, and narrower
+// tiles, whose selections take one round of the block's warps and whose
+// flushes (nearly every low byte occurs) add fewer counters to the global
+// histogram.  The step with tiles of 4, 8 and 16
 // chunks: T = 30,873, E = 256 35 / 37 / 42 us, T = 65,536, E = 64 31 / 35 /
 // 35, T = 524,288, E = 128 185 / 187 / 190, E = 256 321 / 321 / 325, T =
 // 1,048,576, E = 512 1220 / 1219 / 1211.
@@ -379,7 +429,7 @@ HistCut cut_hist(int64_t T, int E, int pass, int blocks) {
   h.tiles = (nch + want - 1) / want;
   h.chunks = (nch + h.tiles - 1) / h.tiles;
   h.tiles = (nch + h.chunks - 1) / h.chunks;
-  h.copies = pass != 2 && per_sm >= 7000 ? 32 / h.chunks : 1;
+  h.copies = pass != 2 && per_sm >= 5000 ? 32 / h.chunks : 1;
   int64_t ranges = blocks / h.tiles;
   const int64_t most = (T * h.chunks + 1023) / 1024;  // a chunk for every thread
   if (ranges > most) ranges = most;
@@ -403,8 +453,10 @@ int launch_hist_pass(const HistArgs& a, const LeiStream& ls, CoefRows cr, cudaSt
   if (int rc = device_info(&di)) return rc;
   cr.blocks = cr.coef ? coef_blocks(a.T, a.E, cr.a.M, di.sm_count) : 0;
   const HistCut h = cut_hist(a.T, a.E, PASS, di.sm_count - cr.blocks);
-  const int smem = bin_words(h.chunks * h.copies) * 4;
-  auto kern = hist_kernel<PASS, LEI>;
+  const int smem = (h.copies > 1 ? kBankWords : bin_words(h.chunks)) * 4;
+  auto kern = hist_kernel<PASS, LEI, false>;
+  if constexpr (PASS != 2)
+    if (h.copies > 1) kern = hist_kernel<PASS, LEI, true>;
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
     return kErrCuda;
   return launch_dependent(kern, dim3((unsigned)(h.tiles * h.ranges + cr.blocks)), dim3(1024), smem, s, a, h.tiles,
@@ -431,12 +483,12 @@ int launch_hist_lei(const HistArgs& a, int pass, const LeiStream& lei, cudaStrea
   LeiStream ls = lei;
   // of 32: the passes are DRAM-bound, and the more warps stream from the start
   // the sooner they are, until counting is what takes longest.  A pass that
-  // carries every token, 8 / 14 / 16 / 18 / 20 / 24: T = 524,288, E = 128 184 /
-  // 182 / 180 / 182 / 182 / 198 us a step, T = 65,536, E = 64 31.4 / 31.2 /
-  // 31.0 / 34.1 / 32.9 / 34.7; half of them each, 8 / 12 / 13 / 14 / 16: T =
-  // 2,097,152, E = 256 1198 / 1180 / 1177 / 1175 / 1191, T = 1,048,576, E =
-  // 512 1209 / 1191 / 1188 / 1185 / 1199.
-  ls.warps = ls.t1 - ls.t0 == a.T ? 16 : 14;
+  // carries every token, 14 / 16 / 18 / 20: T = 65,536, E = 64 30.9 / 31.1 /
+  // 33.9 / 32.7 us a step, T = 200,003, E = 96 72.2 / 71.5 / 71.9 / 71.7, T =
+  // 524,288, E = 256 311.6 / 311.2 / 310.3 / 308.9, T = 2,097,152 1168.7 /
+  // 1166.8 / 1166.1 / 1165.9; half of them each, 8 / 12 / 14 / 16: T =
+  // 2,097,152, E = 256 1198 / 1180 / 1175 / 1191.
+  ls.warps = ls.t1 - ls.t0 < a.T ? 14 : a.T * a.E > int64_t(1) << 26 ? 20 : 16;
   if (!ls.g || !ls.coef || !ls.off || ls.M < 1 || ls.t0 < 0 || ls.t1 < ls.t0) return kErrInvalidArg;
   return pass == 1 ? launch_hist_pass<1, true>(a, ls, CoefRows(), s) : launch_hist_pass<2, true>(a, ls, CoefRows(), s);
 }

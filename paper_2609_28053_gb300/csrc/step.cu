@@ -5,8 +5,8 @@
 // pass, selection, fine pass, selection and the Eq. (2) bias update, and
 // Load-Error Injection (Sec. 4, Eqs. LEI and norm).  LEI needs only the
 // loads, so when its [M,E] coefficient table fits the workspace the
-// coefficients are formed before or beside the coarse pass and the passes
-// stream the injection; otherwise it runs last.  All on one stream.
+// coefficients are formed beside the coarse pass and the fine pass streams
+// the injection; otherwise it runs last.  All on one stream.
 // eqb_router_layer_step starts one step earlier, at the router projection
 // (Eq. 1), and routes from the projection's accumulators where it can; that
 // kernel also counts the coarse histogram, so the fine pass alone reads z
@@ -136,13 +136,13 @@ eqb::HistArgs pass2_args(const Workspace& w, const eqb_bf16* z, const float* tau
 
 // Everything after routing: Algorithm 1's two passes with their selections,
 // the Eq. (2) bias update and LEI.  When the [M,E] coefficient table fits the
-// workspace, the passes stream the injection beside their counting (they are
-// issue-bound, it is DRAM-bound); the results are the same bits as the
-// separate LEI launch.  Up to 2^26 logits blocks of the coarse pass form the
-// table and the fine pass carries all of the injection, which spares a launch
-// (T = 65,536, E = 64 49 -> 39 us, T = 147,456, E = 256 118 -> 115); beyond,
-// each pass carries half of it (T = 2,097,152, E = 256 1196 us against 1222,
-// T = 524,288, E = 256 332 against 332).
+// workspace, blocks of the coarse pass form it and the fine pass streams all
+// of the injection beside its counting (the same bits as the separate LEI
+// launch): the coarse pass alone runs at the copy rate, so it has no time to
+// give, and the table needs no launch of its own.  Half of the injection in
+// each pass, with the table formed before them, against this: T = 65,536, E =
+// 64 49 / 39 us, T = 147,456, E = 256 118 / 115, T = 524,288, E = 256 310 / 309,
+// T = 2,097,152, E = 256 1183 / 1166.
 eqb_status after_routing(const Workspace& w, const eqb_bf16* z, int64_t T, int32_t E, int32_t K,
                          const int64_t* mb_offsets, int32_t M, int64_t r, const float* tau,
                          const int32_t* loads, float* b_next, float* grad_s, float eta, float c,
@@ -151,15 +151,8 @@ eqb_status after_routing(const Workspace& w, const eqb_bf16* z, int64_t T, int32
   const eqb::HistArgs h2 = pass2_args(w, z, tau, T, E, r, b_next, err_flag);
   if (grad_s && static_cast<int64_t>(M) * E <= eqb::kLeiCoefCap) {
     eqb::LeiArgs la{grad_s, loads, mb_offsets, M, 0, T, E, K, eta, c};
-    const int64_t th = T * E <= int64_t(1) << 26 ? 0 : T / 2;  // tokens carried by pass 1
-    if (th == 0) {
-      if (int rc = eqb::launch_hist_coef(h1, la, w.coef, s)) return st(rc);
-    } else {
-      if (int rc = eqb::launch_lei_coef(la, w.coef, s)) return st(rc);
-      eqb::LeiStream l1{grad_s, w.coef, mb_offsets, M, 0, th};
-      if (int rc = eqb::launch_hist_lei(h1, 1, l1, s)) return st(rc);
-    }
-    eqb::LeiStream l2{grad_s, w.coef, mb_offsets, M, th, T};
+    if (int rc = eqb::launch_hist_coef(h1, la, w.coef, s)) return st(rc);
+    eqb::LeiStream l2{grad_s, w.coef, mb_offsets, M, 0, T};
     if (int rc = eqb::launch_hist_lei(h2, 2, l2, s)) return st(rc);
     return EQB_OK;
   }

@@ -1,7 +1,7 @@
 """GPU parity of the histogram passes at the edges of how they are cut into
 blocks: expert counts whose last tile is narrower than the others or whose
 tokens straddle warps, and token counts on both sides of the lines between
-tiles of 8 and 16 chunks and between one copy of the bins and several.
+tiles of 8 and 16 chunks and between rows of bins and bins banked by lane.
 Counts are whole numbers: every bin equals the oracle's."""
 import numpy as np
 import pytest
@@ -14,16 +14,18 @@ from gpu_harness import Guarded, bits_f32, to_dev_bf16
 
 pytestmark = pytest.mark.gpu
 
-# Chunks of z per SM (T E / 8 / 152): the lines lie at 7,000 (copies) and
+# Chunks of z per SM (T E / 8 / 152): the lines lie at 5,000 (banked bins) and
 # 10,000 (16-chunk tiles).
 CUTS = [(1, 8, 2),           # one thread's work
         (130, 264, 8),       # 33 chunks in tiles of 7, the last of 5
         (5000, 104, 3),      # 13 chunks: 7 and 6
-        (35000, 264, 8),     # 7,598: copies of tiles of 7 and 5 chunks
+        (23500, 256, 4),     # 4,947: rows
+        (24500, 264, 4),     # 5,319: banked, tiles of 7 and 5 chunks
+        (35000, 264, 8),     # 7,598
         (47000, 264, 4),     # 10,203: tiles of 11
-        (32000, 392, 8),     # 10,315: 13, 13, 13 and 10 chunks, two copies
-        (200000, 64, 8),     # 10,526: one 8-chunk tile, four copies
-        (1600000, 8, 2)]     # 10,526: one chunk, 32 copies
+        (32000, 392, 8),     # 10,315: 13, 13, 13 and 10 chunks, two columns each
+        (200000, 64, 8),     # 10,526: one 8-chunk tile, four columns each
+        (1600000, 8, 2)]     # 10,526: one chunk, 32 columns
 
 
 @pytest.fixture(scope="module", autouse=True)
