@@ -52,11 +52,17 @@ def test_passes_and_step_match_oracle(T, E, K):
     assert H.intact() and L.intact() and err.item() == 0
     assert np.array_equal(H.view.cpu().numpy(), H_ref)
     assert np.array_equal(L.view.cpu().numpy(), L_ref)
+    # pass 1 beside an injection of half of the tokens: the same counts
+    H2, g = Guarded((E, 256), torch.int32), torch.zeros((T, E), device="cuda")
+    off, coef = torch.tensor([0, T], device="cuda"), torch.rand((1, E), device="cuda")
+    eqb.eqb_margin_hist_lei(zd, td, 1, H2.view, g, coef, off, 0, (T + 1) // 2)
+    torch.cuda.synchronize()
+    assert H2.intact() and np.array_equal(H2.view.cpu().numpy(), H_ref)
+    assert torch.equal(g[:(T + 1) // 2], coef.expand((T + 1) // 2, E)) and not g[(T + 1) // 2:].any()
     # the one-call step, whose fine pass selects by tiles
     loads = torch.zeros((1, E), dtype=torch.int32, device="cuda")
     bn = Guarded((E,), torch.float32)
     ws = torch.full((eqb.eqb_layer_workspace_bytes(E),), 0x5a, dtype=torch.uint8, device="cuda")
-    off = torch.tensor([0, T], device="cuda")
     eqb.eqb_layer_step(zd, torch.from_numpy(b).cuda(), K, off, loads, bn.view, ws, err_flag=err)
     torch.cuda.synchronize()
     assert bn.intact() and err.item() == 0
