@@ -392,8 +392,9 @@ eqb_status eqb_router_route(const eqb_bf16 *x, const eqb_bf16 *W_r, int64_t T, i
  * eqb_layer_step, and so are the arguments from b on; z is an output here
  * (device bf16 [T,E], 16-byte aligned).
  *   x, W_r, d   as in eqb_router_logits.
- * Returns EQB_ERR_UNSUPPORTED for d not a multiple of 64 or E not a
- * multiple of 16, beside eqb_layer_step's own conditions. */
+ * Returns EQB_ERR_UNSUPPORTED for d not a multiple of 64, E not a multiple
+ * of 16 or E > 256 (the projection's limits), beside eqb_layer_step's own
+ * conditions. */
 eqb_status eqb_router_layer_step(const eqb_bf16 *x, const eqb_bf16 *W_r, int64_t T, int32_t d,
                                  int32_t E, int32_t K, const float *b,
                                  const int64_t *mb_offsets, const int64_t *mb_offsets_host,

@@ -421,6 +421,8 @@ int launch_gemm(const uint16_t* x, const uint16_t* W, GemmArgs a, cudaStream_t s
 
 int launch_router_gemm(const uint16_t* x, const uint16_t* W, int64_t T, int d, int E, uint16_t* z,
                        int32_t* err, bool split, cudaStream_t s) {
+  // one UMMA N, two accumulators of E columns in tensor memory
+  if (E > 256 || E % 16 != 0) return kErrUnsupported;
   if (split) {
     DeviceInfo di;
     if (int rc = device_info(&di)) return rc;

@@ -242,6 +242,7 @@ __global__ void __launch_bounds__(192, 1)
 
 int launch_router_pair(const uint16_t* x, const uint16_t* W, int64_t T, int d, int E, uint16_t* z, int32_t* err,
                        cudaStream_t s) {
+  if (E > 256 || E % 32 != 0) return kErrUnsupported;  // one UMMA N over two SMs, two accumulators
   DeviceInfo di;
   if (int rc = device_info(&di)) return rc;
   CUtensorMap tmx, tmw;

@@ -219,7 +219,7 @@ eqb_status eqb_router_layer_step(const eqb_bf16* x, const eqb_bf16* W_r, int64_t
                                  float* grad_s, float eta, float c, void* workspace,
                                  size_t workspace_bytes, int32_t* err_flag, void* stream) {
   if (!x || !W_r || d < 1) return EQB_ERR_INVALID_ARG;
-  if ((d % 64) != 0 || (E % 16) != 0) return EQB_ERR_UNSUPPORTED;
+  if ((d % 64) != 0 || (E % 16) != 0 || E > 256) return EQB_ERR_UNSUPPORTED;
   if (!aligned(x, 16) || !aligned(W_r, 16)) return EQB_ERR_INVALID_ARG;
   Workspace w;
   eqb_status rs = check_step(z, b, T, E, K, mb_offsets, mb_offsets_host, M, topk_idx, tau, loads, b_next,

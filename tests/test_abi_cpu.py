@@ -239,6 +239,7 @@ def test_router_layer_step_rejects(lib):
     import numpy as np
     f = lib.eqb_router_layer_step
     ws = lib.eqb_layer_workspace_bytes(128)
+    wide = lib.eqb_layer_workspace_bytes(1024)
     good = np.array([0, 40, 100], np.int64)
     bad = np.array([0, 60, 50], np.int64)
     fl = ctypes.c_float(0.0)
@@ -251,6 +252,10 @@ def test_router_layer_step_rejects(lib):
     assert call(x=MISALIGNED) == INVALID
     assert call(d=4000) == UNSUPPORTED         # d not a multiple of 64
     assert call(E=72) == UNSUPPORTED           # E not a multiple of 16
+    # more experts than one projection holds, also where pairs of SMs would be chosen
+    assert call(E=272, ws_bytes=wide) == UNSUPPORTED
+    assert call(E=512, T=20000, off_h=None, ws_bytes=wide) == UNSUPPORTED
+    assert call(E=1024, ws_bytes=wide) == UNSUPPORTED
     assert call(off_h=bad) == INVALID
     assert call(ws_bytes=ws - 1) == INVALID
     assert call(z=NULL) == INVALID
