@@ -181,14 +181,20 @@ __device__ __forceinline__ uint32_t kappa2_internal(uint32_t m) {
   return m ^ (sm & 0x7fff7fffu);
 }
 
-// bf16 pattern of fp32 x rounded toward -inf / +inf (exact values kept).
+// bf16 pattern of fp32 x rounded toward -inf / +inf (exact values kept).  A
+// NaN stays one (its payload can lie in the dropped bits alone, which would
+// leave an infinity): routing's bounds rely on it to keep an expert with a NaN
+// bias off the candidate list, where a NaN score would let the -inf experts
+// of a padded row be listed after it.
 __device__ __forceinline__ uint32_t bf16_round_down(float x) {
+  if (x != x) return 0x7fc0u;
   const uint32_t u = __float_as_uint(x);
   const uint32_t hi = u >> 16;
   if ((u & 0xffffu) == 0u) return hi;
   return (u & 0x80000000u) ? hi + 1u : hi;
 }
 __device__ __forceinline__ uint32_t bf16_round_up(float x) {
+  if (x != x) return 0x7fc0u;
   const uint32_t u = __float_as_uint(x);
   const uint32_t hi = u >> 16;
   if ((u & 0xffffu) == 0u) return hi;

@@ -74,6 +74,30 @@ def test_equal_scores(E, K, kind):
         check(brute.bf16_bits_from_f32(z), b, K, 2, seed=E)
 
 
+@pytest.mark.parametrize("E,K", [(8, 7), (24, 15), (136, 15), (200, 4)])
+@pytest.mark.parametrize("pattern", [0xff800001, 0x7f800001, 0xffffffff])
+def test_nan_bias_of_a_padded_row(E, K, pattern):
+    """A NaN bias whose payload lies in the bits that bf16 drops, on a row
+    padded to a wider kernel, with more list entries than groups of finite
+    experts: the call is flagged, and no expert past E is listed or counted
+    (tokens of the last microbatch inside a tile of the one before)."""
+    T = 32 * E + 70
+    rng = np.random.default_rng(E)
+    z = brute.bf16_bits_from_f32(rng.standard_normal((T, E), dtype=np.float32))
+    z[:, K // 2 + 1:E - 1] = 0xff80  # -inf: no more than K finite scores
+    b = np.zeros(E, np.float32)
+    b.view(np.uint32)[E - 1] = pattern
+    off = torch.tensor([0, T - 45, T - 13, T], device="cuda")
+    idx, tau, loads = Guarded((T, K), torch.int32, fill=-7), Guarded((T,), torch.float32), Guarded((3, E), torch.int32)
+    err = torch.zeros(1, dtype=torch.int32, device="cuda")
+    eqb.eqb_route_topk(to_dev_bf16(z), torch.from_numpy(b).cuda(), K, off, idx.view, tau.view, loads.view, err_flag=err)
+    torch.cuda.synchronize()
+    assert err.item() == 4  # EQB_ERR_NONFINITE
+    assert idx.intact() and tau.intact() and loads.intact()
+    assert int(idx.view.min()) >= 0 and int(idx.view.max()) < E
+    assert torch.equal(loads.view.sum(dim=1).cpu(), K * (off[1:] - off[:-1]).cpu().to(torch.int32))
+
+
 def test_microbatches_of_a_warp():
     """More boundaries than a warp loads at once, most of them equal, and
     enough tokens of a wide row for the loads to be counted by segments."""
