@@ -22,8 +22,9 @@
 //
 // Every wait is bounded: a wait that runs out sets a shared abort flag that
 // makes all roles leave their loops, the MMA thread drains its outstanding
-// tensor-core work through one more commit, TMEM is freed, and the kernel
-// reports EQB_ERR_CUDA through the error word.
+// tensor-core work through one more commit, TMEM is freed, the tile loads in
+// flight are waited for (bounded again), and the kernel reports EQB_ERR_CUDA
+// through the error word.
 //
 // Launched as a dependent of the previous kernel: barriers, tensor memory and
 // shared counters are set up while that one drains (16,411 tokens, d = 2,048,
@@ -184,6 +185,7 @@ __global__ void __launch_bounds__(192, 1)
   uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(sm + static_cast<size_t>(S) * stage_bytes +
                                                       8u * (2 * S + 5));
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
+  int* issued = reinterpret_cast<int*>(tmem_holder + 2);  // the producer's loads, for the drain after an abort
   // routing only: b (EC floats), then 4 warps x EC/2 packed load counters
   float* bsm = reinterpret_cast<float*>(tmem_holder + 4);
   uint32_t* lcnt = reinterpret_cast<uint32_t*>(bsm + EC);
@@ -236,11 +238,11 @@ __global__ void __launch_bounds__(192, 1)
     if (lane == 0) {
       asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmx)) : "memory");
       asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmw)) : "memory");
-      int stage = 0;
+      int stage = 0, n = 0;
       uint32_t phase = 0;
       bool ok = true;
       for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
-        for (int kb = 0; kb < KB; ++kb) {
+        for (int kb = 0; kb < KB; ++kb, ++n) {
           if (!mbar_wait(empty(stage), phase ^ 1u, abort_flag)) { ok = false; break; }
           const uint32_t dst = base + static_cast<uint32_t>(stage) * stage_bytes;
           mbar_expect_tx(full(stage), stage_bytes);
@@ -249,6 +251,7 @@ __global__ void __launch_bounds__(192, 1)
           if (++stage == S) { stage = 0; phase ^= 1u; }
         }
       }
+      *issued = n;
     }
   } else if (warp == 1) {
     if (lane == 0) {
@@ -387,7 +390,10 @@ __global__ void __launch_bounds__(192, 1)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols)
                  : "memory");
   }
-  if (threadIdx.x == 0 && *abort_flag) raise_flag(err, kErrCuda);
+  if (threadIdx.x == 0 && *abort_flag) {
+    drain_loads(*issued, S, full);
+    raise_flag(err, kErrCuda);
+  }
 }
 
 template <int EC, int KP1, bool HIST>

@@ -20,7 +20,10 @@
 // 0.39 against 0.58 (130, x from DRAM).  z is the same bit for bit.
 //
 // Every wait is bounded as in router_gemm.cu, and every thread reaches both
-// cluster barriers whether or not a wait ran out.
+// cluster barriers whether or not a wait ran out.  After one that did, each
+// block's producer waits (bounded again) for its loads in flight before the
+// last of them: block 0 on the barriers that they complete on, block 1, which
+// cannot poll those, for the MMAs that read its stages.
 #include "tcgen05.cuh"
 
 namespace eqb {
@@ -145,11 +148,11 @@ __global__ void __launch_bounds__(192, 1)
 
   if (warp == 0) {
     if (lane == 0) {
-      int stage = 0;
+      int stage = 0, issued = 0;
       uint32_t phase = 0;
       bool ok = true;
       for (int p = first; p < pairs && ok; p += step) {
-        for (int kb = 0; kb < KB; ++kb) {
+        for (int kb = 0; kb < KB; ++kb, ++issued) {
           if (!mbar_wait(empty(stage), phase ^ 1u, abort_flag)) { ok = false; break; }
           const uint32_t dst = base + static_cast<uint32_t>(stage) * stage_bytes;
           if (rank == 0) mbar_expect_tx(full(stage), 2u * stage_bytes);  // both blocks' loads
@@ -163,6 +166,10 @@ __global__ void __launch_bounds__(192, 1)
       for (int s = 0; s < S && ok; ++s) {
         ok = mbar_wait(empty(stage), phase ^ 1u, abort_flag);
         if (++stage == S) { stage = 0; phase ^= 1u; }
+      }
+      if (!ok) {
+        if (rank == 0) drain_loads(issued, S, full);
+        else drain_loads(issued, S, empty);  // MMA i's commit is phase i / S of its stage's `empty`
       }
     }
   } else if (warp == 1) {

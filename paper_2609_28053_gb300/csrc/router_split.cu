@@ -16,7 +16,8 @@
 // d = 4,096, where the one long sum has 2,335.
 //
 // Every mbarrier wait is bounded and every thread reaches both cluster
-// barriers, whether or not a wait ran out.
+// barriers, whether or not a wait ran out; after one that did, the tile loads
+// in flight are waited for (bounded again) before the block returns.
 #include "route_warp.cuh"
 #include "tcgen05.cuh"
 
@@ -82,7 +83,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __shared__ uint2 cand[kThreads / 32][32];
   __shared__ __align__(8) uint64_t bars[2 * 8 + 1];  // full, empty, accumulator done
   __shared__ uint32_t tmem_holder;
-  __shared__ int abort_word;
+  __shared__ int abort_word, issued;  // issued: the producer's loads, for the drain after an abort
   volatile int* abort_flag = &abort_word;
   const int T = a.T, N = a.N, S = a.S;
   const uint32_t raw = smem_u32(smem_raw);
@@ -122,9 +123,9 @@ __global__ void __launch_bounds__(kThreads, 1)
 
   if (warp == 0) {
     if (lane == 0) {
-      int stage = 0;
+      int stage = 0, kb = kb0;
       uint32_t phase = 0;
-      for (int kb = kb0; kb < kb1; ++kb) {
+      for (; kb < kb1; ++kb) {
         if (!mbar_wait(empty(stage), phase ^ 1u, abort_flag)) break;
         const uint32_t dst = base + static_cast<uint32_t>(stage) * stage_bytes;
         mbar_expect_tx(full(stage), stage_bytes);
@@ -132,6 +133,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         tma_load_2d(dst + a_bytes, &tmw, full(stage), kb * kBK, 0);
         if (++stage == S) { stage = 0; phase ^= 1u; }
       }
+      issued = kb - kb0;
     }
   } else if (warp == 1) {
     if (lane == 0) {
@@ -233,7 +235,10 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(256u) : "memory");
   }
-  if (threadIdx.x == 0 && *abort_flag) raise_flag(a.err, kErrCuda);
+  if (threadIdx.x == 0 && *abort_flag) {
+    drain_loads(issued, S, full);
+    raise_flag(a.err, kErrCuda);
+  }
 }
 
 }  // namespace

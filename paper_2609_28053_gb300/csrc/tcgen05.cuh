@@ -51,6 +51,18 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   return false;
 }
 
+// After a wait ran out: tile loads may still be on their way into shared
+// memory, which is not this block's any more once it has returned.  Waits for
+// the last min(S, issued) of the `issued` loads of a ring of S stages (load i
+// completes the phase of parity (i / S) & 1 of barrier(i % S)), within one
+// limit for all of them.
+template <class Barrier>
+__device__ __forceinline__ void drain_loads(int issued, int S, Barrier barrier) {
+  uint32_t left = kSpinLimit;
+  for (int i = issued > S ? issued - S : 0; i < issued; ++i)
+    while (left > 0u && !mbar_try_wait(barrier(i % S), static_cast<uint32_t>(i / S) & 1u)) --left;
+}
+
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0,
                                             int c1) {
   asm volatile(
