@@ -33,6 +33,15 @@ __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wa
 // griddep_wait, for this grid to complete).
 __device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Lets `kern` take up to `most` bytes of dynamic shared memory.  The limit
+// belongs to the function, not to the call: a second host thread may set it
+// between this thread's setting and its launch.  So `most` is the same for
+// every call of an instance, whatever the call itself takes.
+template <typename... KArgs>
+inline bool allow_smem(void (*kern)(KArgs...), int most) {
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most) == cudaSuccess;
+}
+
 // Launch `kern` as a programmatic dependent of the previous work in `s`.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_dependent(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,

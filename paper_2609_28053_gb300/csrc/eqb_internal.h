@@ -55,6 +55,9 @@ struct RouteArgs {
 // (per-expert state of the per-microbatch kernels lives in shared memory).
 constexpr int kMaxE = 1024;
 
+// Most microbatches of MaxVio (a double each in shared memory).
+constexpr int kMaxMicrobatches = 16384;
+
 // Most expert tiles a histogram pass is cut into.
 constexpr int kMaxHistTiles = 31;
 

@@ -455,10 +455,13 @@ int launch_hist_pass(const HistArgs& a, const LeiStream& ls, CoefRows cr, cudaSt
   const HistCut h = cut_hist(a.T, a.E, PASS, di.sm_count - cr.blocks);
   const int smem = (h.copies > 1 ? kBankWords : bin_words(h.chunks)) * 4;
   auto kern = hist_kernel<PASS, LEI, false>;
+  int most = bin_words(kMaxTileChunks) * 4;
   if constexpr (PASS != 2)
-    if (h.copies > 1) kern = hist_kernel<PASS, LEI, true>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
-    return kErrCuda;
+    if (h.copies > 1) {
+      kern = hist_kernel<PASS, LEI, true>;
+      most = kBankWords * 4;
+    }
+  if (!allow_smem(kern, most)) return kErrCuda;
   return launch_dependent(kern, dim3((unsigned)(h.tiles * h.ranges + cr.blocks)), dim3(1024), smem, s, a, h.tiles,
                           h.chunks, h.copies, h.tpc, ls, cr) == cudaSuccess
              ? kOk

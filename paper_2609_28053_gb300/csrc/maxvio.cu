@@ -97,8 +97,7 @@ __global__ void __launch_bounds__(kThreads) maxvio_kernel(const int32_t* __restr
 int launch_maxvio(const int32_t* loads, const int64_t* off, int M, int E, int K, double* out, double* per_mb,
                   cudaStream_t s) {
   const int smem = M * static_cast<int>(sizeof(double));
-  if (smem > 48 * 1024 &&
-      cudaFuncSetAttribute(maxvio_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
+  if (smem > 48 * 1024 && !allow_smem(maxvio_kernel, kMaxMicrobatches * static_cast<int>(sizeof(double))))
     return kErrCuda;
   return launch_dependent(maxvio_kernel, dim3(1), dim3(kThreads), smem, s, loads, off, M, E, K, out, per_mb) ==
                  cudaSuccess

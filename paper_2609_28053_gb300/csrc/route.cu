@@ -318,8 +318,7 @@ int launch_route_many(const RouteArgs& a, cudaStream_t s) {
   const int64_t total_warps = grid * nw;
   const int64_t tpw = (ntiles + total_warps - 1) / total_warps;
   auto kern = route_kernel;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
-    return kErrCuda;
+  if (!allow_smem(kern, di.max_smem_optin)) return kErrCuda;
   return launch_dependent(kern, dim3((unsigned)grid), dim3(nw * 32), smem, s, a, tpw, nbuf) == cudaSuccess
              ? kOk
              : kErrCuda;

@@ -239,8 +239,7 @@ int launch_fused_t(const RouteArgs& a, int32_t* hist, cudaStream_t s) {
   if (grid > max_grid) grid = max_grid;
   const int64_t tpw = (ntiles + grid * NW - 1) / (grid * NW);
   auto kern = route_hist_kernel<E, KP1, NW>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
-    return kErrCuda;
+  if (!allow_smem(kern, smem)) return kErrCuda;
   return launch_dependent(kern, dim3((unsigned)grid), dim3(NW * 32), smem, s, a, hist, tpw) == cudaSuccess
              ? kOk
              : kErrCuda;

@@ -110,8 +110,7 @@ int launch_narrow_t(const RouteArgs& a, cudaStream_t s) {
   if (int rc = device_info(&di)) return rc;
   auto kern = route_narrow_kernel<E, KP1, EXACT>;
   constexpr int smem = NarrowLayout<E>::SMEM;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
-    return kErrCuda;
+  if (!allow_smem(kern, smem)) return kErrCuda;
   // resident blocks: six by registers (72 to 83 a thread), or by shared memory
   constexpr int per_sm = 228 * 1024 / (smem + 1024) < 6 ? 228 * 1024 / (smem + 1024) : 6;
   const int64_t ntiles = (a.T + 31) / 32;

@@ -136,8 +136,7 @@ int launch_wide_t(const RouteArgs& a, cudaStream_t s) {
   if (grid > max_grid) grid = max_grid;
   const int64_t tpw = (ntiles + grid * nw - 1) / (grid * nw);
   auto kern = route_wide_kernel<E, KP1, EXACT>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
-    return kErrCuda;
+  if (!allow_smem(kern, L::HEAD + nw_max * L::WARP)) return kErrCuda;
   return launch_dependent(kern, dim3((unsigned)grid), dim3((unsigned)nw * 32), smem, s, a, tpw) == cudaSuccess
              ? kOk
              : kErrCuda;

@@ -415,9 +415,7 @@ int launch_gemm(const uint16_t* x, const uint16_t* W, GemmArgs a, cudaStream_t s
   const int smem = S * stage_bytes + extra;
   const int ntiles = (a.T + kBM - 1) / kBM;
   const int grid = ntiles < di.sm_count ? ntiles : di.sm_count;
-  if (cudaFuncSetAttribute(router_gemm_kernel<EC, KP1, HIST>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) !=
-      cudaSuccess)
-    return kErrCuda;
+  if (!allow_smem(router_gemm_kernel<EC, KP1, HIST>, di.max_smem_optin)) return kErrCuda;
   return launch_dependent(router_gemm_kernel<EC, KP1, HIST>, dim3(grid), dim3(192), smem, s, tmx, tmw, a) == cudaSuccess
              ? kOk
              : kErrCuda;

@@ -258,16 +258,16 @@ int launch_router_pair(const uint16_t* x, const uint16_t* W, int64_t T, int d, i
     return kErrCuda;
   PairArgs a{z, static_cast<int>(T), d, E, 0, err};
   const int stage_bytes = (kBM + E / 2) * kBK * 2;
-  int S = (di.max_smem_optin - 2 * 1024) / stage_bytes;  // the static arrays and the alignment slack
+  const int most = di.max_smem_optin - 1024;  // beside the static arrays
+  int S = (most - 1024) / stage_bytes;        // 1 KiB of alignment slack
   if (S > 8) S = 8;
   a.S = S;
   const int smem = S * stage_bytes + 1024;
-  if (cudaFuncSetAttribute(router_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
-    return kErrCuda;
+  if (!allow_smem(router_pair_kernel, most)) return kErrCuda;
   const int64_t pairs = (T + 2 * kBM - 1) / (2 * kBM);
-  const int64_t most = di.sm_count / 2;
+  const int64_t resident = di.sm_count / 2;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(static_cast<unsigned>(2 * (pairs < most ? pairs : most)));
+  cfg.gridDim = dim3(static_cast<unsigned>(2 * (pairs < resident ? pairs : resident)));
   cfg.blockDim = dim3(192);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;

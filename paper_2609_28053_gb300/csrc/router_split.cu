@@ -270,8 +270,8 @@ int launch_router_split(const uint16_t* x, const uint16_t* W, int64_t T, int d, 
   SplitArgs a{z, static_cast<int>(T), d, E, 0, err, ro};
   const int stage_bytes = (kBM + E) * kBK * 2;
   const int part = kBM * (E + 4) * 4;
-  const int most = di.max_smem_optin - 8 * 1024;  // the static arrays and the alignment slack
-  int S = most / stage_bytes;
+  const int most = di.max_smem_optin - 7 * 1024;  // beside the static arrays
+  int S = (most - 1024) / stage_bytes;            // 1 KiB of alignment slack
   if (S > 8) S = 8;
   const int blocks = d / kBK / n + 1;  // k-blocks of the longest part
   if (S > blocks) S = blocks;
@@ -281,8 +281,7 @@ int launch_router_split(const uint16_t* x, const uint16_t* W, int64_t T, int d, 
   if (smem < part) smem = part;
   smem += 1024;
   auto kern = n == 8 ? router_split_kernel<8> : n == 4 ? router_split_kernel<4> : router_split_kernel<2>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
-    return kErrCuda;
+  if (!allow_smem(kern, most)) return kErrCuda;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)((T + kBM - 1) / kBM * n));
   cfg.blockDim = dim3(kThreads);
