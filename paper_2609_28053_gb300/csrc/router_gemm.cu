@@ -400,6 +400,8 @@ template <int EC, int KP1, bool HIST>
 int launch_gemm(const uint16_t* x, const uint16_t* W, GemmArgs a, cudaStream_t s) {
   DeviceInfo di;
   if (int rc = device_info(&di)) return rc;
+  // before the maps: encoding them needs a context, which a thread's first runtime call makes current
+  if (!allow_smem(router_gemm_kernel<EC, KP1, HIST>, di.max_smem_optin)) return kErrCuda;
   CUtensorMap tmx, tmw;
   if (!make_map(&tmx, x, static_cast<uint64_t>(a.T), static_cast<uint64_t>(a.d), kBM)) return kErrCuda;
   if (!make_map(&tmw, W, static_cast<uint64_t>(a.N), static_cast<uint64_t>(a.d), static_cast<uint32_t>(a.N)))
@@ -415,7 +417,6 @@ int launch_gemm(const uint16_t* x, const uint16_t* W, GemmArgs a, cudaStream_t s
   const int smem = S * stage_bytes + extra;
   const int ntiles = (a.T + kBM - 1) / kBM;
   const int grid = ntiles < di.sm_count ? ntiles : di.sm_count;
-  if (!allow_smem(router_gemm_kernel<EC, KP1, HIST>, di.max_smem_optin)) return kErrCuda;
   return launch_dependent(router_gemm_kernel<EC, KP1, HIST>, dim3(grid), dim3(192), smem, s, tmx, tmw, a) == cudaSuccess
              ? kOk
              : kErrCuda;

@@ -252,18 +252,19 @@ int launch_router_pair(const uint16_t* x, const uint16_t* W, int64_t T, int d, i
   if (E > 256 || E % 32 != 0) return kErrUnsupported;  // one UMMA N over two SMs, two accumulators
   DeviceInfo di;
   if (int rc = device_info(&di)) return rc;
+  const int most = di.max_smem_optin - 1024;  // beside the static arrays
+  // before the maps: encoding them needs a context, which a thread's first runtime call makes current
+  if (!allow_smem(router_pair_kernel, most)) return kErrCuda;
   CUtensorMap tmx, tmw;
   if (!make_map(&tmx, x, static_cast<uint64_t>(T), static_cast<uint64_t>(d), kBM)) return kErrCuda;
   if (!make_map(&tmw, W, static_cast<uint64_t>(E), static_cast<uint64_t>(d), static_cast<uint32_t>(E / 2)))
     return kErrCuda;
   PairArgs a{z, static_cast<int>(T), d, E, 0, err};
   const int stage_bytes = (kBM + E / 2) * kBK * 2;
-  const int most = di.max_smem_optin - 1024;  // beside the static arrays
   int S = (most - 1024) / stage_bytes;        // 1 KiB of alignment slack
   if (S > 8) S = 8;
   a.S = S;
   const int smem = S * stage_bytes + 1024;
-  if (!allow_smem(router_pair_kernel, most)) return kErrCuda;
   const int64_t pairs = (T + 2 * kBM - 1) / (2 * kBM);
   const int64_t resident = di.sm_count / 2;
   cudaLaunchConfig_t cfg = {};

@@ -262,15 +262,18 @@ int launch_router_split(const uint16_t* x, const uint16_t* W, int64_t T, int d, 
                         const SplitRoute& ro, int32_t* err, cudaStream_t s) {
   DeviceInfo di;
   if (int rc = device_info(&di)) return rc;
+  if (ro.b && E > 128) return kErrUnsupported;
+  const int most = di.max_smem_optin - 7 * 1024;  // beside the static arrays
+  // before the maps: encoding them needs a context, which a thread's first runtime call makes current
+  auto kern = n == 8 ? router_split_kernel<8> : n == 4 ? router_split_kernel<4> : router_split_kernel<2>;
+  if (!allow_smem(kern, most)) return kErrCuda;
   CUtensorMap tmx, tmw;
   if (!make_map(&tmx, x, static_cast<uint64_t>(T), static_cast<uint64_t>(d), kBM)) return kErrCuda;
   if (!make_map(&tmw, W, static_cast<uint64_t>(E), static_cast<uint64_t>(d), static_cast<uint32_t>(E)))
     return kErrCuda;
-  if (ro.b && E > 128) return kErrUnsupported;
   SplitArgs a{z, static_cast<int>(T), d, E, 0, err, ro};
   const int stage_bytes = (kBM + E) * kBK * 2;
   const int part = kBM * (E + 4) * 4;
-  const int most = di.max_smem_optin - 7 * 1024;  // beside the static arrays
   int S = (most - 1024) / stage_bytes;            // 1 KiB of alignment slack
   if (S > 8) S = 8;
   const int blocks = d / kBK / n + 1;  // k-blocks of the longest part
@@ -280,8 +283,6 @@ int launch_router_split(const uint16_t* x, const uint16_t* W, int64_t T, int d, 
   int smem = S * stage_bytes;
   if (smem < part) smem = part;
   smem += 1024;
-  auto kern = n == 8 ? router_split_kernel<8> : n == 4 ? router_split_kernel<4> : router_split_kernel<2>;
-  if (!allow_smem(kern, most)) return kErrCuda;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)((T + kBM - 1) / kBM * n));
   cfg.blockDim = dim3(kThreads);

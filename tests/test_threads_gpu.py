@@ -50,6 +50,29 @@ def maxvio(M, E):
     return out, lambda: eqb.eqb_maxvio(loads, off, 1, out=out[0])
 
 
+@pytest.mark.parametrize("T,d,E", [(100, 1024, 64), (100, 512, 64), (16384, 2048, 256)])
+def test_first_call_of_a_thread(T, d, E):
+    """A projection as the first CUDA work of a thread: the context is not
+    current there yet when the call prepares its tensor maps."""
+    out, f = logits(T, d, E)
+    f()
+    torch.cuda.synchronize()
+    ref, failed = out[0].clone(), []
+
+    def work():
+        try:
+            f()
+        except Exception as e:
+            failed.append(e)
+
+    t = threading.Thread(target=work)
+    t.start()
+    t.join()
+    torch.cuda.synchronize()
+    assert not failed, failed
+    assert torch.equal(out[0], ref)
+
+
 @pytest.mark.parametrize("make,small,large", [
     (step, (9000, 256, 8), (120000, 256, 8)),         # tiles of routing, tiles of bins
     (step, (3000, 64, 8), (120000, 64, 8)),
@@ -73,7 +96,6 @@ def test_two_shapes_from_two_threads(make, small, large):
     def work(f):
         try:
             with torch.cuda.stream(torch.cuda.Stream()):
-                torch.zeros(1, device="cuda")  # the thread's context
                 for _ in range(1500):
                     f()
                 torch.cuda.current_stream().synchronize()
