@@ -112,7 +112,8 @@ __global__ void __launch_bounds__(32 * kWarps) route_warp_kernel(RouteArgs a, in
           for (int q = 1; q < N; ++q) si = i == q ? s[q] : si;
           if (m != 0u) {
             const int e = 8 * (lane + 32 * (i >> 3)) + (i & 7);
-            cand[wid][base + __popc(more & ((1u << lane) - 1u))] = make_uint2(__float_as_uint(si), e);
+            cand[wid][base + __popc(more & ((1u << lane) - 1u))] =
+                make_uint2(__float_as_uint(si != si ? INFINITY : si), e);
           }
           base += __popc(more);
           m &= m - 1u;

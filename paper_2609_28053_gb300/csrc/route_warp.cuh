@@ -8,8 +8,9 @@
 // together, which only lowers it), is <= tau_t, so the scores >= it hold the
 // top K + 1; about K + 3 of them do.  They are collected in shared memory, one
 // per lane, each lane counts the ones that come before its own (higher score,
-// ties to the lower index), and the lane of rank r holds entry r.  More than
-// 32 of them (many equal scores, or fewer than K + 1 lanes with a share) are selected one
+// ties to the lower index), and the lane of rank r holds entry r.  A NaN
+// (flagged) is listed as +inf, so that the ranks stay a permutation and every
+// output of the token is written, with experts in range.  More than 32 of them (many equal scores, or fewer than K + 1 lanes with a share) are selected one
 // by one over the whole row instead.
 #pragma once
 
@@ -79,7 +80,7 @@ __device__ __forceinline__ int warp_route(const float (&s)[N], float lmax, int E
       for (int q = 1; q < N; ++q) si = i == q ? s[q] : si;
       if (m != 0u) {
         const int e = expert(i);
-        cand[base + __popc(more & ((1u << lane) - 1u))] = make_uint2(__float_as_uint(si), e);
+        cand[base + __popc(more & ((1u << lane) - 1u))] = make_uint2(__float_as_uint(si != si ? INFINITY : si), e);
       }
       base += __popc(more);
       m &= m - 1u;

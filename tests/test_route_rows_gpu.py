@@ -98,6 +98,51 @@ def test_nan_bias_of_a_padded_row(E, K, pattern):
     assert torch.equal(loads.view.sum(dim=1).cpu(), K * (off[1:] - off[:-1]).cpu().to(torch.int32))
 
 
+def check_flagged(idx, tau, err, E, nan_rows, idx_ref, tau_ref):
+    """A call with NaN scores: flagged, every output written and every index
+    in range, distinct in its row; the other rows as the oracle has them."""
+    idx, tau = idx.cpu().numpy(), tau.cpu().numpy()
+    assert err.item() == 4  # EQB_ERR_NONFINITE
+    assert idx.min() >= 0 and idx.max() < E and not (tau == -7).any()
+    assert all(len(set(row)) == len(row) for row in idx)
+    assert np.array_equal(idx[~nan_rows], idx_ref[~nan_rows])
+    assert np.array_equal(bits_f32(tau[~nan_rows]), bits_f32(tau_ref[~nan_rows]))
+
+
+@pytest.mark.parametrize("E", [256, 512, 1000])
+def test_nan_scores_of_a_warp(E):
+    T, K = 500, 8
+    rng = np.random.default_rng(E)
+    z = brute.bf16_bits_from_f32(rng.standard_normal((T, E), dtype=np.float32))
+    b = (rng.standard_normal(E) * 0.3).astype(np.float32)
+    idx_ref, tau_ref, _ = oracle.route(z, b, K)
+    nan_rows = np.arange(T) % 3 == 0
+    for t in np.flatnonzero(nan_rows):  # one, two or many NaN
+        z[t, rng.choice(E, [1, 2, 20][t // 3 % 3], replace=False)] = [0x7fc0, 0xffc1][t % 2]
+    idx, tau = Guarded((T, K), torch.int32, fill=-7), Guarded((T,), torch.float32, fill=-7.0)
+    loads, err = Guarded((2, E), torch.int32), torch.zeros(1, dtype=torch.int32, device="cuda")
+    off = torch.tensor([0, 200, T], device="cuda")
+    eqb.eqb_route_topk(to_dev_bf16(z), torch.from_numpy(b).cuda(), K, off, idx.view, tau.view, loads.view, err_flag=err)
+    torch.cuda.synchronize()
+    assert idx.intact() and tau.intact() and loads.intact()
+    check_flagged(idx.view, tau.view, err, E, nan_rows, idx_ref, tau_ref)
+    assert torch.equal(loads.view.sum(dim=1).cpu(), torch.tensor([200 * K, (T - 200) * K], dtype=torch.int32))
+
+
+@pytest.mark.parametrize("E", [64, 128])
+@pytest.mark.parametrize("n", [1, 2])
+def test_nan_scores_of_the_split_projection(E, n):
+    T, d, K = 200, 1024, 8
+    x, W = torch.randn((T, d), device="cuda").to(torch.bfloat16), torch.randn((E, d), device="cuda").to(torch.bfloat16)
+    W[5:5 + n] = float("nan")  # n experts of every token
+    idx, tau = Guarded((T, K), torch.int32, fill=-7), Guarded((T,), torch.float32, fill=-7.0)
+    err = torch.zeros(1, dtype=torch.int32, device="cuda")
+    eqb.eqb_router_route(x, W, torch.zeros(E, device="cuda"), K, topk_idx=idx.view, tau=tau.view, err_flag=err)
+    torch.cuda.synchronize()
+    assert idx.intact() and tau.intact()
+    check_flagged(idx.view, tau.view, err, E, np.ones(T, bool), idx.view.cpu().numpy(), tau.view.cpu().numpy())
+
+
 def test_microbatches_of_a_warp():
     """More boundaries than a warp loads at once, most of them equal, and
     enough tokens of a wide row for the loads to be counted by segments."""
