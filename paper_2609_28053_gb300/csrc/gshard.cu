@@ -29,7 +29,7 @@ __global__ void __launch_bounds__(kGsThreads, CPL > 1 ? 2 : 4) gshard_kernel(Gsh
   constexpr int U = CPL < 4 ? 2 : 1;
   __shared__ __align__(16) float Rs[kMaxE];
   __shared__ float cs;
-  __shared__ double inv[2];  // 1 / (K n) and 1 / E
+  __shared__ double inv;  // 1 / (K n E)
   const int E = a.E, nch = E >> 3;
   griddep_wait();
   const int64_t tb = (int64_t)blockIdx.x * tokens_per_cta;
@@ -46,15 +46,18 @@ __global__ void __launch_bounds__(kGsThreads, CPL > 1 ? 2 : 4) gshard_kernel(Gsh
     __syncthreads();  // the previous segment is done with Rs, cs and inv
     const int64_t n = hi - lo;
     if (threadIdx.x == 0) {
-      inv[0] = n > 0 ? 1.0 / ((double)a.K * (double)n) : 0.0;
-      inv[1] = 1.0 / (double)E;
+      inv = n > 0 ? 1.0 / ((double)a.K * (double)n * (double)E) : 0.0;
       cs = n > 0 ? __double2float_rn((double)a.alpha / (double)n) : 0.f;
     }
     __syncthreads();
-    // the divisions once per segment: fp64 runs at two lanes a clock here, and
-    // one per expert took 12 of 115 us at T = 524,288, E = 128
-    for (int e = threadIdx.x; e < E; e += blockDim.x)
-      Rs[e] = n > 0 ? __double2float_rn((double)__ldg(a.loads + (int64_t)l * E + e) * inv[0] - inv[1]) : 0.f;
+    // R = (f E - K n) / (K n E): an exact whole number (below 2^42) times one
+    // reciprocal, so that a balanced load gives 0.  The division once per
+    // segment: fp64 runs at two lanes a clock here, and one per expert took 12
+    // of 115 us at T = 524,288, E = 128
+    for (int e = threadIdx.x; e < E; e += blockDim.x) {
+      const int64_t f = __ldg(a.loads + (int64_t)l * E + e);
+      Rs[e] = __double2float_rn((double)(f * E - (int64_t)a.K * n) * inv);
+    }
     __syncthreads();
     // this lane's chunks: sub, sub + LPT, ... (CPL of them, past nch unused)
     float r[CPL][8];
