@@ -25,15 +25,17 @@ __device__ __forceinline__ uint32_t score_key(float s) {
   return u ^ ((u & 0x80000000u) ? 0xffffffffu : 0x80000000u);
 }
 
-// Microbatch of token t, as microbatch_of, by a whole warp in one round of
-// loads for every 32 boundaries.
+// Microbatch of token t, as microbatch_of, by a whole warp: each round of
+// loads probes 32 boundaries and leaves a 32nd of the microbatches (at most
+// three rounds for 8,192 of them).
 __device__ __forceinline__ int warp_microbatch_of(const int64_t* __restrict__ off, int M, int64_t t, int lane) {
-  int l = 0;
-  for (int j0 = 0; j0 < M - 1; j0 += 32) {
-    const int j = j0 + lane;
-    const unsigned below = __ballot_sync(kFull, j < M - 1 && __ldg(off + j + 1) <= t);
-    l += __popc(below);
-    if (below != kFull) break;
+  int l = 0, n = M;  // the token's is one of [l, l + n)
+  while (n > 1) {
+    const int step = (n + 30) >> 5;
+    const int j = l + step * (lane + 1);
+    const int below = __popc(__ballot_sync(kFull, j < l + n && __ldg(off + j) <= t));
+    l += below * step;
+    n = min(step, n - below * step);
   }
   return l;
 }

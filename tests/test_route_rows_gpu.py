@@ -144,10 +144,10 @@ def test_nan_scores_of_the_split_projection(E, n):
 
 
 def test_microbatches_of_a_warp():
-    """More boundaries than a warp loads at once, most of them equal, and
-    enough tokens of a wide row for the loads to be counted by segments."""
+    """More boundaries than a warp loads at once (two and three rounds of
+    loads), many of them equal, and enough tokens of a wide row for the loads to be counted by segments."""
     E, K = 520, 4
-    for T, M in ((700, 200), (130000, 90)):
+    for T, M in ((700, 200), (1500, 1104), (1500, 9000), (130000, 90)):
         rng = np.random.default_rng(M)
         z = brute.bf16_bits_from_f32(rng.standard_normal((T, E), dtype=np.float32))
         b = (rng.standard_normal(E) * 0.3).astype(np.float32)
