@@ -332,11 +332,19 @@ int launch_route_many(const RouteArgs& a, cudaStream_t s) {
 // against 9.8, T = 30,000, E = 512 15 against 21; below E = 128 tiles take
 // under 4 us), and for rows too wide for a tile with enough warps beside it
 // (T = 300,000, E = 1024 248 us against 598).
+// Lists of 17 and more (us, a warp per token / tiles): the bound from 32 lane
+// maxima leaves more than 32 candidates to more and more tokens, which are
+// then selected one by one.  K = 20: E = 256 9.8 / 28 at T = 2,048, 15.8 / 29
+// at 4,096, 25 / 31 at 8,192; E = 512 24 / 31 and 40 / 31 from 4,096 on; E =
+// 768 25 / 31, 47 / 30; T = 131,072, E = 520 733 / 165.  K = 31: T = 2,048,
+// E = 1024 37 / 105.
 int launch_route(const RouteArgs& a, cudaStream_t s) {
   const int kp1 = a.K + 1;
   if (kp1 > 32) return kErrUnsupported;
-  if (a.E > 512 || (a.E >= 128 && a.E >= 8 * kp1 && a.T <= 32 * (int64_t)a.E)) return launch_route_warp(a, s);
-  if (kp1 > 16) return launch_route_many(a, s);
+  const bool lanes_hold_list = a.E >= 128 && a.E >= 8 * kp1;
+  if (kp1 > 16)
+    return lanes_hold_list && a.T <= (a.E <= 512 ? 4096 : 2048) ? launch_route_warp(a, s) : launch_route_many(a, s);
+  if (a.E > 512 || (lanes_hold_list && a.T <= 32 * (int64_t)a.E)) return launch_route_warp(a, s);
   return a.E <= 128 ? launch_route_narrow(a, s) : launch_route_wide(a, s);
 }
 

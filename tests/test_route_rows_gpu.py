@@ -55,7 +55,7 @@ def test_list_lengths(E, K):
     if K >= E:
         pytest.skip("K < E")
     rng = np.random.default_rng(K)
-    for T in (70, 32 * E + 40):
+    for T in (70, 2100, 32 * E + 40):
         z = brute.bf16_bits_from_f32(rng.standard_normal((T, E), dtype=np.float32))
         check(z, (rng.standard_normal(E) * 0.3).astype(np.float32), K, 3, seed=K)
 
