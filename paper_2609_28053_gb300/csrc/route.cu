@@ -326,12 +326,13 @@ int launch_route_many(const RouteArgs& a, cudaStream_t s) {
 
 }  // namespace
 
-// A warp per token up to 32 E tokens, where tiles leave SMs idle and a tile's
-// serial work is the call's time (T = 4,096: E = 128 4.3 us against 4.5, 256
-// 4.1 against 6.9, 512 5.0 against 10.4; above, tiles: T = 16,411, E = 256 5.9
-// against 9.8, T = 30,000, E = 512 15 against 21; below E = 128 tiles take
-// under 4 us), and for rows too wide for a tile with enough warps beside it
-// (T = 300,000, E = 1024 248 us against 598).
+// A warp per token up to min(32 E, 8,192) tokens, where tiles leave SMs idle
+// and a tile's serial work is the call's time.  Without loads, K = 8, us, a
+// warp / tiles: E = 128 4.5 / 4.6 at T = 4,096, 5.5 / 4.7 at 6,144; E = 256 4.0
+// / 7.1, 5.1 / 6.1, 6.3 / 6.1 at 8,192, 8.3 / 6.1 at 12,288; E = 512 5.0 / 11.0,
+// 6.4 / 9.0, 7.8 / 9.2, 10.4 / 8.5 and 12.8 / 8.0 at 16,384; below E = 128 tiles
+// take under 4 us.  Beyond it also rows too wide for a tile with enough
+// warps beside it (T = 300,000, E = 1024 248 us against 598).
 // Lists of 17 and more (us, a warp per token / tiles): the bound from 32 lane
 // maxima leaves more than 32 candidates to more and more tokens, which are
 // then selected one by one.  K = 20: E = 256 9.8 / 28 at T = 2,048, 15.8 / 29
@@ -344,7 +345,8 @@ int launch_route(const RouteArgs& a, cudaStream_t s) {
   const bool lanes_hold_list = a.E >= 128 && a.E >= 8 * kp1;
   if (kp1 > 16)
     return lanes_hold_list && a.T <= (a.E <= 512 ? 4096 : 2048) ? launch_route_warp(a, s) : launch_route_many(a, s);
-  if (a.E > 512 || (lanes_hold_list && a.T <= 32 * (int64_t)a.E)) return launch_route_warp(a, s);
+  const int64_t few = 32 * a.E < 8192 ? 32 * a.E : 8192;
+  if (a.E > 512 || (lanes_hold_list && a.T <= few)) return launch_route_warp(a, s);
   return a.E <= 128 ? launch_route_narrow(a, s) : launch_route_wide(a, s);
 }
 

@@ -201,8 +201,13 @@ int launch_warp_t(const RouteArgs& a, cudaStream_t s) {
   int64_t tpb = (a.T + most - 1) / most;
   tpb = (tpb + kWarps - 1) / kWarps * kWarps;
   const int64_t grid = (a.T + tpb - 1) / tpb;
-  // A block of many tokens counts its loads in shared memory.
-  const int count_shared = a.loads && tpb > 256 ? 1 : 0;
+  // Loads in shared memory where a block has many tokens, or where many tokens
+  // share a counter: the few lanes of a token add to scattered words of a few
+  // lines, a block's flush to whole lines.  K = 8, us, each token's adds /
+  // flushed: T = 4,096, M = 1 (avg. load 256, 128, 64 at E = 128, 256, 512) 10.7
+  // / 5.3, 11.9 / 7.0 and 8.3 / 6.5; M = 3 8.3 / 5.3, 7.9 / 5.1 and, at 21, 5.7 /
+  // 6.3; M = 16 and more the same or the former.
+  const int count_shared = a.loads && (tpb > 256 || a.T * a.K > 40 * (int64_t)a.M * a.E) ? 1 : 0;
   return launch_dependent(kern, dim3((unsigned)grid), dim3(32 * kWarps), 0, s, a, (int)tpb, count_shared) ==
                  cudaSuccess
              ? kOk

@@ -39,11 +39,22 @@ def check(z, b, K, M, seed):
 WIDTHS = [8, 32, 40, 64, 72, 96, 104, 128, 136, 160, 168, 192, 200, 256, 264, 320, 328, 384, 392, 512, 520, 1024]
 
 
+@pytest.mark.parametrize("E", [128, 512, 1024])
+@pytest.mark.parametrize("T,M", [(40, 1), (1000, 1), (3000, 3), (3001, 40), (8192, 1)])
+def test_loads_of_few_tokens(T, E, M):
+    """A warp per token, on both sides of the line between each token's adds
+    and the block's counters (an average load of 40)."""
+    rng = np.random.default_rng(T + E)
+    z = brute.bf16_bits_from_f32(rng.standard_normal((T, E), dtype=np.float32))
+    check(z, (rng.standard_normal(E) * 0.3).astype(np.float32), 8, M, seed=E)
+
+
 @pytest.mark.parametrize("E", WIDTHS)
 @pytest.mark.parametrize("side", ["one", "warp", "tile"])
 def test_row_widths(E, side):
     K = min(8, E // 4)
-    T = {"one": 1, "warp": 32 * E, "tile": 32 * E + 1}[side]
+    line = min(32 * E, 8192)  # between a warp per token and tiles
+    T = {"one": 1, "warp": line, "tile": line + 1}[side]
     rng = np.random.default_rng(E)
     z = brute.bf16_bits_from_f32(rng.standard_normal((T, E), dtype=np.float32))
     check(z, (rng.standard_normal(E) * 0.3).astype(np.float32), K, 1 if T < 3 else 5, seed=E)
