@@ -145,7 +145,7 @@ int launch_clear(const StepWorkspace& w, int E, int32_t* loads, int64_t n, cudaS
 
 int launch_route(const RouteArgs& a, cudaStream_t s);
 // The routing kernels of compile-time row widths (K + 1 <= 16): E <= 128 and
-// E <= 512.
+// E <= 640.
 int launch_route_narrow(const RouteArgs& a, cudaStream_t s);
 int launch_route_wide(const RouteArgs& a, cudaStream_t s);
 // One warp per token (any E, K + 1 <= 32).

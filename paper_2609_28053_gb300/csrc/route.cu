@@ -331,8 +331,9 @@ int launch_route_many(const RouteArgs& a, cudaStream_t s) {
 // warp / tiles: E = 128 4.5 / 4.6 at T = 4,096, 5.5 / 4.7 at 6,144; E = 256 4.0
 // / 7.1, 5.1 / 6.1, 6.3 / 6.1 at 8,192, 8.3 / 6.1 at 12,288; E = 512 5.0 / 11.0,
 // 6.4 / 9.0, 7.8 / 9.2, 10.4 / 8.5 and 12.8 / 8.0 at 16,384; below E = 128 tiles
-// take under 4 us.  Beyond it also rows too wide for a tile with enough
-// warps beside it (T = 300,000, E = 1024 248 us against 598).
+// take under 4 us; E = 640 9.4 / 10.6 and 11.4 / 10.7 at 8,192.  Beyond it also
+// rows too wide for a tile with enough warps beside it (T = 300,000, E = 1024
+// 248 us against 598), from E = 648 on.
 // Lists of 17 and more (us, a warp per token / tiles): the bound from 32 lane
 // maxima leaves more than 32 candidates to more and more tokens, which are
 // then selected one by one.  K = 20: E = 256 9.8 / 28 at T = 2,048, 15.8 / 29
@@ -346,7 +347,7 @@ int launch_route(const RouteArgs& a, cudaStream_t s) {
   if (kp1 > 16)
     return lanes_hold_list && a.T <= (a.E <= 512 ? 4096 : 2048) ? launch_route_warp(a, s) : launch_route_many(a, s);
   const int64_t few = 32 * a.E < 8192 ? 32 * a.E : 8192;
-  if (a.E > 512 || (lanes_hold_list && a.T <= few)) return launch_route_warp(a, s);
+  if (a.E > 640 || (lanes_hold_list && a.T <= few)) return launch_route_warp(a, s);
   return a.E <= 128 ? launch_route_narrow(a, s) : launch_route_wide(a, s);
 }
 

@@ -1,7 +1,7 @@
 // route_wide.cu -- top-K routing, cutoff tau_t and per-microbatch loads
 // (Sec. 2, Eq. 1 and the QB paragraph of arXiv 2609.28053) for rows of 136 to
-// 512 experts with K + 1 <= 16, at a compile-time row width of 160, 192, 256,
-// 320, 384 or 512 experts (narrower rows padded with -inf).
+// 640 experts with K + 1 <= 16, at a compile-time row width of 160, 192, 224,
+// 256, 320, 384, 512 or 640 experts (narrower rows padded with -inf).
 //
 // One thread owns one token; a warp owns a tile of 32 consecutive tokens,
 // which each lane brings into shared memory with one bulk copy of its row
@@ -13,7 +13,8 @@
 // pipe and by the latency of its dependent instructions (12 warps an SM at
 // E = 256): T = 2,097,152, E = 256, K = 8 takes 211 us (169 at the copy
 // peak), T = 1,000,000, E = 264 152 us (219 with the runtime-width kernel it
-// replaced there), E = 160 91 (139).
+// replaced there), E = 160 91 (139).  Four warps at E = 640: T = 131,072, E =
+// 520 52 us (95; a warp per token 115).
 #include "route_wide.cuh"
 
 namespace eqb {
@@ -170,10 +171,12 @@ int launch_route_wide(const RouteArgs& a, cudaStream_t s) {
   if (a.E == 512) return launch_wide_e<512>(a, s);
   if (a.E <= 160) return launch_wide_padded<160>(a, s);
   if (a.E <= 192) return launch_wide_padded<192>(a, s);
+  if (a.E <= 224) return launch_wide_padded<224>(a, s);
   if (a.E <= 256) return launch_wide_padded<256>(a, s);
   if (a.E <= 320) return launch_wide_padded<320>(a, s);
   if (a.E <= 384) return launch_wide_padded<384>(a, s);
   if (a.E <= 512) return launch_wide_padded<512>(a, s);
+  if (a.E <= 640) return launch_wide_padded<640>(a, s);
   return kErrUnsupported;
 }
 

@@ -36,7 +36,8 @@ def check(z, b, K, M, seed):
     assert np.array_equal(loads.view.cpu().numpy(), loads_ref)
 
 
-WIDTHS = [8, 32, 40, 64, 72, 96, 104, 128, 136, 160, 168, 192, 200, 256, 264, 320, 328, 384, 392, 512, 520, 1024]
+WIDTHS = [8, 32, 40, 64, 72, 96, 104, 128, 136, 160, 168, 192, 200, 224, 232, 256, 264, 320, 328, 384, 392, 512, 520,
+          640, 648, 1024]
 
 
 @pytest.mark.parametrize("E", [128, 512, 1024])
