@@ -28,9 +28,11 @@ def inputs(T, d, E, seed):
 
 
 @pytest.mark.parametrize("T", [1, 8, 127, 129, 1024, 1025, 1153, 4096, 4225, 8192, 8449])
-@pytest.mark.parametrize("d,E", [(1024, 128), (4096, 64)])
-def test_route(T, d, E):
-    K, M = (8, 5) if T > 8 else (3, 1)
+@pytest.mark.parametrize("d,E,M", [(1024, 128, 5), (4096, 64, 5), (1088, 64, 100)])
+def test_route(T, d, E, M):
+    """Few microbatches, where a tile's loads are counted together, and more than
+    a tile has tokens of one."""
+    K, M = (8, M) if T > 8 else (3, 1)
     x, W, z_ref = inputs(T, d, E, seed=T + E)
     b = torch.randn(E, device="cuda") * 30.0
     off = torch.from_numpy(ragged_offsets(T, M, seed=T) if M > 1 else np.array([0, T], np.int64)).cuda()
