@@ -187,7 +187,7 @@ struct SplitRoute {
   float* tau = nullptr;
   int32_t* loads = nullptr;
 };
-int router_splits(int64_t T, int d, int sm_count);
+int router_splits(int64_t T, int d, int E, int sm_count);
 // Many experts, columns and tokens (router_pair.cu; E a multiple of 32, at
 // most 256): pairs of SMs.
 int launch_router_pair(const uint16_t* x, const uint16_t* W, int64_t T, int d, int E, uint16_t* z, int32_t* err,

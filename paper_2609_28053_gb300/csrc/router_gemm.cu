@@ -431,7 +431,7 @@ int launch_router_gemm(const uint16_t* x, const uint16_t* W, int64_t T, int d, i
   if (split) {
     DeviceInfo di;
     if (int rc = device_info(&di)) return rc;
-    if (const int n = router_splits(T, d, di.sm_count); n > 1) {
+    if (const int n = router_splits(T, d, E, di.sm_count); n > 1) {
       const SplitRoute none;
       return launch_router_split(x, W, T, d, E, n, z, none, err, s);
     }
@@ -462,7 +462,7 @@ int launch_router_route(const uint16_t* x, const uint16_t* W, int64_t T, int d, 
   if (split) {
     DeviceInfo di;
     if (int rc = device_info(&di)) return rc;
-    if (const int n = router_splits(T, d, di.sm_count); n > 1) {
+    if (const int n = router_splits(T, d, E, di.sm_count); n > 1) {
       const SplitRoute ro{b, K, off, M, idx, tau, loads};
       const int rc = launch_router_split(x, W, T, d, E, n, z, ro, err, s);
       if (rc || !hist) return rc;

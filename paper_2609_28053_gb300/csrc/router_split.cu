@@ -270,13 +270,19 @@ __global__ void __launch_bounds__(kThreads, 1)
 // 4 / 8: T = 128, d = 4,096, E = 128 19.9 / 13.8 / 9.5 / 7.8; d = 1,024 7.9 /
 // 7.8 / 6.4 / 6.1, E = 256 9.3 / 8.4 / 8.4 / 8.5; T = 2,048, d = 4,096, E =
 // 128 20.5 / 14.2 / 9.9 / 15.0; T = 8,192 20.7 / 15.1 / 19.9 / 36.9; d = 512,
-// E = 256, T = 128 7.2 / 7.4 / 7.8 / 8.2.
-int router_splits(int64_t T, int d, int sm_count) {
+// E = 256, T = 128 7.2 / 7.4 / 7.8 / 8.2.  With routing, 64 tokens a block by a
+// warp each take longer than 128 from the accumulator beside the next tile's
+// MMAs, so two blocks pay from more columns on (T = 4,225, n = 1 / 2): E = 64 9.8
+// / 12.6 at d = 1,024, 13.9 / 14.8 at 2,048, 18.0 / 16.9 at 3,072; E = 128 11.8 /
+// 12.4 at 1,024, 13.9 / 13.4 at 1,536.  The rule does not ask whether
+// there is routing: logits must not depend on it.
+int router_splits(int64_t T, int d, int E, int sm_count) {
   const int64_t tiles = (T + kBM - 1) / kBM;
   if (d < 1024) return 1;
   if (tiles * 16 <= sm_count * 7 / 8) return 8;
   if (tiles * 4 <= sm_count * 7 / 8) return 4;
-  return tiles * 2 <= sm_count * 7 / 8 ? 2 : 1;
+  const int least = E == 64 ? 3072 : E <= 128 ? 1536 : 1024;  // columns from which two pay
+  return d >= least && tiles * 2 <= sm_count * 7 / 8 ? 2 : 1;
 }
 
 int launch_router_split(const uint16_t* x, const uint16_t* W, int64_t T, int d, int E, int n, uint16_t* z,

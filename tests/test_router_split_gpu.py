@@ -52,7 +52,18 @@ def test_route(T, d, E, M):
     assert torch.equal(loads.view, loads2) and torch.equal(hist.view, hist2)
 
 
-@pytest.mark.parametrize("T,d,E", [(5, 1024, 16), (300, 1088, 48), (130, 2048, 240), (1100, 1024, 256), (4300, 1600, 256)])
+@pytest.mark.parametrize("E,d", [(64, 1024), (64, 3008), (64, 3072), (128, 1472), (128, 1536)])
+@pytest.mark.parametrize("T", [100, 3000, 6000, 9000])
+def test_logits_do_not_depend_on_routing(T, d, E):
+    """On inputs whose sums depend on their order, the logits of the call that
+    routes are those of the call that does not, bit for bit."""
+    x, W = (torch.randn(s, device="cuda").to(torch.bfloat16) for s in ((T, d), (E, d)))
+    z, _, _ = eqb.eqb_router_route(x, W, torch.zeros(E, device="cuda"), 8)
+    assert torch.equal(z.view(torch.int16), eqb.eqb_router_logits(x, W).view(torch.int16))
+
+
+@pytest.mark.parametrize("T,d,E", [(5, 1024, 16), (300, 1088, 48), (130, 2048, 240), (1100, 1024, 256), (4300, 1600, 256),
+                                   (4300, 1024, 144)])
 def test_logits(T, d, E):
     """Expert counts that fill no whole run of lanes, columns that the blocks
     of a cluster share unevenly."""
