@@ -439,12 +439,21 @@ HistCut cut_hist(int64_t T, int E, int pass, int blocks) {
   return h;
 }
 
-// A warp forms a row of the coefficient table in 2-3 us; a short pass gives
-// the rows up to 16 SMs, so that few share the fp64 pipe of one, a long one
-// four.
+// SMs that form the coefficient table.  A warp takes 2-3 us a row and a row
+// some 500 clocks of its SM's fp64 pipe, so that many microbatches need more
+// SMs: a short pass gives them 16 and one for every 16 rows, a long one four
+// and one for every 32, at most 64.  The step, us, with 4 / 16 / 32 / 64: T =
+// 16,384, E = 64, M = 16 23.3 (16), M = 256 38.9 / 25.3 / 24.2 / 24.3, M = 1,024 93 /
+// 39.7 / 30.7 / 26.2; T = 147,456, E = 256, M = 64 100.5 / 101.6 / 102.6 / 106.4;
+// T = 524,288, E = 128, M = 32 175.0 / 176.6 / 178.6, M = 512 203.6 / 180.4 / 182.6
+// / 188.8; T = 1,000,003, E = 16, M = 4,096 317 / 137 / 106 / 91 (122 with the
+// table in a kernel of its own).
 int coef_blocks(int64_t T, int E, int M, int sm_count) {
-  const int most = T * (E >> 3) / sm_count < 10000 ? 16 : 4;
-  return M < most ? M : most;
+  const bool brief = T * (E >> 3) / sm_count < 10000;
+  int n = brief ? M / 16 : M / 32;
+  const int least = brief ? 16 : 4;
+  n = n < least ? least : n > 64 ? 64 : n;
+  return M < n ? M : n;
 }
 
 template <int PASS, bool LEI>

@@ -112,11 +112,12 @@ def test_fused_pass_rejects_bad_ranges():
 
 
 @pytest.mark.parametrize("T,E,K,M", [(20000, 1024, 8, 64), (20000, 1024, 8, 65), (30000, 256, 8, 300),
-                                     (20000, 128, 8, 4)])
+                                     (20000, 128, 8, 4), (20000, 8, 2, 8192), (800000, 16, 4, 2000)])
 def test_layer_step_at_and_past_the_coefficient_table(T, E, K, M):
     """M * E = 65,536 runs the fused passes; one microbatch more (or many
     small ones) runs LEI last.  Both reproduce the oracle, and both give the
-    bits of the separate LEI launch."""
+    bits of the separate LEI launch; so do thousands of rows, which more SMs
+    form."""
     rng = np.random.default_rng(T + M)
     z = brute.bf16_bits_from_f32(rng.standard_normal((T, E)).astype(np.float32))
     b = (rng.standard_normal(E) * 0.3).astype(np.float32)
