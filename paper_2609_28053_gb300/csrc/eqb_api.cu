@@ -12,7 +12,6 @@
 namespace eqb {
 
 namespace {
-constexpr int kMaxDevices = 64;
 std::atomic<int> g_info_ready[kMaxDevices];
 DeviceInfo g_info[kMaxDevices];
 }  // namespace
@@ -26,6 +25,7 @@ int device_info(DeviceInfo* out) {
     return kOk;
   }
   DeviceInfo di;
+  di.dev = dev;
   if (cudaDeviceGetAttribute(&di.sm_count, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return kErrCuda;
   if (cudaDeviceGetAttribute(&di.max_smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) !=

@@ -10,6 +10,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "eqb_internal.h"
 
 namespace eqb {
@@ -40,6 +42,22 @@ __device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.
 template <typename... KArgs>
 inline bool allow_smem(void (*kern)(KArgs...), int most) {
   return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most) == cudaSuccess;
+}
+
+// Blocks of `kern` that an SM holds at once, at a block size and a size of
+// dynamic shared memory that are the instance's own; asked once per device
+// (`known`: the instance's [kMaxDevices], zero at first).  0 on failure.  For
+// grids of one round: with more blocks per SM the rest run alone afterwards,
+// with fewer they pile up on some SMs whenever the kernel is launched while
+// its predecessor still holds the others.
+template <typename... KArgs>
+inline int resident_blocks(void (*kern)(KArgs...), int threads, size_t smem, int dev, std::atomic<int>* known) {
+  int n = known[dev].load(std::memory_order_relaxed);
+  if (n == 0) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, threads, smem) != cudaSuccess) return 0;
+    known[dev].store(n, std::memory_order_relaxed);
+  }
+  return n;
 }
 
 // Launch `kern` as a programmatic dependent of the previous work in `s`.

@@ -17,7 +17,10 @@ enum : int {
   kErrRank = 5,
 };
 
+constexpr int kMaxDevices = 64;
+
 struct DeviceInfo {
+  int dev;             // its number, below kMaxDevices
   int sm_count;
   int max_smem_optin;  // bytes of dynamic shared memory a block may opt into
 };

@@ -111,8 +111,10 @@ int launch_narrow_t(const RouteArgs& a, cudaStream_t s) {
   auto kern = route_narrow_kernel<E, KP1, EXACT>;
   constexpr int smem = NarrowLayout<E>::SMEM;
   if (!allow_smem(kern, smem)) return kErrCuda;
-  // resident blocks: six by registers (72 to 83 a thread), or by shared memory
-  constexpr int per_sm = 228 * 1024 / (smem + 1024) < 6 ? 228 * 1024 / (smem + 1024) : 6;
+  // by registers (72 to 98 a thread) or by shared memory
+  static std::atomic<int> known[kMaxDevices];
+  const int per_sm = resident_blocks(kern, 32 * kNarrowWarps, smem, di.dev, known);
+  if (per_sm < 1) return kErrCuda;
   const int64_t ntiles = (a.T + 31) / 32;
   int64_t grid = (int64_t)di.sm_count * per_sm;
   const int64_t max_grid = (ntiles + kNarrowWarps - 1) / kNarrowWarps;

@@ -15,13 +15,12 @@ namespace eqb {
 namespace {
 
 constexpr int kWarps = 8;  // per block
-// Blocks that an SM holds (47, 59 and 94 registers a thread).
+// Blocks that an SM holds, by registers (48, 62 and 110 a thread).
 template <int CPL>
 constexpr int kResident = CPL == 1 ? 5 : CPL == 2 ? 4 : 2;
-
 // CPL chunks per lane: rows of up to 256 * CPL experts.
 template <int CPL>
-__global__ void __launch_bounds__(32 * kWarps) route_warp_kernel(RouteArgs a, int tokens_per_block, int count_shared) {
+__global__ void __launch_bounds__(32 * kWarps, kResident<CPL>) route_warp_kernel(RouteArgs a, int tokens_per_block, int count_shared) {
   constexpr int N = 8 * CPL;
   __shared__ __align__(16) float bs[256 * CPL];
   __shared__ int cnt[256 * CPL];  // the block's loads of one microbatch (count_shared)
@@ -197,7 +196,10 @@ int launch_warp_t(const RouteArgs& a, cudaStream_t s) {
   DeviceInfo di;
   if (int rc = device_info(&di)) return rc;
   auto kern = route_warp_kernel<CPL>;
-  const int64_t most = (int64_t)di.sm_count * kResident<CPL>;
+  static std::atomic<int> known[kMaxDevices];
+  const int per_sm = resident_blocks(kern, 32 * kWarps, 0, di.dev, known);
+  if (per_sm < 1) return kErrCuda;
+  const int64_t most = (int64_t)di.sm_count * per_sm;
   int64_t tpb = (a.T + most - 1) / most;
   tpb = (tpb + kWarps - 1) / kWarps * kWarps;
   const int64_t grid = (a.T + tpb - 1) / tpb;

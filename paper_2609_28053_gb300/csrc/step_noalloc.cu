@@ -33,7 +33,7 @@ namespace {
 constexpr size_t kStaticWorkspaceBytes = eqb::step_workspace_bytes(256);
 static __device__ __align__(256) unsigned char g_step_scratch[kStaticWorkspaceBytes];
 
-constexpr int kMaxDevices = 64;
+using eqb::kMaxDevices;
 void* g_scratch_ptr[kMaxDevices] = {};
 std::mutex g_scratch_mu;
 
