@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(1024) hist_kernel(HistArgs a, int tiles, int t
     griddep_wait();
     // a warp per row, the rows dealt out to the blocks first
     const int first = (threadIdx.x >> 5) * cr.blocks + blockIdx.x - (gridDim.x - cr.blocks);
-    for (int l = first; l < cr.a.M; l += 32 * cr.blocks) {
+    for (int l = first; l < cr.a.M; l += (blockDim.x >> 5) * cr.blocks) {
       const int64_t n = __ldg(cr.a.off + l + 1) - __ldg(cr.a.off + l);
       warp_lei_coef(cr.a.loads + (int64_t)l * E, n, E, cr.a.K, cr.a.eta, cr.a.c, cr.coef + (int64_t)l * E,
                     threadIdx.x & 31);
@@ -391,9 +391,10 @@ __global__ void __launch_bounds__(1024) hist_kernel(HistArgs a, int tiles, int t
 
 // How a pass is cut into blocks: expert tiles of `chunks` 8-expert chunks
 // times token ranges of `tpc` tokens, about one block per SM, with `copies`
-// columns for each chunk of the banked layout (1: rows of bins).
+// columns for each chunk of the banked layout (1: rows of bins), `threads` to a
+// block.  `counted`: the tiles have counters (HistArgs::done).
 struct HistCut {
-  int tiles, chunks, copies, ranges;
+  int tiles, chunks, copies, ranges, threads;
   int64_t tpc;
 };
 
@@ -417,21 +418,29 @@ struct HistCut {
 // chunks: T = 30,873, E = 256 35 / 37 / 42 us, T = 65,536, E = 64 31 / 35 /
 // 35, T = 524,288, E = 128 185 / 187 / 190, E = 256 321 / 321 / 325, T =
 // 1,048,576, E = 512 1220 / 1219 / 1211.
-HistCut cut_hist(int64_t T, int E, int pass, int blocks) {
+// The smallest batches take one or two chunks a tile and, unless warps of the
+// block stream LEI, 512 threads: little else than the fixed cost is left.  Pass
+// 1 / pass 2 alone, us, 8 and 4 chunks with 1,024 threads / now (33 one-chunk
+// tiles before the cut by size): T = 100, E = 264 4.45 / 2.6 (2.45) and 4.95 /
+// 3.3 (2.90); T = 1,000 4.75 / 4.2 (4.1) and 5.42 / 4.06 (3.80); T = 60,000, E =
+// 24 5.93 / 4.43 (4.86) in pass 2, T = 20,000, E = 200 7.14 / 6.29 (6.11).
+HistCut cut_hist(int64_t T, int E, int pass, bool lei, bool counted, int blocks) {
   const int nch = E >> 3;
   const int64_t per_sm = T * nch / blocks;  // chunks of z to count per SM
-  int want = per_sm < 10000 ? 8 : 16;
+  int want = T <= 512 ? 1 : per_sm < 1000 && !lei ? 2 : per_sm < 10000 ? 8 : 16;
   if (pass == 2) {
-    want = per_sm < 64000 ? 4 : per_sm < 200000 ? 8 : 16;
-    if (want * kMaxHistTiles < nch) want = (nch + kMaxHistTiles - 1) / kMaxHistTiles;
+    const bool one = per_sm < 2000 ? !lei || T <= 512 : per_sm < 10000 && nch <= 5;
+    want = one ? 1 : per_sm < (lei ? 4000 : 5000) ? 2 : per_sm < 64000 ? 4 : per_sm < 200000 ? 8 : 16;
+    if (counted && want * kMaxHistTiles < nch) want = (nch + kMaxHistTiles - 1) / kMaxHistTiles;
   }
   HistCut h;
   h.tiles = (nch + want - 1) / want;
   h.chunks = (nch + h.tiles - 1) / h.tiles;
   h.tiles = (nch + h.chunks - 1) / h.chunks;
+  h.threads = per_sm <= 512 && h.chunks <= 2 && !lei ? 512 : 1024;
   h.copies = pass != 2 && per_sm >= 5000 ? 32 / h.chunks : 1;
   int64_t ranges = blocks / h.tiles;
-  const int64_t most = (T * h.chunks + 1023) / 1024;  // a chunk for every thread
+  const int64_t most = (T * h.chunks + h.threads - 1) / h.threads;  // a chunk for every thread
   if (ranges > most) ranges = most;
   if (ranges < 1) ranges = 1;
   h.tpc = (T + ranges - 1) / ranges;
@@ -461,7 +470,7 @@ int launch_hist_pass(const HistArgs& a, const LeiStream& ls, CoefRows cr, cudaSt
   DeviceInfo di;
   if (int rc = device_info(&di)) return rc;
   cr.blocks = cr.coef ? coef_blocks(a.T, a.E, cr.a.M, di.sm_count) : 0;
-  const HistCut h = cut_hist(a.T, a.E, PASS, di.sm_count - cr.blocks);
+  const HistCut h = cut_hist(a.T, a.E, PASS, LEI, a.done != nullptr, di.sm_count - cr.blocks);
   const int smem = (h.copies > 1 ? kBankWords : bin_words(h.chunks)) * 4;
   auto kern = hist_kernel<PASS, LEI, false>;
   int most = bin_words(kMaxTileChunks) * 4;
@@ -471,7 +480,7 @@ int launch_hist_pass(const HistArgs& a, const LeiStream& ls, CoefRows cr, cudaSt
       most = kBankWords * 4;
     }
   if (!allow_smem(kern, most)) return kErrCuda;
-  return launch_dependent(kern, dim3((unsigned)(h.tiles * h.ranges + cr.blocks)), dim3(1024), smem, s, a, h.tiles,
+  return launch_dependent(kern, dim3((unsigned)(h.tiles * h.ranges + cr.blocks)), dim3(h.threads), smem, s, a, h.tiles,
                           h.chunks, h.copies, h.tpc, ls, cr) == cudaSuccess
              ? kOk
              : kErrCuda;

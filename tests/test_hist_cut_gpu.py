@@ -18,6 +18,12 @@ pytestmark = pytest.mark.gpu
 # 10,000 (16-chunk tiles).
 CUTS = [(1, 8, 2),           # one thread's work
         (130, 264, 8),       # 33 chunks in tiles of 7, the last of 5
+        (500, 264, 8),       # one chunk a tile, 512 threads
+        (600, 1024, 8),      # 505: two, or five where the tiles are counted
+        (1700, 264, 8),      # 369: 512 threads, several ranges
+        (2600, 264, 8),      # 564: 1,024
+        (14000, 200, 8),     # 2,302: two chunks a tile in pass 2
+        (60000, 24, 4),      # 1,184: one
         (5000, 104, 3),      # 13 chunks: 7 and 6
         (23500, 256, 4),     # 4,947: rows
         (24500, 264, 4),     # 5,319: banked, tiles of 7 and 5 chunks
