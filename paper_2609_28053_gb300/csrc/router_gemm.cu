@@ -440,8 +440,15 @@ int launch_router_gemm(const uint16_t* x, const uint16_t* W, int64_t T, int d, i
   // E = 256 18.4 / 19.4 at d = 1,024, 26.2 / 25.9 at 2,048, 44.8 / 38.4 at 4,096;
   // T = 131,072 92.4 / 91.3, 143.7 / 130.9 and 262.4 / 218.7; T = 9,000, d =
   // 2,048 22.5 / 23.4; d = 4,096, E = 224 38.5 / 38.3 and 224.2 / 213.4, E = 160
-  // 35.5 / 36.1 and 203.3 / 200.2.
-  if (E >= 224 && E % 32 == 0 && d >= 2048 && T >= 16384) return launch_router_pair(x, W, T, d, E, z, err, s);
+  // 35.5 / 36.1 and 203.3 / 200.2.  Logits alone at E = 224 in one wave of tiles:
+  // d = 2,048 17.3 / 17.9 (14.1 / 15.7 with x in L2), 3,072 25.6 / 25.1; in two
+  // 29.1 / 28.6 at d = 2,048.
+  if (E >= 224 && E % 32 == 0 && T >= 16384) {
+    DeviceInfo di;
+    if (int rc = device_info(&di)) return rc;
+    const bool one_wave = T <= (int64_t)di.sm_count * kBM;
+    if (d >= (E < 256 && one_wave ? 3072 : 2048)) return launch_router_pair(x, W, T, d, E, z, err, s);
+  }
   GemmArgs a{z, static_cast<int>(T), d, E, 0, err, nullptr, 0, nullptr, 0, nullptr, nullptr, nullptr, nullptr};
   return launch_gemm<0, 1, false>(x, W, a, s);
 }

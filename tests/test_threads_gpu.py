@@ -78,7 +78,7 @@ def test_first_call_of_a_thread(T, d, E):
     (step, (3000, 64, 8), (120000, 64, 8)),
     (logits, (100, 1024, 16), (100, 4096, 256)),      # the split projection's stages
     (logits, (100, 512, 16), (100, 512, 256)),        # the one-SM projection's
-    (logits, (16384, 2048, 224), (16384, 2048, 256)),
+    (logits, (16384, 3072, 224), (16384, 3072, 256)),
     (route, (300, 32, 20), (300, 256, 20)),           # long lists
     (maxvio, (6200, 8), (16384, 8))])
 def test_two_shapes_from_two_threads(make, small, large):
