@@ -42,11 +42,20 @@ def _p(t):
     return None if t is None else t.data_ptr()
 
 
+# torch's own shortcuts to the raw handle of the current stream (a stream object
+# takes longer to make than a small call to launch); they are private, so a
+# release without them falls back to the public call
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream(stream):
     """The raw stream handle; the current stream of the current device by
     default (the tensors of a call are on the GPU, so CUDA is initialised)."""
     if stream is None:
-        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+        if _raw_stream is not None and _raw_device is not None:
+            return _raw_stream(_raw_device())
+        stream = torch.cuda.current_stream()
     return stream.cuda_stream
 
 

@@ -337,3 +337,20 @@ def test_noalloc_wrapper_requires_the_current_device(monkeypatch):
         eqb._on_current_device(Fake(), "z")
     monkeypatch.setattr(torch.cuda, "current_device", lambda: 0)
     eqb._on_current_device(Fake(), "z")  # same device: accepted
+
+
+def test_stream_without_the_private_shortcuts(monkeypatch):
+    """A torch release without the raw-stream shortcuts: the public call serves."""
+    import torch
+
+    import paper_2609_28053_gb300 as eqb
+
+    class Stream:
+        cuda_stream = 77
+
+    monkeypatch.setattr(torch.cuda, "current_stream", Stream)
+    for gone in ("_raw_stream", "_raw_device"):
+        with monkeypatch.context() as m:
+            m.setattr(eqb, gone, None)
+            assert eqb._stream(None) == 77
+    assert eqb._stream(Stream()) == 77
