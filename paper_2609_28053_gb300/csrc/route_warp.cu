@@ -5,9 +5,10 @@
 // in shared memory.
 //
 // Lanes read the row straight into registers, the next token's while this one
-// is routed, as in warp_route (route_warp.cuh).  The steps are written out
-// here: called as that function, the same steps compile to a schedule that
-// takes 12% longer (T = 300,000, E = 1024 277 us against 248).
+// is routed.  The steps are those of warp_route (route_warp.cuh) for runs of
+// eight experts, written out: as a call of such a function they compile to a
+// schedule that takes 2% longer at K = 2, 10% at 8 and 14% at 12 (T = 300,000, E
+// = 1024, K = 8 274 us against 250).  What is mended here is mended there.
 #include "route_warp.cuh"
 
 namespace eqb {
@@ -18,9 +19,11 @@ constexpr int kWarps = 8;  // per block
 // Blocks that an SM holds, by registers (48, 62 and 110 a thread).
 template <int CPL>
 constexpr int kResident = CPL == 1 ? 5 : CPL == 2 ? 4 : 2;
+
 // CPL chunks per lane: rows of up to 256 * CPL experts.
 template <int CPL>
-__global__ void __launch_bounds__(32 * kWarps, kResident<CPL>) route_warp_kernel(RouteArgs a, int tokens_per_block, int count_shared) {
+__global__ void __launch_bounds__(32 * kWarps, kResident<CPL>)
+    route_warp_kernel(RouteArgs a, int tokens_per_block, int count_shared) {
   constexpr int N = 8 * CPL;
   __shared__ __align__(16) float bs[256 * CPL];
   __shared__ int cnt[256 * CPL];  // the block's loads of one microbatch (count_shared)

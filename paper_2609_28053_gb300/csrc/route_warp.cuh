@@ -1,17 +1,19 @@
 // route_warp.cuh -- one token routed by one warp (Sec. 2, Eq. 1 and the QB
-// paragraph of arXiv 2609.28053), for route_warp.cu and the split router
-// projection (router_split.cu).
+// paragraph of arXiv 2609.28053): warp_route for the split router projection
+// (router_split.cu), and the score key and microbatch search that it shares
+// with route_warp.cu, which writes the same steps out for wider rows.
 //
 // Every lane holds the exact scores s_e = fp32(z_e) + b_e of its share of the
-// row, runs of P experts P apart by lanes.  The (K+1)st largest of the 32 lane
-// maxima, found by K + 1 warp reductions (lanes with equal maxima leave
-// together, which only lowers it), is <= tau_t, so the scores >= it hold the
-// top K + 1; about K + 3 of them do.  They are collected in shared memory, one
-// per lane, each lane counts the ones that come before its own (higher score,
-// ties to the lower index), and the lane of rank r holds entry r.  A NaN
-// (flagged) is listed as +inf, so that the ranks stay a permutation and every
-// output of the token is written, with experts in range.  More than 32 of them (many equal scores, or fewer than K + 1 lanes with a share) are selected one
-// by one over the whole row instead.
+// row, four experts in a run.  The (K+1)st largest of the 32 lane maxima, found
+// by K + 1 warp reductions (lanes with equal maxima leave together, which only
+// lowers it), is <= tau_t, so the scores >= it hold the top K + 1; about K + 3
+// of them do.  They are collected in shared memory, one per lane, each lane
+// counts the ones that come before its own (higher score, ties to the lower
+// index), and the lane of rank r holds entry r.  A NaN (flagged) is listed as
+// +inf, so that the ranks stay a permutation and every output of the token is
+// written, with experts in range.  More than 32 of them (many equal scores, or
+// fewer than K + 1 lanes with a share) are selected one by one over the whole
+// row instead.
 #pragma once
 
 #include "eqb_device.cuh"
@@ -40,17 +42,14 @@ __device__ __forceinline__ int warp_microbatch_of(const int64_t* __restrict__ of
   return l;
 }
 
-// One token routed by a whole warp.  s[] are the lane's exact scores: of the
-// experts P (lane + 32 (i / P)) + i mod P in ascending i, -inf past E, lmax their
-// maximum (NaN if there is one); cand 32 entries of the warp's own.  The lane of rank r <= K gets entry r of the
-// list: r, the expert my_e and its score my_s (the lane of rank K holds the
-// cutoff); the other lanes a rank above K.
-template <int P, int N>
-__device__ __forceinline__ int warp_route(const float (&s)[N], float lmax, int E, int K, uint2* cand, int lane, int32_t* err,
-                                          int& my_e, float& my_s) {
-  constexpr int L = P == 8 ? 3 : 2;
-  static_assert(P == 1 << L, "runs of four or eight experts");
-  auto expert = [&](int i) { return P * (lane + 32 * (i >> L)) + (i & (P - 1)); };
+// One token routed by a whole warp.  s[] are the lane's exact scores, of the
+// experts 4 lane .. 4 lane + 3, -inf past E (a multiple of 4), lmax their maximum
+// (NaN if there is one); cand 32 entries of the warp's own.  The lane of rank r
+// <= K gets entry r of the list: r, the expert my_e and its score my_s (the lane
+// of rank K holds the cutoff); the other lanes a rank above K.
+__device__ __forceinline__ int warp_route(const float (&s)[4], float lmax, int E, int K, uint2* cand, int lane,
+                                          int32_t* err, int& my_e, float& my_s) {
+  constexpr int N = 4;
   if (lmax != lmax) raise_flag(err, kErrNonfinite);
 
   // ---- bound: the (K+1)st largest lane maximum
@@ -81,7 +80,7 @@ __device__ __forceinline__ int warp_route(const float (&s)[N], float lmax, int E
 #pragma unroll
       for (int q = 1; q < N; ++q) si = i == q ? s[q] : si;
       if (m != 0u) {
-        const int e = expert(i);
+        const int e = 4 * lane + i;
         cand[base + __popc(more & ((1u << lane) - 1u))] = make_uint2(__float_as_uint(si != si ? INFINITY : si), e);
       }
       base += __popc(more);
@@ -108,7 +107,7 @@ __device__ __forceinline__ int warp_route(const float (&s)[N], float lmax, int E
       int bi = -1;
 #pragma unroll
       for (int i = 0; i < N; ++i) {
-        const bool in = !(gone >> i & 1u) && expert(i & ~(P - 1)) < E;  // E is a multiple of P
+        const bool in = !(gone >> i & 1u) && 4 * lane < E;
         if (in && (bi < 0 || s[i] > best)) {
           best = s[i];
           bi = i;
@@ -116,7 +115,7 @@ __device__ __forceinline__ int warp_route(const float (&s)[N], float lmax, int E
       }
       const uint32_t bk = bi < 0 ? 0u : score_key(best);
       const uint32_t top = __reduce_max_sync(kFull, bk);
-      const unsigned be = bi < 0 ? 0xffffu : static_cast<unsigned>(expert(bi));
+      const unsigned be = bi < 0 ? 0xffffu : static_cast<unsigned>(4 * lane + bi);
       const unsigned win = __reduce_min_sync(kFull, bk == top ? be : 0xffffu);
       const bool mine = bi >= 0 && be == win;
       if (mine) gone |= 1u << bi;

@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       s[3] = bf16_hi(lo.y) + bv.w;
     }
     const float lmax = fmax_nan(fmax_nan(s[0], s[1]), fmax_nan(s[2], s[3]));
-    const int r = warp_route<4>(s, lmax, N, K, cand[warp], lane, a.err, e, sc);
+    const int r = warp_route(s, lmax, N, K, cand[warp], lane, a.err, e, sc);
     if (r == K) {
       a.ro.tau[t] = sc;
       if (!isfinite(sc)) raise_flag(a.err, kErrNonfinite);

@@ -52,6 +52,23 @@ def test_route(T, d, E, M):
     assert torch.equal(loads.view, loads2) and torch.equal(hist.view, hist2)
 
 
+@pytest.mark.parametrize("E", [64, 128])
+@pytest.mark.parametrize("kind", ["constant", "two values", "zeros"])
+def test_equal_scores(E, kind):
+    """More candidates than a warp lists: scores from the bias alone, all equal,
+    of two values, or zeros of both signs (equal scores)."""
+    T, d, K = 300, 1024, 8
+    x, W = torch.zeros((T, d), dtype=torch.bfloat16, device="cuda"), torch.ones((E, d), dtype=torch.bfloat16, device="cuda")
+    odd = torch.arange(E, device="cuda") % 3 == 0
+    b = {"constant": torch.full((E,), 1.5), "two values": torch.where(odd.cpu(), 0.25, -0.75),
+         "zeros": torch.where(odd.cpu(), -0.0, 0.0)}[kind].cuda()
+    z, idx, tau = eqb.eqb_router_route(x, W, b, K, topk_idx=torch.full((T, K), -7, dtype=torch.int32, device="cuda"))
+    idx2, tau2 = eqb.eqb_route_topk(z, b, K, topk_idx=torch.empty_like(idx))
+    assert torch.equal(idx, idx2) and torch.equal(tau, tau2)
+    best = torch.sort(b, descending=True, stable=True).indices[:K].to(torch.int32)  # ties to the lower index
+    assert torch.equal(idx, best.expand(T, K))
+
+
 @pytest.mark.parametrize("E,d", [(64, 1024), (64, 3008), (64, 3072), (128, 1472), (128, 1536)])
 @pytest.mark.parametrize("T", [100, 3000, 6000, 9000])
 def test_logits_do_not_depend_on_routing(T, d, E):
