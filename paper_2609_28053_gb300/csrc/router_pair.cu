@@ -36,15 +36,6 @@ struct PairArgs {
   int32_t* err;
 };
 
-__device__ __forceinline__ uint32_t cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 // Block 0's barrier at this block's address `bar`.
 __device__ __forceinline__ uint32_t leader_bar(uint32_t bar) {
   uint32_t r;

@@ -37,15 +37,6 @@ struct SplitArgs {
   SplitRoute ro;
 };
 
-__device__ __forceinline__ uint32_t cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 // 16 bytes of block `rank`'s shared memory at this block's address `addr`.
 __device__ __forceinline__ float4 ld_dsmem(uint32_t addr, uint32_t rank) {
   uint32_t ra;

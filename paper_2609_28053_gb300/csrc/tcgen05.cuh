@@ -1,6 +1,7 @@
 // tcgen05.cuh -- what the router projection kernels (router_gemm.cu,
-// router_split.cu) share: mbarriers with bounded waits, TMA tile loads, the
-// tcgen05 descriptors and instructions, and the tensor maps of their operands.
+// router_split.cu, router_pair.cu) share: mbarriers with bounded waits, TMA tile
+// loads, the tcgen05 descriptors and instructions, clusters, and the tensor maps
+// of their operands.
 #pragma once
 
 #include <cuda.h>
@@ -127,6 +128,17 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
         "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr));
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
+// This block's place in its cluster, and the cluster's barrier.
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 constexpr uint32_t kTmemCols = 512;  // the whole TMEM of the SM: one CTA per SM
