@@ -424,13 +424,20 @@ struct HistCut {
 // tiles before the cut by size): T = 100, E = 264 4.45 / 2.6 (2.45) and 4.95 /
 // 3.3 (2.90); T = 1,000 4.75 / 4.2 (4.1) and 5.42 / 4.06 (3.80); T = 60,000, E =
 // 24 5.93 / 4.43 (4.86) in pass 2, T = 20,000, E = 200 7.14 / 6.29 (6.11).
-HistCut cut_hist(int64_t T, int E, int pass, bool lei, bool counted, int blocks) {
+// Shards of a few hundred tokens are flushed one by one, which wide tiles do in
+// fewer rounds: the rank average of 1,000 shards, T = 524,288, in tiles of 4 / 16
+// chunks in pass 2: E = 128 556 / 517, E = 256 986 / 910.
+HistCut cut_hist(int64_t T, int E, int pass, bool lei, bool counted, int shards, int blocks) {
   const int nch = E >> 3;
   const int64_t per_sm = T * nch / blocks;  // chunks of z to count per SM
   int want = T <= 512 ? 1 : per_sm < 1000 && !lei ? 2 : per_sm < 10000 ? 8 : 16;
   if (pass == 2) {
-    const bool one = per_sm < 2000 ? !lei || T <= 512 : per_sm < 10000 && nch <= 5;
-    want = one ? 1 : per_sm < (lei ? 4000 : 5000) ? 2 : per_sm < 64000 ? 4 : per_sm < 200000 ? 8 : 16;
+    want = per_sm < (lei ? 4000 : 5000) ? 2 : per_sm < 64000 ? 4 : per_sm < 200000 ? 8 : 16;
+    if (shards > 1) {
+      if (T / shards < 600) want = 16;
+    } else if (per_sm < 2000 ? !lei || T <= 512 : per_sm < 10000 && nch <= 5) {
+      want = 1;
+    }
     if (counted && want * kMaxHistTiles < nch) want = (nch + kMaxHistTiles - 1) / kMaxHistTiles;
   }
   HistCut h;
@@ -470,7 +477,7 @@ int launch_hist_pass(const HistArgs& a, const LeiStream& ls, CoefRows cr, cudaSt
   DeviceInfo di;
   if (int rc = device_info(&di)) return rc;
   cr.blocks = cr.coef ? coef_blocks(a.T, a.E, cr.a.M, di.sm_count) : 0;
-  const HistCut h = cut_hist(a.T, a.E, PASS, LEI, a.done != nullptr, di.sm_count - cr.blocks);
+  const HistCut h = cut_hist(a.T, a.E, PASS, LEI, a.done != nullptr, a.shard_off ? a.P : 1, di.sm_count - cr.blocks);
   const int smem = (h.copies > 1 ? kBankWords : bin_words(h.chunks)) * 4;
   auto kern = hist_kernel<PASS, LEI, false>;
   int most = bin_words(kMaxTileChunks) * 4;
