@@ -110,8 +110,9 @@ eqb_status eqb_route_topk(const eqb_bf16 *z, const float *b, int64_t T, int32_t 
  * then counts the same staged tile, so z is read from DRAM once instead of
  * twice.  E = 128 or 256 and K + 1 <= 16, else EQB_ERR_UNSUPPORTED.
  * Arguments as in eqb_route_topk; hist_hi is required.  Bit-identical
- * outputs; slower than the two kernels on GB300, where both are bound by
- * instruction issue rather than by DRAM. */
+ * outputs; slower than the two kernels on GB300, although they read z twice:
+ * beside the routing tiles the counting has a third of the coarse pass's warps
+ * and a window of bins that takes more instructions. */
 eqb_status eqb_route_hist_fused(const eqb_bf16 *z, const float *b, int64_t T, int32_t E,
                                 int32_t K, const int64_t *mb_offsets, int32_t M,
                                 int32_t *topk_idx, float *tau, int32_t *loads,
@@ -189,8 +190,9 @@ eqb_status lei_coefficients(const int32_t *loads, const int64_t *mb_offsets,
  * err_flag used, u ignored), pass 2 is eqb_margin_hist_pass2 (hist =
  * hist_lo, u required, err_flag ignored), and for the tokens t in
  * [lei_t0, lei_t1) every grad_s[t, e] += coef[l(t), e] in fp32, l(t) the
- * microbatch of t (Sec. 4, Eq. LEI).  The counting is issue-bound and the
- * injection DRAM-bound, so the two share the GPU better than back to back.
+ * microbatch of t (Sec. 4, Eq. LEI).  The counting takes issue slots beside its
+ * reads and the injection is a DRAM stream, so the two share the GPU better
+ * than back to back.
  * Results are bit-identical to the separate calls; the one-call step runs
  * pass 2 with all of the tokens.
  *   grad_s  device fp32 [T,E], 16-byte aligned, updated in place on [lei_t0, lei_t1)
@@ -269,14 +271,22 @@ eqb_status eqb_layer_step_noalloc(const eqb_bf16 *z, const float *b, int64_t T, 
  * in tensor memory).  The accumulation order is the hardware's, so an entry
  * can differ from the exactly rounded value by one bf16 ulp plus the fp32
  * accumulation error.
+ * The order also depends on how many tokens share the call.  With d >= 1,024
+ * the columns are summed in eight parts up to T = 1,024, in four up to 4,224
+ * and in two up to 8,448 (there from d = 3,072 on at E = 64, from 1,536 on at
+ * other E <= 128), and the parts then added in order; otherwise in one sum
+ * (the limits are those of 152 SMs).  So a token's z, and at near ties its
+ * experts, can differ by a bf16 rounding between calls of different T.  The
+ * same call on the same inputs gives the same bits; no order is further from
+ * the exact sums than the one sum.
  *   x        device bf16 [T, d] row-major, 16-byte aligned     (in)
  *   W_r      device bf16 [E, d] row-major, 16-byte aligned     (in)
  *   z        device bf16 [T, E] row-major, 16-byte aligned     (out)
  *   err_flag device int32 (nullable): EQB_ERR_CUDA if the kernel's pipeline
  *            stalled and it gave up waiting (no result is then valid).
  * Supported: d a positive multiple of 64, E a multiple of 16 with
- * 16 <= E <= 256, 0 <= T <= 2^31 - 2^24.  Uses all tensor memory of each SM
- * it runs on, one block per SM. */
+ * 16 <= E <= 256, 0 <= T <= 2^31 - 2^24.  One block per SM, which takes all of
+ * the SM's tensor memory (half of it where the columns are summed in parts). */
 eqb_status eqb_router_logits(const eqb_bf16 *x, const eqb_bf16 *W_r, int64_t T, int32_t d,
                              int32_t E, eqb_bf16 *z, int32_t *err_flag, void *stream);
 
@@ -355,10 +365,11 @@ eqb_status eqb_fixed_hist_bias(const eqb_bf16 *z, const float *tau, int64_t T, i
 eqb_status eqb_maxvio(const int32_t *loads, const int64_t *mb_offsets, int32_t M, int32_t E,
                       int32_t K, double *maxvio, double *per_mb, void *stream);
 
-/* Router logits, routing and the coarse pass in one kernel: eqb_router_logits
- * followed by eqb_route_topk, with each token routed straight from the
- * tensor-memory accumulator of its row, so z is written once and not read
- * back for routing.  The paper computes the same steps one after the other
+/* Router logits and routing in one kernel, with the coarse pass in the same
+ * kernel or after it: eqb_router_logits followed by eqb_route_topk.  Each token
+ * is routed from the tensor-memory accumulator of its row, or, where the
+ * columns are summed in parts, from the sum of its row, so z is written once
+ * and not read back for routing.  The paper computes the same steps one after the other
  * (Sec. 2, Eq. 1, then top-K of s = z + b, then Algorithm 1 step 1); fusing
  * them is a property of this library.
  *   x, W_r, z   as in eqb_router_logits; z is still written (the fine pass
@@ -368,9 +379,11 @@ eqb_status eqb_maxvio(const int32_t *loads, const int64_t *mb_offsets, int32_t M
  *               loads [M,E] += (nullable; then mb_offsets may be NULL),
  *               hist_hi [E,256] += (nullable): the coarse histogram, counted
  *               in the same kernel from the rows it just stored (read back
- *               from L2) when no block of the kernel routes more than 65,535
- *               tokens (T <= 65,408 x the SM count: 511 tiles of 128 rows per
- *               block), else by the coarse pass over z after it
+ *               from L2) when the columns are summed in one sum and no block of
+ *               the kernel routes more than 65,535 tokens (T <= 65,408 x the SM
+ *               count: 511 tiles of 128 rows per block), else by the coarse
+ *               pass over z after it
+ * The order of the sums is that of eqb_router_logits for the same T, d and E.
  * Results equal those of the calls made one after the other on the same
  * inputs, bit for bit.  err_flag: EQB_ERR_NONFINITE as in eqb_route_topk,
  * EQB_ERR_CUDA as in eqb_router_logits.
@@ -385,10 +398,13 @@ eqb_status eqb_router_route(const eqb_bf16 *x, const eqb_bf16 *W_r, int64_t T, i
 /* The routing-balance step of one layer from the router input: the router
  * projection z = bf16(x W_r^T) (Sec. 2, Eq. 1) followed by everything
  * eqb_layer_step does.  For E in {64, 128} and K <= 8 the projection, the
- * routing and the coarse histogram run as one kernel (eqb_router_route with
+ * routing and the coarse histogram run as one kernel (as eqb_router_route with
  * hist_hi), and the fine pass then streams all of LEI (when M * E <=
- * 65,536); otherwise eqb_router_logits then eqb_route_topk and the schedule
- * of eqb_layer_step.  The other steps are those of
+ * 65,536); otherwise the projection, then eqb_route_topk and the schedule
+ * of eqb_layer_step.  The projection here always takes the columns in one sum,
+ * whatever T is: where eqb_router_logits and eqb_router_route take them in
+ * parts (few tokens), their z can differ from the step's by a bf16 rounding,
+ * and the top-K at near ties with it.  The other steps are those of
  * eqb_layer_step, and so are the arguments from b on; z is an output here
  * (device bf16 [T,E], 16-byte aligned).
  *   x, W_r, d   as in eqb_router_logits.

@@ -20,7 +20,9 @@ namespace {
 constexpr int kGsThreads = 256;
 
 // At most 128 registers where a lane holds several chunks: with one block an
-// SM instead of two, E = 264, T = 241,812 takes 286 us instead of 172.
+// SM instead of two, E = 264, T = 241,812 takes 286 us instead of 172.  ptxas
+// spills 8 to 16 bytes within these bounds (none at 1 lane, 32 lanes of one
+// chunk, or 2 and 4 chunks).
 template <int LPT, int CPL>
 __global__ void __launch_bounds__(kGsThreads, CPL > 1 ? 2 : 4) gshard_kernel(GshardArgs a, int64_t tokens_per_cta) {
   constexpr int TPW = 32 / LPT;  // tokens per warp step

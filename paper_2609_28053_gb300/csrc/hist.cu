@@ -22,10 +22,13 @@
 // chunk i mod nct (8 experts) of token slot i / nct, so a warp reads
 // contiguous pieces of rows whatever the expert count.
 // Two layouts.  Banked (BANK, from 5,000 chunks of z per SM on, passes 1 and
-// 3): 32 columns, a warp's lanes each in their own (chunk, and where the warp
-// holds several tokens of the tile, copy), the bank of every word of a column
-// the same, so no two lanes of an increment meet: word (bin * 4 + pair) * 32 +
-// column.  What bounds these passes otherwise is the banks in which random
+// 3): 32 columns, a lane's by its chunk and, where the warp holds several tokens
+// of the tile, copy, the bank of every word of a column the same: word (bin * 4
+// + pair) * 32 + column.  Where the tile's chunks divide 32 every lane of a warp
+// has a column of its own, so no two lanes of an increment meet.  Otherwise
+// (tiles of 5, 7, 11 or 13 chunks) there are fewer columns than lanes and up to
+// 32 - nct * copies lanes share one, the same word at times: the increments have
+// to be atomic.  What bounds these passes otherwise is the banks in which random
 // bins meet: 2.8 to 3.7 clocks an increment of a warp, against 1.4 or less.
 // T = 2,097,152, E = 256 202 -> 160 us (the copy rate), T = 524,288, E = 128
 // 34 -> 26, T = 147,456, E = 256 21 -> 16.6; pass 3 260 -> 192 and 49 -> 40 (a
@@ -58,7 +61,8 @@ namespace {
 // 16-byte loads in flight per thread (64 registers at 1024 threads).  Pass 1
 // (before its banked bins) / pass 2 alone at T = 2,097,152, E = 256: 187 / 171 us with six, 185 / 185
 // with seven, 194 / 184 with eight, 221 / 181 with four.  Beside the injection
-// eight (the step at T = 1,048,576, E = 512 1229 us, 1241 with six).
+// eight (the step at T = 1,048,576, E = 512 1229 us, 1241 with six); ptxas then
+// spills 32 bytes in the fine pass, which runs at 99% of the copy rate with them.
 template <bool LEI>
 constexpr int kUnroll = LEI ? 8 : 6;
 constexpr int64_t kFlushTokens = 65535;

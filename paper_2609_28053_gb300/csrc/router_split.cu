@@ -15,8 +15,8 @@
 // that its tile starts in in shared memory and adds them as whole lines: T =
 // 4,224, d = 1,024, E = 64, M = 4 with the coarse pass 14.0 us, 20.5 with each
 // token's eight scattered adds to global memory (15.6 unsplit).  Each partial sum is shorter than the whole:
-// 300 of 1e6 logits round to another bf16 value than the 64-bit sums do at
-// d = 4,096, where the one long sum has 2,335.
+// 329, 672 and 1,226 of 1e6 logits round to another bf16 value than the 64-bit
+// sums do in eight, four and two parts (d = 4,096, E = 128), 2,295 in one sum.
 //
 // Every mbarrier wait is bounded and every thread reaches both cluster
 // barriers, whether or not a wait ran out; after one that did, the tile loads
