@@ -422,19 +422,21 @@ struct HistCut {
 // chunks: T = 30,873, E = 256 35 / 37 / 42 us, T = 65,536, E = 64 31 / 35 /
 // 35, T = 524,288, E = 128 185 / 187 / 190, E = 256 321 / 321 / 325, T =
 // 1,048,576, E = 512 1220 / 1219 / 1211.
-// The smallest batches take one or two chunks a tile and, unless warps of the
-// block stream LEI, 512 threads: little else than the fixed cost is left.  Pass
-// 1 / pass 2 alone, us, 8 and 4 chunks with 1,024 threads / now (33 one-chunk
-// tiles before the cut by size): T = 100, E = 264 4.45 / 2.6 (2.45) and 4.95 /
-// 3.3 (2.90); T = 1,000 4.75 / 4.2 (4.1) and 5.42 / 4.06 (3.80); T = 60,000, E =
-// 24 5.93 / 4.43 (4.86) in pass 2, T = 20,000, E = 200 7.14 / 6.29 (6.11).
+// The smallest batches take one or two chunks a tile and 512 threads (half of
+// them stream LEI as half of 1,024 do): little else than the fixed cost is left.
+// Pass 1 / pass 2 alone, us, 8 and 4 chunks with 1,024 threads / now (33
+// one-chunk tiles before the cut by size): T = 100, E = 264 4.45 / 2.6 (2.45)
+// and 4.95 / 3.3 (2.90); T = 1,000 4.75 / 4.2 (4.1) and 5.42 / 4.06 (3.80); T =
+// 60,000, E = 24 5.93 / 4.43 (4.86) in pass 2, T = 20,000, E = 200 7.14 / 6.29
+// (6.11).  Pass 2 with LEI: T = 1,000, E = 8 6.3 / 5.5 (5.7), E = 256 5.9 / 5.1.
+// The step: T = 4,096, E = 8 16.8 / 15.3, E = 128 22.8 / 21.2.
 // Shards of a few hundred tokens are flushed one by one, which wide tiles do in
 // fewer rounds: the rank average of 1,000 shards, T = 524,288, in tiles of 4 / 16
 // chunks in pass 2: E = 128 556 / 517, E = 256 986 / 910.
 HistCut cut_hist(int64_t T, int E, int pass, bool lei, bool counted, int shards, int blocks) {
   const int nch = E >> 3;
   const int64_t per_sm = T * nch / blocks;  // chunks of z to count per SM
-  int want = T <= 512 ? 1 : per_sm < 1000 && !lei ? 2 : per_sm < 10000 ? 8 : 16;
+  int want = T <= 512 ? 1 : per_sm <= (lei ? 512 : 1000) ? 2 : per_sm < 10000 ? 8 : 16;
   if (pass == 2) {
     want = per_sm < (lei ? 4000 : 5000) ? 2 : per_sm < 64000 ? 4 : per_sm < 200000 ? 8 : 16;
     if (shards > 1) {
@@ -448,7 +450,7 @@ HistCut cut_hist(int64_t T, int E, int pass, bool lei, bool counted, int shards,
   h.tiles = (nch + want - 1) / want;
   h.chunks = (nch + h.tiles - 1) / h.tiles;
   h.tiles = (nch + h.chunks - 1) / h.chunks;
-  h.threads = per_sm <= 512 && h.chunks <= 2 && !lei ? 512 : 1024;
+  h.threads = per_sm <= 512 && h.chunks <= 2 ? 512 : 1024;
   h.copies = pass != 2 && per_sm >= 5000 ? 32 / h.chunks : 1;
   int64_t ranges = blocks / h.tiles;
   const int64_t most = (T * h.chunks + h.threads - 1) / h.threads;  // a chunk for every thread
@@ -477,11 +479,12 @@ int coef_blocks(int64_t T, int E, int M, int sm_count) {
 }
 
 template <int PASS, bool LEI>
-int launch_hist_pass(const HistArgs& a, const LeiStream& ls, CoefRows cr, cudaStream_t s) {
+int launch_hist_pass(const HistArgs& a, LeiStream ls, CoefRows cr, cudaStream_t s) {
   DeviceInfo di;
   if (int rc = device_info(&di)) return rc;
   cr.blocks = cr.coef ? coef_blocks(a.T, a.E, cr.a.M, di.sm_count) : 0;
   const HistCut h = cut_hist(a.T, a.E, PASS, LEI, a.done != nullptr, a.shard_off ? a.P : 1, di.sm_count - cr.blocks);
+  if (LEI) ls.warps = ls.warps * h.threads / 1024;
   const int smem = (h.copies > 1 ? kBankWords : bin_words(h.chunks)) * 4;
   auto kern = hist_kernel<PASS, LEI, false>;
   int most = bin_words(kMaxTileChunks) * 4;
@@ -513,7 +516,7 @@ int launch_hist_coef(const HistArgs& a, const LeiArgs& la, float* coef, cudaStre
 
 int launch_hist_lei(const HistArgs& a, int pass, const LeiStream& lei, cudaStream_t s) {
   LeiStream ls = lei;
-  // of 32: the passes are DRAM-bound, and the more warps stream from the start
+  // of 32 (half of them of 16): the passes are DRAM-bound, and the more warps stream from the start
   // the sooner they are, until counting is what takes longest.  A pass that
   // carries every token, 14 / 16 / 18 / 20: T = 65,536, E = 64 30.9 / 31.1 /
   // 33.9 / 32.7 us a step, T = 200,003, E = 96 72.2 / 71.5 / 71.9 / 71.7, T =
