@@ -14,9 +14,11 @@
 // (warp_route, route_warp.cuh).  A block counts the loads of the microbatch
 // that its tile starts in in shared memory and adds them as whole lines: T =
 // 4,224, d = 1,024, E = 64, M = 4 with the coarse pass 14.0 us, 20.5 with each
-// token's eight scattered adds to global memory (15.6 unsplit).  Each partial sum is shorter than the whole:
-// 329, 672 and 1,226 of 1e6 logits round to another bf16 value than the 64-bit
-// sums do in eight, four and two parts (d = 4,096, E = 128), 2,295 in one sum.
+// token's eight scattered adds to global memory (15.6 unsplit).
+//
+// Each partial sum is shorter than the whole: 329, 672 and 1,226 of 1e6 logits
+// round to another bf16 value than the 64-bit sums do in eight, four and two
+// parts (d = 4,096, E = 128), 2,295 in one sum.
 //
 // Every mbarrier wait is bounded and every thread reaches both cluster
 // barriers, whether or not a wait ran out; after one that did, the tile loads
@@ -265,8 +267,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 // warp each take longer than 128 from the accumulator beside the next tile's
 // MMAs, so two blocks pay from more columns on (T = 4,225, n = 1 / 2): E = 64 9.8
 // / 12.6 at d = 1,024, 13.9 / 14.8 at 2,048, 18.0 / 16.9 at 3,072; E = 128 11.8 /
-// 12.4 at 1,024, 13.9 / 13.4 at 1,536.  The rule does not ask whether
-// there is routing: logits must not depend on it.
+// 12.4 at 1,024, 13.9 / 13.4 at 1,536.  The rule does not ask whether there is
+// routing: logits must not depend on it.
 int router_splits(int64_t T, int d, int E, int sm_count) {
   const int64_t tiles = (T + kBM - 1) / kBM;
   if (d < 1024) return 1;
